@@ -125,7 +125,8 @@ typedef struct {
  * microseconds the launches cost more than the work.  Without this flag,
  * PR_OPT_DEVICE_LOOP or a host-loop flag, the device loop runs in one kernel
  * when the graphs of the update hold fewer than PR_ONE_KERNEL_SLOTS in-CSR
- * slots in all; PR_OPT_DEVICE_LOOP alone asks for the CUDA graph.  At most one
+ * slots in all (one graph alone: fewer than three times as many, unless one
+ * in-row holds most of them); PR_OPT_DEVICE_LOOP alone asks for the CUDA graph.  At most one
  * of PR_OPT_HOST_LOOP, PR_OPT_DEVICE_LOOP and PR_OPT_ONE_KERNEL may be set.
  * The result is the same bit for bit.  A barrier wait gives up after about a
  * second (a block that never arrives); the update then returns PR_ETIMEOUT

@@ -1131,7 +1131,8 @@ pr_status pr_update(pr_graph* h, pr_method method, double alpha, double tau, con
       flags & (PR_OPT_HOST_LOOP | PR_OPT_TIME_SWEEPS | PR_OPT_FORCE_PULL | PR_OPT_FORCE_PUSH | PR_OPT_ASYNC);
   const bool loopable = method != PR_DYNAMIC_TRAVERSAL;
   if (loopable &&
-      ((flags & (PR_OPT_DEVICE_LOOP | PR_OPT_ONE_KERNEL)) || (!host_flags && g->in.cap < PR_DEVICE_LOOP_SLOTS))) {
+      ((flags & (PR_OPT_DEVICE_LOOP | PR_OPT_ONE_KERNEL)) ||
+       (!host_flags && g->in.cap < PR_DEVICE_LOOP_SLOTS))) {
     // the iteration loop on the device: a group of this one graph, on its stream
     if (!h->solo) {
       pr_graph* one[1] = {h};

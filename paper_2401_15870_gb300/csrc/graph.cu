@@ -14,6 +14,7 @@
 #include "graph.cuh"
 #include "prim.cuh"
 #include "sweep.cuh"
+#include "loop.cuh"
 
 namespace dfpr {
 
@@ -211,11 +212,19 @@ int refresh_full_tiles(Graph* g) {
   TRY(cudaMemsetAsync(g->rowbase, 0, sizeof(int32_t) * padded, g->stream));
   {
     int32_t* tmp;
-    TRY(dev_malloc(&tmp, sizeof(int32_t) * scan_tmp_elems(words)));
+    int32_t shares[2] = {0, 0};
+    TRY(dev_malloc(&tmp, sizeof(int32_t) * (scan_tmp_elems(words) + 2)));
+    int32_t* sh = tmp + scan_tmp_elems(words);
     cudaError_t e = launch_row_start_index(g->in.off, g->n, quads, g->rowbits, g->rowbase, tmp, g->stream);
-    cudaStreamSynchronize(g->stream);
+    if (e == cudaSuccess) e = launch_loop_shares(g->in.off, g->n, quads, g->rowbits, g->rowbase, sh, g->stream);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(shares, sh, sizeof(shares), cudaMemcpyDeviceToHost, g->stream);
+    cudaError_t es = cudaStreamSynchronize(g->stream);
     cudaFree(tmp);
     TRY(e);
+    TRY(es);
+    g->loop_rows = shares[0];
+    g->loop_quads = shares[1];
   }
   if (g->full_tfirst) {
     for (auto& p : g->allocs)

@@ -82,6 +82,7 @@ struct Graph {
   int64_t full_ntiles = 0;
   uint32_t* rowbits = nullptr;              // full sweeps: in-CSR quads where a row starts
   int32_t* rowbase = nullptr;               // rows starting before each 32-quad word
+  int32_t loop_rows = 0, loop_quads = 0;    // largest rows / quads of a block's share in the one-barrier loop (loop.cu)
   uint32_t* anyb = nullptr;                 // full pull sweeps: an in-neighbour expanded (n bits)
   int32_t* done = nullptr;                  // one-launch full sweeps: gather units counted per 128-vertex chunk
 

@@ -31,6 +31,7 @@
 #include "prim.cuh"
 #include "pull_step.cuh"
 #include "group.cuh"
+#include "loop.cuh"
 
 using namespace dfpr;
 
@@ -562,6 +563,12 @@ struct pr_group {
   cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
   // resident blocks per SM of the one-kernel loop [form][relative measure], 0 until asked
   int loop_bps[2][2] = {{0, 0}, {0, 0}};
+  // an update of one graph in the one-barrier loop (loop.cu): its barrier and
+  // outcome on the device, the outcome on the host, and whether the update in
+  // flight is one
+  LoopState* d_loop = nullptr;
+  LoopOut* h_loop = nullptr;
+  bool loop_clean = false, one_barrier = false;
   // the update in flight: its members (group indices) and method
   std::vector<int32_t> members;
   bool in_flight = false;
@@ -574,9 +581,10 @@ static void group_free(pr_group* q) {
   if (!q) return;
   if (q->stream) cudaStreamSynchronize(q->stream);
   for (int k = 0; k < 2; k++) drop_exec(q, k);
-  for (void* p : {(void*)q->d_run, (void*)q->d_desc, (void*)q->d_state, (void*)q->d_pre, (void*)q->tab_sc})
+  for (void* p : {(void*)q->d_run, (void*)q->d_desc, (void*)q->d_state, (void*)q->d_pre, (void*)q->tab_sc,
+                  (void*)q->d_loop})
     if (p) cudaFree(p);
-  for (void* p : {(void*)q->h_run, (void*)q->h_desc, (void*)q->h_state, (void*)q->h_pre})
+  for (void* p : {(void*)q->h_run, (void*)q->h_desc, (void*)q->h_state, (void*)q->h_pre, (void*)q->h_loop})
     if (p) cudaFreeHost(p);
   for (cudaEvent_t e : q->ev)
     if (e) cudaEventDestroy(e);
@@ -716,6 +724,8 @@ pr_status pr_group_create(int32_t count, pr_graph* const* graphs, void* stream, 
             dev_malloc((void**)&q->d_state, sizeof(GState) * count) == cudaSuccess &&
             dev_malloc((void**)&q->d_pre, sizeof(int64_t) * pre_elems) == cudaSuccess &&
             dev_malloc((void**)&q->tab_sc, sizeof(double) * TAB) == cudaSuccess &&
+            dev_malloc((void**)&q->d_loop, loop_state_bytes()) == cudaSuccess &&
+            cudaMallocHost((void**)&q->h_loop, sizeof(LoopOut)) == cudaSuccess &&
             cudaMallocHost((void**)&q->h_run, sizeof(GRun)) == cudaSuccess &&
             cudaMallocHost((void**)&q->h_desc, sizeof(GDesc) * count) == cudaSuccess &&
             cudaMallocHost((void**)&q->h_state, sizeof(GState) * count) == cudaSuccess &&
@@ -739,14 +749,27 @@ static const void* loop_fn(int k, bool rel) {
   return k ? (const void*)k_g_loop<true, false> : (const void*)k_g_loop<false, false>;
 }
 
-// the whole update as one cooperative launch of every resident block.  Two
-// such grids launched from different streams at once could each hold part of
-// the SMs while waiting at a barrier for blocks that the other keeps out, so
-// every launch of the process is ordered after the previous one on the
-// device (an event per device; the host does not wait)
-static cudaError_t launch_one_kernel(pr_group* q, int k, bool rel) {
+// Cooperative grids wait for their own blocks: two of them launched from
+// different streams at once could each hold part of the SMs while waiting at a
+// barrier for blocks that the other keeps out, so every such launch of the
+// process is ordered after the previous one on the device (an event per
+// device; the host does not wait)
+template <class Launch>
+static cudaError_t one_after_another(pr_group* q, Launch launch) {
   static std::mutex mu;
   static std::map<int, cudaEvent_t> last;
+  std::lock_guard<std::mutex> lock(mu);
+  cudaEvent_t& ev = last[q->dev];
+  cudaError_t e = cudaSuccess;
+  if (!ev) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+  else e = cudaStreamWaitEvent(q->stream, ev, 0);
+  if (e == cudaSuccess) e = launch();
+  if (e != cudaSuccess) return e;
+  return cudaEventRecord(ev, q->stream);
+}
+
+// the whole update as one cooperative launch of every resident block
+static cudaError_t launch_one_kernel(pr_group* q, int k, bool rel) {
   const void* fn = loop_fn(k, rel);
   const size_t smem = 4 * prefix_bytes(q) + sizeof(uint32_t) * (size_t)q->G;
   int& bps = q->loop_bps[k][rel ? 1 : 0];
@@ -757,16 +780,56 @@ static cudaError_t launch_one_kernel(pr_group* q, int k, bool rel) {
     bps = std::min(bps, LOOP_BPS);
   }
   void* args[] = {&q->d_run, &q->d_desc, &q->d_state};
-  std::lock_guard<std::mutex> lock(mu);
-  cudaEvent_t& ev = last[q->dev];
-  cudaError_t e = cudaSuccess;
-  if (!ev) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
-  else e = cudaStreamWaitEvent(q->stream, ev, 0);
+  return one_after_another(q, [&] {
+    note_launch();
+    return cudaLaunchCooperativeKernel(fn, dim3(num_sms() * bps), dim3(GR_THREADS), args, smem, q->stream);
+  });
+}
+
+// the update of one graph in the one-barrier loop
+static cudaError_t launch_one_barrier(pr_group* q, Graph* g, pr_method method, double alpha, double tau,
+                                      const pr_options& o, int metric) {
+  cudaStream_t s = q->stream;
+  if (!q->loop_clean) {
+    cudaError_t e = loop_reset(q->d_loop, s);
+    if (e != cudaSuccess) return e;
+    q->loop_clean = true;
+  }
+  LoopParams p;
+  memset(&p, 0, sizeof(p));
+  p.n = g->n;
+  p.method = (int32_t)method;
+  p.max_iter = o.max_iter;
+  p.metric = metric;
+  p.id_bits = g->id_bits;
+  p.icol = g->in.col;
+  p.ioff = g->in.off;
+  p.rowbits = g->rowbits;
+  p.rowbase = g->rowbase;
+  p.nquads = g->in.cap >> 2;
+  p.odeg = g->out.deg;
+  p.ideg = g->in.deg;
+  p.R = g->R;
+  p.C[0] = g->C[g->ccur];
+  p.C[1] = g->C[g->ccur ^ 1];
+  p.X[0] = (uint8_t*)g->rnew;   // the push sweeps' rank buffer (8 n bytes), free in this loop
+  p.X[1] = p.X[0] + g->n;
+  p.S = g->bits[0];
+  p.dmin = g->dmin;
+  p.dplus = g->dplus;
+  p.n_dmin = g->n_dmin;
+  p.n_dplus = g->n_dplus;
+  p.alpha = alpha;
+  p.C0 = (1.0 - alpha) / (double)g->n;
+  p.tau = tau;
+  p.tau_f = o.tau_f;
+  p.tau_p = o.tau_p;
+  p.tab_sc = q->tab_sc;
+  p.tab_ab = g->tab_ab;
+  p.st = q->d_loop;
+  cudaError_t e = one_after_another(q, [&] { return launch_loop(g, p, s); });
   if (e != cudaSuccess) return e;
-  note_launch();
-  e = cudaLaunchCooperativeKernel(fn, dim3(num_sms() * bps), dim3(GR_THREADS), args, smem, q->stream);
-  if (e != cudaSuccess) return e;
-  return cudaEventRecord(ev, q->stream);
+  return cudaMemcpyAsync(q->h_loop, &q->d_loop->out, sizeof(LoopOut), cudaMemcpyDeviceToHost, s);
 }
 
 // the same kernels launched one by one, the loop condition read back after
@@ -841,7 +904,12 @@ pr_status group_launch(pr_group* q, pr_method method, double alpha, double tau, 
   // the loop in one kernel when asked, or by default when the sweeps are short
   int64_t slots = 0;
   for (int i = 0; i < G; i++) slots += q->graphs[mem[i]]->g.in.cap;
-  const bool one = (o.flags & PR_OPT_ONE_KERNEL) || (loops_asked == 0 && slots < PR_ONE_KERNEL_SLOTS);
+  // (one graph whose rows can be shared out to the blocks: the loop with one
+  // barrier per iteration, whatever its size)
+  q->one_barrier = G == 1 && loop_fits(&q->graphs[mem[0]]->g) &&
+                   ((o.flags & PR_OPT_ONE_KERNEL) || (loops_asked == 0 && loop_default(&q->graphs[mem[0]]->g)));
+  const bool one =
+      !q->one_barrier && ((o.flags & PR_OPT_ONE_KERNEL) || (loops_asked == 0 && slots < PR_ONE_KERNEL_SLOTS));
   const int64_t gq = one ? 32 * LOOP_QPT : 32 * GR_QPT[q->qi] * GR_STEPS[q->qi];   // quads per gather unit
   const int64_t fu = one ? LOOP_FU : GR_FU[q->fi];                                 // chunks per epilogue unit
   int64_t* wpre = q->h_pre;
@@ -923,6 +991,16 @@ pr_status group_launch(pr_group* q, pr_method method, double alpha, double tau, 
       g->tab_alpha = alpha;
     }
   }
+  if (q->one_barrier) {
+    if (launch_one_barrier(q, &q->graphs[mem[0]]->g, method, alpha, tau, o, r.metric) != cudaSuccess) {
+      cudaGetLastError();
+      return PR_ECUDA;
+    }
+    if (cudaEventRecord(q->ev[1], s) != cudaSuccess) return PR_ECUDA;
+    q->in_flight = true;
+    q->cur_method = method;
+    return PR_OK;
+  }
   if (cudaMemcpyAsync(q->d_pre, q->h_pre, sizeof(int64_t) * 4 * (size_t)(G + 1), cudaMemcpyHostToDevice, s) !=
           cudaSuccess ||
       cudaMemcpyAsync(q->d_desc, q->h_desc, sizeof(GDesc) * G, cudaMemcpyHostToDevice, s) != cudaSuccess ||
@@ -964,6 +1042,24 @@ pr_status group_complete(pr_group* q, pr_stats* stats) {
   q->in_flight = false;
   if (cudaEventSynchronize(q->ev[1]) != cudaSuccess) return PR_ECUDA;
   const pr_method method = q->cur_method;
+  if (q->one_barrier) {
+    // the outcome in the form the other loops leave it
+    const LoopOut& lo = *q->h_loop;
+    GState& st = q->h_state[0];
+    memset(&st, 0, sizeof(st));
+    st.iter = lo.iter;
+    st.converged = lo.converged;
+    st.cur = lo.cur;
+    st.dR_last = lo.dR_last;
+    for (int b = 0; b < loop_blocks(); b++) {
+      st.edges += lo.part[b][0];
+      st.verts += lo.part[b][1];
+      st.ever += lo.part[b][2];
+    }
+    q->h_run->use_graph = 0;
+    q->h_run->err = lo.err;
+    if (lo.err) q->loop_clean = false;
+  }
   if (q->h_run->err) {
     // a grid barrier of the one-kernel loop gave up: the ranks are partial
     for (int32_t gi : q->members) q->graphs[gi]->g.has_ranks = false;

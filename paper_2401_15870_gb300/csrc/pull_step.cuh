@@ -81,6 +81,19 @@ __device__ __forceinline__ long long ld_weak_hint(const long long* p, uint64_t p
   asm volatile("ld.global.L2::cache_hint.b64 %0, [%1], %2;" : "=l"(v) : "l"(p), "l"(pol) : "memory");
   return v;
 }
+// (the two loads of ld_contrib as ordinary loads)
+__device__ __forceinline__ long long ld_weak_contrib(const long long* p, const long long* hub_end, uint64_t pol) {
+  long long v;
+  asm volatile(
+      "{\n\t.reg .pred h;\n\t"
+      "setp.lt.u64 h, %1, %2;\n\t"
+      "@h ld.global.L2::cache_hint.b64 %0, [%1], %3;\n\t"
+      "@!h ld.global.L1::no_allocate.L2::cache_hint.b64 %0, [%1], %3;\n\t}"
+      : "=l"(v)
+      : "l"(p), "l"(hub_end), "l"(pol)
+      : "memory");
+  return v;
+}
 __device__ __forceinline__ uint32_t ld_weak(const uint32_t* p) {
   uint32_t v;
   asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
