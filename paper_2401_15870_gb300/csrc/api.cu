@@ -239,6 +239,7 @@ static void destroy_handle(pr_graph* h) {
   if (g->dplus) cudaFree(g->dplus);
   if (g->ctl_h) cudaFreeHost(g->ctl_h);
   if (g->small_h) cudaFreeHost(g->small_h);
+  if (g->stage_h) cudaFreeHost(g->stage_h);
   for (int i = 0; i < 6; i++)
     if (h->ev[i]) cudaEventDestroy(h->ev[i]);
   for (cudaEvent_t e : h->saux.ev)
@@ -876,18 +877,8 @@ static pr_status apply_common(pr_graph* h, const int32_t* ds, const int32_t* dd,
     for (int64_t i = 0; i < ni; i++)
       if (is[i] < 0 || is[i] >= n || id[i] < 0 || id[i] >= n)
         return (pr_status)set_error(g, ERANGE_, "pr_apply_batch: vertex id out of range");
-    int64_t nk = nd + ni;
-    void* stage;
-    TRY(scratch_get(g, 0, sizeof(int32_t) * (size_t)(2 * nk + 4) + 1024, &stage));
-    int32_t* b = (int32_t*)stage;
-    if (nd) {
-      TRY(cudaMemcpyAsync(b, ds, sizeof(int32_t) * nd, cudaMemcpyHostToDevice, s));
-      TRY(cudaMemcpyAsync(b + nd, dd, sizeof(int32_t) * nd, cudaMemcpyHostToDevice, s));
-    }
-    if (ni) {
-      TRY(cudaMemcpyAsync(b + 2 * nd, is, sizeof(int32_t) * ni, cudaMemcpyHostToDevice, s));
-      TRY(cudaMemcpyAsync(b + 2 * nd + ni, id, sizeof(int32_t) * ni, cudaMemcpyHostToDevice, s));
-    }
+    int32_t* b;
+    RC(stage_host_batch(g, ds, dd, nd, is, id, ni, &b));
     rc = apply_batch_device(g, b, b + nd, nd, b + 2 * nd, b + 2 * nd + ni, ni, true);
   }
   if (rc != OK) return (pr_status)rc;
@@ -1016,19 +1007,11 @@ static pr_status apply_many(int32_t count, pr_graph* const* graphs, const int32_
       g->stream = aux;
     }
     queued[i] = 1;
-    if (!device && nd + ni > 0) {   // staged in the graph's scratch (slot 0), as pr_apply_batch does
-      void* stage;
-      cudaError_t e = scratch_get(g, 0, sizeof(int32_t) * (size_t)(2 * (nd + ni) + 4) + 1024, &stage);
-      int32_t* b = (int32_t*)stage;
-      if (e == cudaSuccess && nd) e = cudaMemcpyAsync(b, ds, sizeof(int32_t) * nd, cudaMemcpyHostToDevice, g->stream);
-      if (e == cudaSuccess && nd)
-        e = cudaMemcpyAsync(b + nd, dd, sizeof(int32_t) * nd, cudaMemcpyHostToDevice, g->stream);
-      if (e == cudaSuccess && ni)
-        e = cudaMemcpyAsync(b + 2 * nd, is, sizeof(int32_t) * ni, cudaMemcpyHostToDevice, g->stream);
-      if (e == cudaSuccess && ni)
-        e = cudaMemcpyAsync(b + 2 * nd + ni, id, sizeof(int32_t) * ni, cudaMemcpyHostToDevice, g->stream);
-      if (e != cudaSuccess) {
-        fail((pr_status)cuda_fail(g, e, "pr_apply_batches"));
+    if (!device && nd + ni > 0) {
+      int32_t* b;
+      const int rs = stage_host_batch(g, ds, dd, nd, is, id, ni, &b);
+      if (rs != OK) {
+        fail((pr_status)rs);
         continue;
       }
       ds = b;

@@ -15,6 +15,9 @@
 // new degree exceeds its capacity triggers a repack of that direction (a full
 // rebuild with fresh slack).
 #include <algorithm>
+#include <climits>
+#include <cstring>
+#include <new>
 #include "batch.cuh"
 #include "frontier.cuh"
 #include "prim.cuh"
@@ -174,8 +177,7 @@ __device__ __forceinline__ int64_t chunk_row(const int64_t* pre, int64_t nr, int
 __global__ void k_row_copy(const uint64_t* __restrict__ rows, const int64_t* __restrict__ nrp,
                            const int64_t* __restrict__ sofs, const int64_t* __restrict__ cpre,
                            const int64_t* __restrict__ off, const int32_t* __restrict__ deg,
-                           const int32_t* __restrict__ col, int32_t* __restrict__ scratch, const int32_t* skip) {
-  if (skip && *skip) return;
+                           const int32_t* __restrict__ col, int32_t* __restrict__ scratch) {
   const int64_t nr = *nrp;
   const int lane = threadIdx.x & 31;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -199,8 +201,7 @@ __global__ void k_row_survivors(const uint64_t* __restrict__ rows, const int64_t
                                 const int64_t* __restrict__ wpre, const uint64_t* __restrict__ dl,
                                 const uint64_t* __restrict__ il, int bits, const int64_t* __restrict__ off,
                                 const int32_t* __restrict__ deg, int32_t* __restrict__ col,
-                                const int32_t* __restrict__ scratch, int32_t sent, const int32_t* skip) {
-  if (skip && *skip) return;
+                                const int32_t* __restrict__ scratch, int32_t sent) {
   const int64_t nr = *nrp;
   const int lane = threadIdx.x & 31;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -238,8 +239,7 @@ __global__ void k_row_insertions(const uint64_t* __restrict__ rows, const int64_
                                  const uint64_t* __restrict__ dl, const uint64_t* __restrict__ il,
                                  const int64_t* __restrict__ nip, int bits, const int64_t* __restrict__ off,
                                  const int32_t* __restrict__ deg, int32_t* __restrict__ col,
-                                 const int32_t* __restrict__ scratch, const int32_t* skip) {
-  if (skip && *skip) return;
+                                 const int32_t* __restrict__ scratch) {
   const int64_t nr = *nrp, ni = *nip;
   const uint64_t mask = (1ull << bits) - 1;
   GRID_STRIDE(k, ni) {
@@ -268,8 +268,7 @@ __global__ void k_row_insertions(const uint64_t* __restrict__ rows, const int64_
 }
 
 __global__ void k_row_degrees(const uint64_t* __restrict__ rows, const int64_t* __restrict__ nrp,
-                              const int64_t* __restrict__ plan, int32_t* __restrict__ deg, const int32_t* skip) {
-  if (skip && *skip) return;
+                              const int64_t* __restrict__ plan, int32_t* __restrict__ deg) {
   const int64_t nr = *nrp;
   GRID_STRIDE(j, nr) {
     const uint64_t r = rows[j];
@@ -602,14 +601,14 @@ static int edit_direction(Graph* g, Csr* c, const uint64_t* dl, int64_t nd, cons
     TRY(scratch_get(g, 5, sizeof(int32_t) * (size_t)(stot + 1), &sp));
     int32_t* S = (int32_t*)sp;
     const int wgrid = num_sms() * 16;
-    note_launch(); k_row_copy<<<wgrid, 256, 0, s>>>(rows, cnt, sofs, cpre, c->off, c->deg, c->col, S, nullptr);
+    note_launch(); k_row_copy<<<wgrid, 256, 0, s>>>(rows, cnt, sofs, cpre, c->off, c->deg, c->col, S);
     note_launch(); k_row_survivors<<<wgrid, 256, 0, s>>>(rows, cnt, plan, sofs, wpre, dl, il, bits, c->off, c->deg, c->col,
-                                                         S, g->n, nullptr);
+                                                         S, g->n);
     if (ni) {
       note_launch(); k_row_insertions<<<grid_for(ni, 256), 256, 0, s>>>(rows, cnt, plan, sofs, dl, il, ni_dev, bits,
-                                                                        c->off, c->deg, c->col, S, nullptr);
+                                                                        c->off, c->deg, c->col, S);
     }
-    note_launch(); k_row_degrees<<<grid_for(nr, 256), 256, 0, s>>>(rows, cnt, plan, c->deg, nullptr);
+    note_launch(); k_row_degrees<<<grid_for(nr, 256), 256, 0, s>>>(rows, cnt, plan, c->deg);
     TRY(cudaGetLastError());
     return OK;
   }
@@ -621,297 +620,504 @@ static int edit_direction(Graph* g, Csr* c, const uint64_t* dl, int64_t nd, cons
 
 // ------------------------------------------------------------------ small batches
 //
-// A batch of at most SMALL_MAX edges is ingested by one thread block with the
-// keys in shared memory: validation, packed keys, sort (bitonic), effective
-// flags, compaction, the same lists keyed (dst, src), and for each direction
-// the touched rows with their edit plans and prefix sums.  The row rewrite
-// kernels above then read every count from the device, so the whole batch
-// costs about ten launches and one host synchronisation (the status read at
-// the end) instead of ~170 launches and six synchronisations.  A direction
-// whose rows overflow their capacity, or whose staging buffer is too small,
-// is skipped by the device and finished by the host after the status read.
-constexpr int SMALL_MAX = 4096;                 // edges of a batch (deletions + insertions)
+// A batch of at most SMALL_MAX edges costs four launches and one host
+// synchronisation (the status read at the end).  It is bound by latency, not
+// by bytes: a chain of launches, of dependent loads and of block barriers.
+//   k_small_keys    one thread per edge over the whole chip: ids checked,
+//                   packed key, and whether the edge is in E_{t-1} (a search of
+//                   its out-row, eight ways per step);
+//   k_small_ingest  one block per direction, side by side: the keys sorted as
+//                   (src, dst) and as (dst, src) in registers (bitonic: strides
+//                   within a thread and a warp need no barrier), effective
+//                   flags, compaction, touched rows with their edit plans;
+//   k_small_copy    the old elements of touched rows longer than a chunk into
+//                   scratch (a row is edited in place, by many warps);
+//   k_small_edit    one warp per touched row, staged in shared memory, or per
+//                   chunk of a longer row; both directions at once, with the
+//                   new degrees and the contributions of the sources.
+// Before, one block ran both directions in turn with the sort in shared memory
+// (53 us at 168 edges, 143 at 1300, 312 at 4000) and five kernels per direction
+// followed: 166 us of device time per batch at 2^14 vertices and 262 edges.
+// A direction whose rows overflow their capacity, or whose scratch is too
+// small, is left alone by the device and finished by the host.
+constexpr int SMALL_MAX = 16384;                // edges of a batch (deletions + insertions)
 constexpr int SMALL_THREADS = 1024;
-constexpr int SMALL_SORT = 2 * SMALL_MAX;       // sort slots (each side padded to a power of two)
+constexpr uint64_t BAD = ~1ull;                  // key of an edge with an id out of range (no packed key: ids are below 2^31)
 
-struct SmallStatus {
-  int64_t n_del, n_ins;   // effective deletions / insertions
-  int64_t nr[2];          // touched rows, out (0) and in (1)
-  int64_t stot[2];        // staging elements (old degrees of the touched rows)
-  int32_t skip[2];        // the device left this direction's rows unchanged
-  int32_t bad, ovf[2], need[2], pad;
+}  // namespace dfpr
+
+struct dfpr::SmallStatus {
+  int32_t n_del, n_ins;   // effective deletions / insertions
+  int32_t bad;
+  // per direction (out 0, in 1): touched rows, those longer than a chunk and
+  // their chunks; the device left the direction unchanged (skip), because rows
+  // overflow (ovf) or the scratch is too small (need)
+  int32_t nr[2], nlong[2], chunks[2], skip[2], ovf[2], need[2];
 };
 
-struct SmallBufs {
-  uint64_t edl[SMALL_MAX], eil[SMALL_MAX];   // Delta-, Delta+ sorted by (src, dst)
-  uint64_t sdl[SMALL_MAX], sil[SMALL_MAX];   // the same sorted by (dst, src)
-  uint64_t rows[2][SMALL_MAX];
-  int64_t plan[2][4 * SMALL_MAX];
-  int64_t sofs[2][SMALL_MAX + 1], cpre[2][SMALL_MAX + 1], wpre[2][SMALL_MAX + 1];
-  SmallStatus st;
+// device arrays of one small batch, all in one scratch buffer
+struct dfpr::SmallBufs {
+  uint64_t* key;           // packed (src, dst, insertion, present)
+  uint64_t *dl[2], *il[2];   // Delta-, Delta+ sorted by (src, dst) and by (dst, src)
+  int32_t* rows[2];
+  int4* plan[2];           // per touched row: its deletions [x, y) and insertions [z, w)
+  int32_t* od[2];          // its degree before the batch
+  int32_t *lrow[2], *lpre[2];   // rows longer than a chunk: index into rows, chunks before
+  SmallStatus* st;
 };
 
-constexpr size_t SMALL_SMEM = sizeof(uint64_t) * (2 * SMALL_SORT + SMALL_MAX) + sizeof(int64_t) * SMALL_MAX;
+namespace dfpr {
+
+static size_t small_carve(void* base, int64_t cap, SmallBufs* B) {
+  Carve c(base);
+  B->key = c.take<uint64_t>(cap);
+  B->dl[0] = B->il[0] = nullptr;   // the graph's own buffers
+  B->dl[1] = c.take<uint64_t>(cap);
+  B->il[1] = c.take<uint64_t>(cap);
+  for (int d = 0; d < 2; d++) {
+    B->rows[d] = c.take<int32_t>(cap);
+    B->plan[d] = c.take<int4>(cap);
+    B->od[d] = c.take<int32_t>(cap);
+    B->lrow[d] = c.take<int32_t>(cap);
+    B->lpre[d] = c.take<int32_t>(cap + 1);
+  }
+  B->st = c.take<SmallStatus>(1);
+  return c.used;
+}
 
 __host__ __device__ __forceinline__ int pow2_at_least(int x) {
-  int p = x > 0 ? 1 : 0;
+  int p = 1;
   while (p < x) p <<= 1;
   return p;
 }
 
-// ascending bitonic sort of a[0..N), N a power of two (or 0), whole block
-__device__ void block_bitonic(uint64_t* a, int N) {
-  for (int k = 2; k <= N; k <<= 1)
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        const int x = i ^ j;
-        if (x > i) {
-          const uint64_t p = a[i], q = a[x];
-          if ((p > q) == ((i & k) == 0)) {
-            a[i] = q;
-            a[x] = p;
+// whether x is in the sorted row[0..deg): seven pivots per step, their loads
+// together, then the last few elements together
+__device__ __forceinline__ bool in_sorted_row(const int32_t* __restrict__ row, int32_t deg, int32_t x) {
+  int32_t lo = 0, hi = deg;   // the first element >= x is at [lo, hi]
+  while (hi - lo > 8) {
+    const int32_t s = (hi - lo) >> 3;
+    int c = 0;
+#pragma unroll
+    for (int k = 1; k < 8; k++) c += row[lo + k * s] < x ? 1 : 0;
+    const int32_t l2 = c > 0 ? lo + c * s + 1 : lo;
+    hi = c < 7 ? lo + (c + 1) * s : hi;
+    lo = l2;
+  }
+  bool found = false;
+#pragma unroll
+  for (int k = 0; k <= 8; k++) found |= lo + k <= hi && lo + k < deg && row[lo + k] == x;
+  return found;
+}
+
+__global__ void __launch_bounds__(256) k_small_keys(const int32_t* __restrict__ ds, const int32_t* __restrict__ dd, int nd,
+                                                    const int32_t* __restrict__ is, const int32_t* __restrict__ id,
+                                                    int ni, int32_t n, int bits, const int32_t* __restrict__ perm,
+                                                    const int64_t* __restrict__ oo, const int32_t* __restrict__ od,
+                                                    const int32_t* __restrict__ oc, uint64_t* __restrict__ key) {
+  GRID_STRIDE(i, nd + ni) {
+    const bool del = i < nd;
+    const int32_t u = del ? ds[i] : is[i - nd], v = del ? dd[i] : id[i - nd];
+    uint64_t k = DROP;   // self-loops are re-added with every batch
+    if (u < 0 || u >= n || v < 0 || v >= n) {
+      k = BAD;
+    } else if (u != v) {
+      const int32_t a = perm[u], b = perm[v];
+      const bool present = in_sorted_row(oc + oo[a], od[a], b);
+      k = (((((uint64_t)a << bits) | (uint64_t)b) << 1 | (del ? 0u : 1u)) << 1) | (present ? 1u : 0u);
+    }
+    key[i] = k;
+  }
+}
+
+// ascending bitonic sort of the block's P keys (a power of two, at most
+// SMALL_THREADS x E), thread t holding keys [t E, t E + E); x: P keys of shared
+// memory
+template <int E>
+__device__ __forceinline__ void block_sort(uint64_t (&k)[E], int P, uint64_t* x) {
+  const int t = threadIdx.x;
+  for (int size = 2; size <= P; size <<= 1)
+    for (int j = size >> 1; j > 0; j >>= 1) {
+      if (j < E) {
+#pragma unroll
+        for (int jj = E / 2; jj > 0; jj >>= 1)
+          if (j == jj) {
+#pragma unroll
+            for (int e = 0; e < E; e++)
+              if ((e & jj) == 0) {
+                const bool up = ((t * E + e) & size) == 0;
+                const uint64_t a = k[e], b = k[e | jj];
+                const bool sw = (a > b) == up;
+                k[e] = sw ? b : a;
+                k[e | jj] = sw ? a : b;
+              }
           }
+      } else if (j < 32 * E) {
+#pragma unroll
+        for (int e = 0; e < E; e++) {
+          const int i = t * E + e;
+          const uint64_t o = __shfl_xor_sync(0xffffffffu, k[e], j / E);
+          const bool low = ((i & j) == 0) == ((i & size) == 0);   // keeps the smaller
+          k[e] = (o < k[e]) == low ? o : k[e];
+        }
+      } else {
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < E; e++) x[e * SMALL_THREADS + t] = k[e];
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < E; e++) {
+          const int i = t * E + e;
+          const uint64_t o = x[e * SMALL_THREADS + (t ^ (j / E))];
+          const bool low = ((i & j) == 0) == ((i & size) == 0);
+          k[e] = (o < k[e]) == low ? o : k[e];
         }
       }
-      __syncthreads();
     }
 }
 
-// exclusive prefix sum of w[0..len) in place, whole block; returns the total
-__device__ int64_t block_excl_scan(int64_t* w, int len, int64_t* wsum /* 32 */) {
-  const int T = blockDim.x, tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
-  const int per = (len + T - 1) / T;
-  const int b = min(tid * per, len), e = min(b + per, len);
-  int64_t loc = 0;
-  for (int i = b; i < e; i++) loc += w[i];
-  int64_t x = loc;
+// exclusive prefix of one value per thread over the block; *total the sum
+__device__ __forceinline__ uint64_t block_excl(uint64_t v, uint64_t* wsum /* 33 */, uint64_t* total) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  uint64_t x = v;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+    const uint64_t y = __shfl_up_sync(0xffffffffu, x, o);
     if (lane >= o) x += y;
   }
-  if (lane == 31) wsum[wp] = x;
+  __syncthreads();   // wsum may still be read from the call before
+  if (lane == 31) wsum[w] = x;
   __syncthreads();
-  if (wp == 0) {
-    int64_t z = lane < (T >> 5) ? wsum[lane] : 0;
+  if (w == 0) {
+    uint64_t z = wsum[lane];
+    const uint64_t own = z;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      int64_t y = __shfl_up_sync(0xffffffffu, z, o);
+      const uint64_t y = __shfl_up_sync(0xffffffffu, z, o);
       if (lane >= o) z += y;
     }
-    wsum[lane] = z;
+    wsum[lane] = z - own;
+    if (lane == 31) wsum[32] = z;
   }
   __syncthreads();
-  int64_t before = (wp ? wsum[wp - 1] : 0) + x - loc;
-  const int64_t total = wsum[(T >> 5) - 1];
-  for (int i = b; i < e; i++) {
-    const int64_t v = w[i];
-    w[i] = before;
-    before += v;
-  }
-  __syncthreads();
-  return total;
+  *total = wsum[32];
+  return wsum[w] + x - v;
 }
 
-// touched rows of one direction and their edit plans; L holds the deletions
-// [0, nde) and insertions [nde, nde + nie), each sorted by (row, col)
-__device__ void small_plan(int dir, const uint64_t* L, int nde, int nie, int bits, const int64_t* __restrict__ off,
-                           const int32_t* __restrict__ deg, int64_t scap, uint64_t* R, int64_t* W, int64_t* wsum,
-                           SmallBufs* B) {
-  __shared__ int ovf;
-  const int tid = threadIdx.x, T = blockDim.x;
-  const int tot = nde + nie, P = pow2_at_least(tot);
-  if (tid == 0) ovf = 0;
-  for (int i = tid; i < P; i += T) R[i] = i < tot ? (L[i] >> bits) : DROP;
-  __syncthreads();
-  block_bitonic(R, P);
-  for (int i = tid; i < tot; i += T) W[i] = (i == 0 || R[i - 1] != R[i]) ? 1 : 0;
-  __syncthreads();
-  const int nr = (int)block_excl_scan(W, tot, wsum);
-  uint64_t* rows = B->rows[dir];
-  for (int i = tid; i < tot; i += T)
-    if (i == 0 || R[i - 1] != R[i]) rows[W[i]] = R[i];
-  __syncthreads();
-  int64_t* plan = B->plan[dir];
-  for (int j = tid; j < nr; j += T) {
-    const uint64_t r = rows[j];
-    const int64_t d0 = lower_key(L, 0, nde, r << bits), d1 = lower_key(L, d0, nde, (r + 1) << bits);
-    const int64_t i0 = lower_key(L + nde, 0, nie, r << bits), i1 = lower_key(L + nde, i0, nie, (r + 1) << bits);
-    const int64_t dg = deg[r];
-    const int64_t nd2 = dg - (d1 - d0) + (i1 - i0);
-    plan[4 * j + 0] = d0;
-    plan[4 * j + 1] = d1;
-    plan[4 * j + 2] = i0;
-    plan[4 * j + 3] = i1;
-    if (round4(nd2) > off[r + 1] - off[r]) ovf = 1;
-    W[j] = dg;
-  }
-  __syncthreads();
-  const int64_t stot = block_excl_scan(W, nr, wsum);
-  for (int j = tid; j < nr; j += T) B->sofs[dir][j] = W[j];
-  for (int j = tid; j < nr; j += T) W[j] = cdiv((int64_t)deg[rows[j]], RW_CH);
-  __syncthreads();
-  const int64_t ctot = block_excl_scan(W, nr, wsum);
-  for (int j = tid; j < nr; j += T) B->cpre[dir][j] = W[j];
-  for (int j = tid; j < nr; j += T) {
-    const int64_t dg = deg[rows[j]];
-    const int64_t nd2 = dg - (plan[4 * j + 1] - plan[4 * j]) + (plan[4 * j + 3] - plan[4 * j + 2]);
-    W[j] = cdiv(round4(dg > nd2 ? dg : nd2), RW_CH);
-  }
-  __syncthreads();
-  const int64_t wtot = block_excl_scan(W, nr, wsum);
-  for (int j = tid; j < nr; j += T) B->wpre[dir][j] = W[j];
-  if (tid == 0) {
-    B->sofs[dir][nr] = stot;
-    B->cpre[dir][nr] = ctot;
-    B->wpre[dir][nr] = wtot;
-    SmallStatus& st = B->st;
-    st.nr[dir] = nr;
-    st.stot[dir] = stot;
-    st.ovf[dir] = ovf;
-    st.need[dir] = stot > scap ? 1 : 0;
-    st.skip[dir] = (ovf || stot > scap) ? 1 : 0;
-  }
-  __syncthreads();
+struct SmallCsr {
+  const int64_t* off;
+  const int32_t* deg;
+  int64_t scap;   // scratch elements for rows longer than a chunk
+};
+
+// shared memory: the keys, and per key the deletions before it and the first
+// key of each row
+template <int E>
+constexpr size_t small_smem() {
+  return (sizeof(uint64_t) + 2 * sizeof(uint16_t)) * (size_t)(SMALL_THREADS * E + 8);
 }
 
-__global__ void __launch_bounds__(SMALL_THREADS) k_small_ingest(
-    const int32_t* __restrict__ ds, const int32_t* __restrict__ dd, int nd, const int32_t* __restrict__ is,
-    const int32_t* __restrict__ id, int ni, int32_t n, int bits, const int32_t* __restrict__ perm,
-    const int64_t* __restrict__ ooff, const int32_t* __restrict__ odeg, const int32_t* __restrict__ ocol,
-    const int64_t* __restrict__ ioff, const int32_t* __restrict__ ideg, int64_t scap_out, int64_t scap_in,
-    SmallBufs* B) {
-  extern __shared__ uint64_t smem[];
-  uint64_t* A = smem;                           // SMALL_SORT: sorts
-  uint64_t* L = A + SMALL_SORT;                 // SMALL_MAX: effective lists of the current direction
-  uint64_t* R = L + SMALL_MAX;                  // SMALL_SORT: row ids, flags
-  int64_t* W = reinterpret_cast<int64_t*>(R + SMALL_SORT);   // SMALL_MAX: scans
-  __shared__ int64_t wsum[32];
-  __shared__ int bad;
-  const int tid = threadIdx.x, T = blockDim.x;
+template <int E>
+__global__ void __launch_bounds__(SMALL_THREADS, 1)
+    k_small_ingest(int N, int bits, const __grid_constant__ SmallCsr out, const __grid_constant__ SmallCsr in,
+                   const __grid_constant__ SmallBufs B) {
+  extern __shared__ uint64_t K[];   // the sorted keys, then the effective changes (row, col, insertion)
+  uint16_t* const DP = reinterpret_cast<uint16_t*>(K + SMALL_THREADS * E + 8);
+  uint16_t* const RS = DP + SMALL_THREADS * E + 8;
+  __shared__ uint64_t wsum[33];
+  const int dir = blockIdx.x, t = threadIdx.x;
+  const SmallCsr& c = dir == 0 ? out : in;
   const uint64_t mask = (1ull << bits) - 1;
-  if (tid == 0) bad = 0;
-  __syncthreads();
-  const int Pd = pow2_at_least(nd), Pi = pow2_at_least(ni);
-  uint64_t* dk = A;
-  uint64_t* ik = A + Pd;
-  // keys in internal ids; self-loops and padding sort last as DROP
-  for (int i = tid; i < Pd + Pi; i += T) {
-    const bool del = i < Pd;
-    const int k = del ? i : i - Pd;
-    uint64_t key = DROP;
-    if (k < (del ? nd : ni)) {
-      const int32_t u = del ? ds[k] : is[k], v = del ? dd[k] : id[k];
-      if (u < 0 || u >= n || v < 0 || v >= n) bad = 1;
-      else if (u != v) key = ((uint64_t)perm[u] << bits) | (uint64_t)perm[v];
+  SmallStatus& st = *B.st;
+  uint64_t k[E];
+  bool bad = false;
+#pragma unroll
+  for (int e = 0; e < E; e++) {
+    const int i = t * E + e;
+    k[e] = i < N ? B.key[i] : DROP;
+    bad |= k[e] == BAD;
+    if (dir == 1 && k[e] != DROP) {
+      const uint64_t edge = k[e] >> 2;
+      k[e] = (((edge & mask) << bits | edge >> bits) << 2) | (k[e] & 3);
     }
-    A[i] = key;
   }
-  __syncthreads();
-  if (bad) {
-    if (tid == 0) {
-      SmallStatus& st = B->st;
-      memset(&st, 0, sizeof(st));
+  if (__syncthreads_or(bad)) {
+    if (t == 0) {
       st.bad = 1;
-      st.skip[0] = st.skip[1] = 1;
+      st.nr[dir] = st.nlong[dir] = st.chunks[dir] = 0;
+      st.skip[dir] = 1;
     }
     return;
   }
-  block_bitonic(dk, Pd);
-  block_bitonic(ik, Pi);
+  const int P = pow2_at_least(N);
+  block_sort<E>(k, P, K);
+  __syncthreads();
+#pragma unroll
+  for (int e = 0; e < E; e++)
+    if (t * E + e < P) K[t * E + e] = k[e];
+  __syncthreads();
   // effective flags (Sec. 3.2): a deletion is a first occurrence, present in
-  // E_{t-1} and not re-inserted; an insertion is a first occurrence absent from E_{t-1}
-  for (int i = tid; i < nd + ni; i += T) {
-    const bool del = i < nd;
-    const uint64_t key = del ? dk[i] : ik[i - nd];
-    const uint64_t prev = del ? (i > 0 ? dk[i - 1] : DROP) : (i > nd ? ik[i - nd - 1] : DROP);
-    bool e = key != DROP && key != prev;
-    if (e) {
-      const int32_t u = (int32_t)(key >> bits), v = (int32_t)(key & mask);
-      const bool present = in_row(ocol, ooff[u], odeg[u], v);
-      e = del ? (present && !key_in(ik, ni, key)) : !present;
+  // E_{t-1} and not re-inserted; an insertion is a first occurrence absent from
+  // E_{t-1}.  Equal edges lie together, deletions first.
+  unsigned fd = 0, fi = 0;
+#pragma unroll
+  for (int e = 0; e < E; e++) {
+    const int i = t * E + e;
+    const uint64_t x = k[e];
+    if (i >= P || x == DROP || (i > 0 && K[i - 1] == x)) continue;
+    if (x & 2) {
+      if (!(x & 1)) fi |= 1u << e;
+    } else if (x & 1) {
+      int j = i + 1;
+      while (j < P && K[j] == x) j++;
+      if (!(j < P && (K[j] >> 1) == ((x >> 1) | 1))) fd |= 1u << e;
     }
-    R[i] = e;
-    W[i] = e;
   }
+  uint64_t tot;
+  uint64_t pre = block_excl((uint64_t)__popc(fd) | (uint64_t)__popc(fi) << 32, wsum, &tot);   // (its barriers end the reads of K)
+  const int nde = (int)(uint32_t)tot, nie = (int)(tot >> 32), ne = nde + nie;
+  {
+    int pd = (int)(uint32_t)pre, pi = (int)(pre >> 32);
+#pragma unroll
+    for (int e = 0; e < E; e++) {
+      const bool d = (fd >> e) & 1u, a = (fi >> e) & 1u;
+      if (!d && !a) continue;
+      K[pd + pi] = k[e] >> 1;
+      DP[pd + pi] = (uint16_t)pd;
+      if (d) B.dl[dir][pd++] = k[e] >> 2;
+      else B.il[dir][pi++] = k[e] >> 2;
+    }
+  }
+  if (t == 0) DP[ne] = (uint16_t)nde;
   __syncthreads();
-  const int nde = (int)block_excl_scan(W, nd, wsum);
-  const int nie = (int)block_excl_scan(W + nd, ni, wsum);
-  for (int i = tid; i < nd + ni; i += T) {
-    if (!R[i]) continue;
-    if (i < nd) {
-      L[W[i]] = dk[i];
-      B->edl[W[i]] = dk[i];
+  // touched rows
+  unsigned heads = 0;
+#pragma unroll
+  for (int e = 0; e < E; e++) {
+    const int i = t * E + e;
+    if (i < ne && (i == 0 || K[i] >> (bits + 1) != K[i - 1] >> (bits + 1))) heads |= 1u << e;
+  }
+  pre = block_excl((uint64_t)__popc(heads), wsum, &tot);
+  const int nr = (int)tot;
+  {
+    int j = (int)pre;
+#pragma unroll
+    for (int e = 0; e < E; e++)
+      if ((heads >> e) & 1u) RS[j++] = (uint16_t)(t * E + e);
+  }
+  if (t == 0) RS[nr] = (uint16_t)ne;
+  __syncthreads();
+  // their edit plans; rows longer than a chunk are listed with their chunks
+  bool ovf = false;
+  uint64_t carry = 0;
+  for (int j0 = 0; j0 < nr; j0 += SMALL_THREADS) {
+    const int j = j0 + t;
+    uint64_t longs = 0;
+    if (j < nr) {
+      const int a = RS[j], b = RS[j + 1];
+      const int d0 = DP[a], d1 = DP[b], i0 = a - d0, i1 = b - d1;
+      const int32_t r = (int32_t)(K[a] >> (bits + 1));
+      const int32_t dg = c.deg[r];
+      const int32_t dn = dg - (d1 - d0) + (i1 - i0);
+      B.rows[dir][j] = r;
+      B.plan[dir][j] = make_int4(d0, d1, i0, i1);
+      B.od[dir][j] = dg;
+      ovf |= round4(dn) > c.off[r + 1] - c.off[r];
+      const int32_t len = dg > dn ? dg : dn;
+      if (len > RW_CH) longs = 1ull << 32 | (uint64_t)cdiv(round4(len), RW_CH);
+    }
+    if (__syncthreads_or(longs != 0)) {
+      const uint64_t before = carry + block_excl(longs, wsum, &tot);
+      if (longs) {
+        B.lrow[dir][before >> 32] = j;
+        B.lpre[dir][before >> 32] = (int32_t)(uint32_t)before;
+      }
+      carry += tot;
+    }
+  }
+  const int any_ovf = __syncthreads_or(ovf);
+  if (t == 0) {
+    const int64_t chunks = (int64_t)(uint32_t)carry;
+    st.bad = 0;
+    st.n_del = nde;
+    st.n_ins = nie;
+    st.nr[dir] = nr;
+    st.nlong[dir] = (int32_t)(carry >> 32);
+    st.chunks[dir] = (int32_t)chunks;
+    B.lpre[dir][carry >> 32] = (int32_t)chunks;
+    st.ovf[dir] = any_ovf ? 1 : 0;
+    st.need[dir] = chunks * RW_CH > c.scap ? 1 : 0;
+    st.skip[dir] = st.ovf[dir] | st.need[dir];
+  }
+}
+
+struct SmallEdit {
+  const int64_t* off[2];
+  int32_t* deg[2];
+  int32_t* col[2];
+  int32_t* S[2];          // scratch of rows longer than a chunk: chunk c of the direction at c x RW_CH
+  int32_t sent;
+  const double* R;        // ranks, or null: no contributions to refresh
+  long long* C;
+  const double* tab_sc;
+  int dirs;               // bit d: work on direction d
+};
+
+// the long row that chunk c belongs to
+__device__ __forceinline__ int long_row(const int32_t* pre, int nlong, int c) {
+  int lo = 0, hi = nlong - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (pre[mid] <= c) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
+__global__ void __launch_bounds__(256) k_small_copy(const __grid_constant__ SmallBufs B,
+                                                    const __grid_constant__ SmallEdit p) {
+  const SmallStatus& st = *B.st;
+  const int lane = threadIdx.x & 31;
+  const int nw = (gridDim.x * blockDim.x) >> 5, w0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  for (int d = 0; d < 2; d++) {
+    if (!((p.dirs >> d) & 1) || st.skip[d]) continue;
+    const int nc = st.chunks[d];
+    for (int c = w0; c < nc; c += nw) {
+      const int l = long_row(B.lpre[d], st.nlong[d], c), j = B.lrow[d][l];
+      const int32_t x0 = (c - B.lpre[d][l]) * RW_CH, x1 = min(x0 + RW_CH, B.od[d][j]);
+      const int32_t* row = p.col[d] + p.off[d][B.rows[d][j]];
+      int32_t* S = p.S[d] + (int64_t)B.lpre[d][l] * RW_CH;
+      for (int32_t x = x0 + lane; x < x1; x += 32) S[x] = row[x];
+    }
+  }
+}
+
+__device__ __forceinline__ int32_t lower_i32(const int32_t* a, int32_t lo, int32_t hi, int32_t x) {
+  while (lo < hi) {
+    const int32_t mid = (lo + hi) >> 1;
+    if (a[mid] < x) lo = mid + 1;
+    else hi = mid;
+  }
+  return lo;
+}
+
+// one warp: positions [x0, x1) of a touched row (old elements S[0..d_old), the
+// padding after them included) and its insertions [k0, k1) written to their
+// new places: a survivor x goes to x - (deletions below it) + (insertions below
+// it), an insertion to its rank among the insertions + old elements below it -
+// deletions below it
+__device__ __forceinline__ void edit_row_part(const int32_t* S, int32_t x0, int32_t x1, int k0, int k1, int32_t r, int4 pl,
+                                              int32_t d_old, int32_t cap, const uint64_t* __restrict__ dl,
+                                              const uint64_t* __restrict__ il, uint64_t mask, int bits,
+                                              int32_t* __restrict__ row, int32_t sent) {
+  const int lane = threadIdx.x & 31;
+  const int nd = pl.y - pl.x, ni = pl.w - pl.z;
+  const int32_t d_new = d_old - nd + ni;
+  const bool few = nd + ni <= 32;   // the row's changes in registers, one per lane
+  const int32_t mine = few && lane < nd + ni ? (int32_t)((lane < nd ? dl[pl.x + lane] : il[pl.z + lane - nd]) & mask) : 0;
+  const uint64_t rk = (uint64_t)r << bits;
+  for (int32_t xb = x0; xb < x1; xb += 32) {
+    const int32_t x = xb + lane;
+    const bool old = x < x1 && x < d_old;
+    const int32_t v = old ? S[x] : 0;
+    int dlt = 0, ilt = 0;
+    bool dead = false;
+    if (few) {
+      for (int k = 0; k < nd; k++) {
+        const int32_t y = __shfl_sync(0xffffffffu, mine, k);
+        dlt += y < v;
+        dead |= y == v;
+      }
+      for (int k = nd; k < nd + ni; k++) ilt += __shfl_sync(0xffffffffu, mine, k) < v;
+    } else if (old) {
+      const int64_t a = lower_key(dl, pl.x, pl.y, rk | (uint64_t)v);
+      dead = a < pl.y && dl[a] == (rk | (uint64_t)v);
+      dlt = (int)(a - pl.x);
+      ilt = (int)(lower_key(il, pl.z, pl.w, rk | (uint64_t)v) - pl.z);
+    }
+    if (old && !dead) {
+      const int32_t pos = x - dlt + ilt;
+      if (pos >= 0 && pos < cap) row[pos] = v;
+    }
+    if (x < x1 && x >= d_new && x < cap) row[x] = sent;
+  }
+  for (int k = k0 + lane; k < k1; k += 32) {
+    const int32_t y = (int32_t)(il[k] & mask);
+    const int32_t pos = (k - pl.z) + lower_i32(S, 0, d_old, y) - (int32_t)(lower_key(dl, pl.x, pl.y, rk | (uint64_t)y) - pl.x);
+    if (pos >= 0 && pos < cap) row[pos] = y;
+  }
+}
+
+__global__ void __launch_bounds__(256) k_small_edit(const __grid_constant__ SmallBufs B,
+                                                    const __grid_constant__ SmallEdit p, int bits) {
+  __shared__ int32_t stage[8][RW_CH];
+  const SmallStatus& st = *B.st;
+  const int lane = threadIdx.x & 31;
+  const int nw = (gridDim.x * blockDim.x) >> 5;
+  const uint64_t mask = (1ull << bits) - 1;
+  // the work: touched rows of both directions, then chunks of both
+  const bool on0 = (p.dirs & 1) && !st.skip[0], on1 = (p.dirs & 2) && !st.skip[1];
+  const int e0 = on0 ? st.nr[0] : 0, e1 = e0 + (on1 ? st.nr[1] : 0);
+  const int e2 = e1 + (on0 ? st.chunks[0] : 0), e3 = e2 + (on1 ? st.chunks[1] : 0);
+  for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < e3; w += nw) {
+    const bool chunk = w >= e1;
+    const int d = chunk ? (w >= e2 ? 1 : 0) : (w >= e0 ? 1 : 0);
+    const int item = chunk ? w - (d ? e2 : e1) : w - (d ? e0 : 0);
+    const int l = chunk ? long_row(B.lpre[d], st.nlong[d], item) : 0;
+    const int j = chunk ? B.lrow[d][l] : item;
+    const int32_t r = B.rows[d][j], d_old = B.od[d][j];
+    const int4 pl = B.plan[d][j];
+    const int32_t d_new = d_old - (pl.y - pl.x) + (pl.w - pl.z);
+    const int32_t len = d_old > d_new ? d_old : d_new;
+    const int64_t base = p.off[d][r];
+    const int64_t cap64 = p.off[d][r + 1] - base;
+    const int32_t cap = (int32_t)(cap64 < INT32_MAX ? cap64 : INT32_MAX), end = (int32_t)round4(len);
+    int32_t* const row = p.col[d] + base;
+    if (!chunk) {
+      if (len > RW_CH) continue;   // a long row: its chunks are items of their own
+      int32_t* const S = stage[threadIdx.x >> 5];
+      __syncwarp();
+      for (int32_t x = lane; x < d_old; x += 32) S[x] = row[x];
+      __syncwarp();
+      edit_row_part(S, 0, end, pl.z, pl.w, r, pl, d_old, cap, B.dl[d], B.il[d], mask, bits, row, p.sent);
     } else {
-      L[nde + W[i]] = ik[i - nd];
-      B->eil[W[i]] = ik[i - nd];
+      const int part = item - B.lpre[d][l], parts = B.lpre[d][l + 1] - B.lpre[d][l];
+      const int per = (pl.w - pl.z + parts - 1) / parts;
+      const int k0 = min(pl.z + part * per, pl.w), k1 = min(k0 + per, pl.w);
+      edit_row_part(p.S[d] + (int64_t)B.lpre[d][l] * RW_CH, part * RW_CH, min((part + 1) * RW_CH, end), k0, k1, r, pl,
+                    d_old, cap, B.dl[d], B.il[d], mask, bits, row, p.sent);
+      if (part > 0) continue;
     }
-  }
-  __syncthreads();
-  small_plan(0, L, nde, nie, bits, ooff, odeg, scap_out, R, W, wsum, B);
-  // the same lists keyed (dst, src) for the in-CSR
-  const int Pde = pow2_at_least(nde), Pie = pow2_at_least(nie);
-  for (int i = tid; i < Pde + Pie; i += T) {
-    const bool del = i < Pde;
-    const int k = del ? i : i - Pde;
-    uint64_t key = DROP;
-    if (k < (del ? nde : nie)) {
-      const uint64_t x = L[del ? k : nde + k];
-      key = ((x & mask) << bits) | (x >> bits);
+    if (lane == 0) {
+      p.deg[d][r] = d_new;
+      if (d == 0 && p.R) {   // the source's contribution with its new out-degree
+        const double sc = d_new < TAB ? p.tab_sc[d_new] : FIX_ONE / (double)d_new;
+        p.C[r] = __double2ll_rn(p.R[r] * sc);
+      }
     }
-    A[i] = key;
-  }
-  __syncthreads();
-  block_bitonic(A, Pde);
-  block_bitonic(A + Pde, Pie);
-  for (int i = tid; i < nde + nie; i += T) {
-    const bool del = i < nde;
-    const uint64_t key = del ? A[i] : A[Pde + i - nde];
-    L[i] = key;
-    if (del) B->sdl[i] = key;
-    else B->sil[i - nde] = key;
-  }
-  __syncthreads();
-  small_plan(1, L, nde, nie, bits, ioff, ideg, scap_in, R, W, wsum, B);
-  if (tid == 0) {
-    B->st.n_del = nde;
-    B->st.n_ins = nie;
-    B->st.bad = 0;
   }
 }
 
-// contributions of the touched out-rows' vertices (the sources of the change)
-__global__ void k_small_contrib(const uint64_t* __restrict__ rows, const int64_t* __restrict__ nrp,
-                                const int32_t* skip, const double* __restrict__ R, long long* __restrict__ C,
-                                const int32_t* __restrict__ odeg, const double* __restrict__ tab_sc) {
-  if (*skip) return;
-  const int64_t nr = *nrp;
-  GRID_STRIDE(j, nr) {
-    const int32_t u = (int32_t)rows[j];
-    const int32_t d = odeg[u];
-    const double sc = d < TAB ? tab_sc[d] : FIX_ONE / (double)d;
-    C[u] = __double2ll_rn(R[u] * sc);
-  }
-}
-
-static void launch_small_edit(Graph* g, Csr* c, SmallBufs* B, int dir, int32_t* S, int64_t nk) {
+static void launch_small_edit(Graph* g, const SmallApply* A, int dirs) {
   cudaStream_t s = g->stream;
-  const int bits = g->id_bits;
-  const uint64_t* dl = dir == 0 ? B->edl : B->sdl;
-  const uint64_t* il = dir == 0 ? B->eil : B->sil;
-  const int32_t* skip = &B->st.skip[dir];
-  const int64_t* nrp = &B->st.nr[dir];
-  const int wgrid = num_sms() * 4;
-  note_launch(); k_row_copy<<<wgrid, 256, 0, s>>>(B->rows[dir], nrp, B->sofs[dir], B->cpre[dir], c->off, c->deg, c->col,
-                                                 S, skip);
-  note_launch(); k_row_survivors<<<wgrid, 256, 0, s>>>(B->rows[dir], nrp, B->plan[dir], B->sofs[dir], B->wpre[dir], dl,
-                                                      il, bits, c->off, c->deg, c->col, S, g->n, skip);
-  note_launch(); k_row_insertions<<<grid_for(nk, 256), 256, 0, s>>>(B->rows[dir], nrp, B->plan[dir], B->sofs[dir], dl, il,
-                                                                   &B->st.n_ins, bits, c->off, c->deg, c->col, S, skip);
-  note_launch(); k_row_degrees<<<grid_for(nk, 256), 256, 0, s>>>(B->rows[dir], nrp, B->plan[dir], c->deg, skip);
+  SmallEdit p;
+  const Csr* c[2] = {&g->out, &g->in};
+  for (int d = 0; d < 2; d++) {
+    p.off[d] = c[d]->off;
+    p.deg[d] = c[d]->deg;
+    p.col[d] = c[d]->col;
+    p.S[d] = A->S[d];
+  }
+  p.sent = g->n;
+  p.R = g->has_ranks ? g->R : nullptr;
+  p.C = g->C[g->ccur];
+  p.tab_sc = g->tab_sc;
+  p.dirs = dirs;
+  note_launch(); k_small_copy<<<num_sms() * 2, 256, 0, s>>>(*A->B, p);
+  note_launch(); k_small_edit<<<num_sms() * 4, 256, 0, s>>>(*A->B, p, g->id_bits);
 }
 
-// grow-only staging buffer of one direction (scratch slot 5: out, 7: in)
+// grow-only scratch of one direction's long rows (scratch slot 5: out, 7: in)
 static cudaError_t small_staging(Graph* g, int dir, int64_t elems, int32_t** out, int64_t* cap) {
   const int slot = dir == 0 ? 5 : 7;
   void* p;
@@ -922,101 +1128,125 @@ static cudaError_t small_staging(Graph* g, int dir, int64_t elems, int32_t** out
   return cudaSuccess;
 }
 
+// the list of one side of the effective change with room for `need` keys,
+// keeping the keys it holds (a batch that is refused leaves the last one's
+// change in place)
+static cudaError_t grow_delta(Graph* g, uint64_t** list, int64_t* cap, int64_t used, int64_t need) {
+  if (*cap >= need) return cudaSuccess;
+  uint64_t* p = nullptr;
+  cudaError_t e = dev_malloc(&p, sizeof(uint64_t) * (size_t)(need + 1));
+  if (e != cudaSuccess) return e;
+  if (used > 0)
+    e = cudaMemcpyAsync(p, *list, sizeof(uint64_t) * (size_t)used, cudaMemcpyDeviceToDevice, g->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
+  if (e != cudaSuccess) {
+    cudaFree(p);
+    return e;
+  }
+  if (*list) cudaFree(*list);
+  *list = p;
+  *cap = need;
+  return cudaSuccess;
+}
+
+template <int E>
+static cudaError_t launch_ingest(Graph* g, int N, const SmallCsr& out, const SmallCsr& in, const SmallBufs& B) {
+  int bps;   // (raises the kernel's shared memory limit once)
+  cudaError_t e = gather_occupancy((const void*)k_small_ingest<E>, SMALL_THREADS, small_smem<E>(), &bps);
+  if (e != cudaSuccess) return e;
+  note_launch();
+  k_small_ingest<E><<<2, SMALL_THREADS, small_smem<E>(), g->stream>>>(N, g->id_bits, out, in, B);
+  return cudaGetLastError();
+}
+
 // phase 1 of a small batch: everything up to the status copy to the host,
 // queued on the graph's stream without waiting
 static int small_launch(Graph* g, const int32_t* ds, const int32_t* dd, int64_t nd, const int32_t* is,
                         const int32_t* id, int64_t ni, SmallApply* A) {
   cudaStream_t s = g->stream;
-  const int32_t n = g->n;
-  const int64_t nk = nd + ni;
+  const int N = (int)(nd + ni);
+  const int64_t cap = std::max(1024, pow2_at_least(N));
+  SmallBufs B;
   void* bp;
-  TRY(scratch_get(g, 6, sizeof(SmallBufs), &bp));
-  SmallBufs* B = (SmallBufs*)bp;
+  TRY(scratch_get(g, 6, small_carve(nullptr, cap, &B) + 256, &bp));
+  small_carve(bp, cap, &B);
   if (!g->small_h) TRY(cudaMallocHost(&g->small_h, sizeof(SmallStatus)));
-  SmallStatus* h = (SmallStatus*)g->small_h;
-  int32_t** S = A->S;
-  int64_t* cap = A->cap;
-  // staging of at least 64K elements per direction; larger rows are handled by growing it
-  TRY(small_staging(g, 0, 65536, &S[0], &cap[0]));
-  TRY(small_staging(g, 1, 65536, &S[1], &cap[1]));
-  static bool attr_set[64] = {false};
-  const bool known = g->dev >= 0 && g->dev < 64;
-  if (!known || !attr_set[g->dev]) {
-    TRY(cudaFuncSetAttribute(k_small_ingest, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMALL_SMEM));
-    if (known) attr_set[g->dev] = true;
+  TRY(grow_delta(g, &g->dmin, &g->cap_dmin, g->n_dmin, nd));
+  TRY(grow_delta(g, &g->dplus, &g->cap_dplus, g->n_dplus, ni));
+  B.dl[0] = g->dmin;
+  B.il[0] = g->dplus;
+  // scratch for at least 64 chunks of long rows per direction; more is handled by growing it
+  SmallCsr csr[2];
+  for (int d = 0; d < 2; d++) {
+    const Csr& c = d == 0 ? g->out : g->in;
+    TRY(small_staging(g, d, 65536, &A->S[d], &csr[d].scap));
+    csr[d].off = c.off;
+    csr[d].deg = c.deg;
   }
+  A->B = new (std::nothrow) SmallBufs(B);
+  if (!A->B) return set_error(g, ENOMEM_, "pr_apply_batch: host memory");
   note_launch();
-  k_small_ingest<<<1, SMALL_THREADS, SMALL_SMEM, s>>>(ds, dd, (int)nd, is, id, (int)ni, n, g->id_bits, g->perm,
-                                                      g->out.off, g->out.deg, g->out.col, g->in.off, g->in.deg, cap[0],
-                                                      cap[1], B);
-  TRY(cudaGetLastError());
-  launch_small_edit(g, &g->out, B, 0, S[0], nk);
-  launch_small_edit(g, &g->in, B, 1, S[1], nk);
-  if (g->has_ranks) {
-    note_launch();
-    k_small_contrib<<<grid_for(nk, 256), 256, 0, s>>>(B->rows[0], &B->st.nr[0], &B->st.skip[0], g->R, g->C[g->ccur],
-                                                      g->out.deg, g->tab_sc);
+  k_small_keys<<<grid_for(N, 256), 256, 0, s>>>(ds, dd, (int)nd, is, id, (int)ni, g->n, g->id_bits, g->perm, g->out.off,
+                                                g->out.deg, g->out.col, B.key);
+  cudaError_t e = N <= SMALL_THREADS       ? launch_ingest<1>(g, N, csr[0], csr[1], B)
+                  : N <= 2 * SMALL_THREADS ? launch_ingest<2>(g, N, csr[0], csr[1], B)
+                  : N <= 4 * SMALL_THREADS ? launch_ingest<4>(g, N, csr[0], csr[1], B)
+                  : N <= 8 * SMALL_THREADS ? launch_ingest<8>(g, N, csr[0], csr[1], B)
+                                           : launch_ingest<16>(g, N, csr[0], csr[1], B);
+  if (e == cudaSuccess) {
+    launch_small_edit(g, A, 3);
+    e = cudaGetLastError();
   }
-  TRY(cudaMemcpyAsync(h, &B->st, sizeof(SmallStatus), cudaMemcpyDeviceToHost, s));
-  A->B = B;
-  A->nk = nk;
+  if (e == cudaSuccess) e = cudaMemcpyAsync(g->small_h, B.st, sizeof(SmallStatus), cudaMemcpyDeviceToHost, s);
+  if (e != cudaSuccess) {
+    delete A->B;
+    A->B = nullptr;
+    return cuda_fail(g, e, "pr_apply_batch");
+  }
   return OK;
 }
 
 // phase 2: wait for the status, keep the effective change, and finish on the
-// host what the device left (a larger staging buffer, or a repack)
+// host what the device left (a larger scratch, or a repack)
 static int small_complete(Graph* g, SmallApply* A) {
   cudaStream_t s = g->stream;
   const int32_t n = g->n;
-  SmallBufs* B = A->B;
-  SmallStatus* h = (SmallStatus*)g->small_h;
-  int32_t** S = A->S;
-  int64_t* cap = A->cap;
-  const int64_t nk = A->nk;
+  const SmallBufs B = *A->B;
+  struct Release {
+    SmallApply* a;
+    ~Release() {
+      delete a->B;
+      a->B = nullptr;
+    }
+  } release{A};
   TRY(cudaStreamSynchronize(s));
-  if (h->bad) return set_error(g, ERANGE_, "pr_apply_batch: vertex id out of range");
-  const int64_t a = h->n_del, b = h->n_ins;
-  // the effective change, kept for the update (grow-only buffers owned by the graph)
-  if (g->cap_dmin < a) {
-    if (g->dmin) cudaFree(g->dmin);
-    g->dmin = nullptr;
-    g->cap_dmin = 0;
-    TRY(dev_malloc(&g->dmin, sizeof(uint64_t) * (a + 1)));
-    g->cap_dmin = a;
-  }
-  if (g->cap_dplus < b) {
-    if (g->dplus) cudaFree(g->dplus);
-    g->dplus = nullptr;
-    g->cap_dplus = 0;
-    TRY(dev_malloc(&g->dplus, sizeof(uint64_t) * (b + 1)));
-    g->cap_dplus = b;
-  }
-  if (a) TRY(cudaMemcpyAsync(g->dmin, B->edl, sizeof(uint64_t) * a, cudaMemcpyDeviceToDevice, s));
-  if (b) TRY(cudaMemcpyAsync(g->dplus, B->eil, sizeof(uint64_t) * b, cudaMemcpyDeviceToDevice, s));
+  g->stage_busy = false;
+  const SmallStatus h = *(SmallStatus*)g->small_h;
+  if (h.bad) return set_error(g, ERANGE_, "pr_apply_batch: vertex id out of range");
+  const int64_t a = h.n_del, b = h.n_ins;
   g->n_dmin = a;
   g->n_dplus = b;
   if (a + b == 0) return OK;
-  // directions the device skipped: a larger staging buffer, or a repack
-  bool redo_out = false, rep_in = false;
+  bool rep[2] = {false, false};
   for (int dir = 0; dir < 2; dir++) {
-    if (!h->skip[dir]) continue;
+    if (!h.skip[dir]) continue;
     Csr* c = dir == 0 ? &g->out : &g->in;
-    if (h->ovf[dir]) {
-      int rc = repack_direction(g, c, dir == 0 ? B->edl : B->sdl, a, dir == 0 ? B->eil : B->sil, b);
+    if (h.ovf[dir]) {
+      int rc = repack_direction(g, c, B.dl[dir], a, B.il[dir], b);
       if (rc) return rc;
-      if (dir == 1) rep_in = true;
+      rep[dir] = true;
     } else {
-      TRY(small_staging(g, dir, h->stot[dir], &S[dir], &cap[dir]));
-      TRY(cudaMemsetAsync(&B->st.skip[dir], 0, sizeof(int32_t), s));
-      launch_small_edit(g, c, B, dir, S[dir], nk);
+      int64_t cap;
+      TRY(small_staging(g, dir, (int64_t)h.chunks[dir] * RW_CH, &A->S[dir], &cap));
+      TRY(cudaMemsetAsync(&B.st->skip[dir], 0, sizeof(int32_t), s));
+      launch_small_edit(g, A, 1 << dir);
     }
-    if (dir == 0) redo_out = true;
   }
-  if (rep_in) {
+  if (rep[1]) {
     int rc = refresh_full_tiles(g);
     if (rc) return rc;
   }
-  if (redo_out && g->has_ranks) {
+  if (rep[0] && g->has_ranks) {
     TRY(cudaMemsetAsync(g->aux, 0, sizeof(uint32_t) * (size_t)(cdiv(n, 32) + 1), s));
     TRY(cudaMemsetAsync(&g->ctl->count[0], 0, sizeof(int32_t), s));
     TRY(launch_mark_sources(g->dmin, a, g->dplus, b, g->id_bits, g->aux, g->wl[0], &g->ctl->count[0], s));
@@ -1024,6 +1254,42 @@ static int small_complete(Graph* g, SmallApply* A) {
     TRY(cudaMemsetAsync(&g->ctl->count[0], 0, sizeof(int32_t), s));
   }
   TRY(cudaGetLastError());
+  return OK;
+}
+
+// the endpoint arrays of a host batch on the device (scratch slot 0): deletion
+// sources and targets, insertion sources and targets, one after another.  A
+// small batch goes through the graph's pinned buffer in one copy: four copies
+// from pageable memory take about 8 us of host time each.
+int stage_host_batch(Graph* g, const int32_t* ds, const int32_t* dd, int64_t nd, const int32_t* is, const int32_t* id,
+                     int64_t ni, int32_t** out) {
+  cudaStream_t s = g->stream;
+  void* stage;
+  TRY(scratch_get(g, 0, sizeof(int32_t) * (size_t)(2 * (nd + ni) + 4) + 1024, &stage));
+  int32_t* b = (int32_t*)stage;
+  *out = b;
+  const int32_t* src[4] = {ds, dd, is, id};
+  const int64_t len[4] = {nd, nd, ni, ni};
+  if (nd + ni <= SMALL_MAX) {
+    if (!g->stage_h) TRY(cudaMallocHost(&g->stage_h, sizeof(int32_t) * 2 * SMALL_MAX));
+    if (g->stage_busy) TRY(cudaDeviceSynchronize());   // the copy of a call that failed after it
+    int32_t* h = (int32_t*)g->stage_h;
+    for (int k = 0; k < 4; k++)
+      if (len[k]) {
+        memcpy(h, src[k], sizeof(int32_t) * (size_t)len[k]);
+        h += len[k];
+      }
+    if (nd + ni > 0) {
+      g->stage_busy = true;
+      TRY(cudaMemcpyAsync(b, g->stage_h, sizeof(int32_t) * 2 * (size_t)(nd + ni), cudaMemcpyHostToDevice, s));
+    }
+    return OK;
+  }
+  for (int k = 0; k < 4; k++)
+    if (len[k]) {
+      TRY(cudaMemcpyAsync(b, src[k], sizeof(int32_t) * (size_t)len[k], cudaMemcpyHostToDevice, s));
+      b += len[k];
+    }
   return OK;
 }
 

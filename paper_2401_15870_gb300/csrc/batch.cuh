@@ -9,15 +9,20 @@ int apply_batch_device(Graph* g, const int32_t* ds, const int32_t* dd, int64_t n
                        const int32_t* id, int64_t ni, bool validated);
 
 // the same in two phases, so that the batches of many graphs are queued before
-// the host waits for any: a small batch (at most 4096 edges) is queued by
+// the host waits for any: a small batch (at most 16384 edges) is queued by
 // apply_batch_launch and finished by apply_batch_complete (which waits for the
 // graph's stream); a larger one is applied whole by apply_batch_launch.
+struct SmallStatus;
+struct SmallBufs;
 struct SmallApply {
-  struct SmallBufs* B = nullptr;   // set while a small batch is pending
+  SmallBufs* B = nullptr;   // set while a small batch is pending
   int32_t* S[2] = {nullptr, nullptr};
-  int64_t cap[2] = {0, 0};
-  int64_t nk = 0;
 };
+// a host batch's endpoint arrays copied to the device, queued on the graph's
+// stream: *out holds nd deletion sources, nd targets, ni insertion sources, ni
+// targets
+int stage_host_batch(Graph* g, const int32_t* ds, const int32_t* dd, int64_t nd, const int32_t* is, const int32_t* id,
+                     int64_t ni, int32_t** out);
 int apply_batch_launch(Graph* g, const int32_t* ds, const int32_t* dd, int64_t nd, const int32_t* is,
                        const int32_t* id, int64_t ni, bool validated, SmallApply* pending);
 int apply_batch_complete(Graph* g, SmallApply* pending);

@@ -97,6 +97,8 @@ struct Graph {
 
   Scratch scr[8];
   void* small_h = nullptr;  // pinned host copy of the small-batch status (batch.cu)
+  void* stage_h = nullptr;  // pinned endpoint arrays of a small host batch, and whether their copy may be under way
+  bool stage_busy = false;
   std::vector<void*> allocs;
   std::string err;
 };
