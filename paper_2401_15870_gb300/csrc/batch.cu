@@ -635,9 +635,13 @@ static int edit_direction(Graph* g, Csr* c, const uint64_t* dl, int64_t nd, cons
 //   k_small_edit    one warp per touched row, staged in shared memory, or per
 //                   chunk of a longer row; both directions at once, with the
 //                   new degrees and the contributions of the sources.
-// Before, one block ran both directions in turn with the sort in shared memory
-// (53 us at 168 edges, 143 at 1300, 312 at 4000) and five kernels per direction
-// followed: 166 us of device time per batch at 2^14 vertices and 262 edges.
+// Device time of a batch: 50 us for 168 edges on a graph of 2^20 vertices, 115
+// for 4000 and 145 for 6300 on one of 2.6M (k_small_keys 4 to 8, k_small_ingest
+// 9 / 37 / 63, k_small_copy 6 to 8, k_small_edit 12 to 37).  Before, one block
+// ran both directions in turn with the sort in shared memory (53 us at 168
+// edges, 143 at 1300, 312 at 4000) and five kernels per direction followed: 166
+// us in all for 168 edges, 450 for 4000; above 4096 edges the path below, 930
+// us for 6300.
 // A direction whose rows overflow their capacity, or whose scratch is too
 // small, is left alone by the device and finished by the host.
 constexpr int SMALL_MAX = 16384;                // edges of a batch (deletions + insertions)
@@ -974,20 +978,36 @@ __device__ __forceinline__ int long_row(const int32_t* pre, int nlong, int c) {
   return lo;
 }
 
+// one warp: the first `len` (at most RW_CH) elements of src, a row position
+// that is a multiple of four, to dst, in whole quads (a row's slots are a
+// multiple of four), every load of a lane before its stores
+__device__ __forceinline__ void copy_chunk(const int32_t* src, int32_t len, int32_t* dst) {
+  const int lane = threadIdx.x & 31;
+  int4 v[RW_CH / 128];
+#pragma unroll
+  for (int k = 0; k < RW_CH / 128; k++) {
+    const int q = k * 32 + lane;
+    if (4 * q < len) v[k] = reinterpret_cast<const int4*>(src)[q];
+  }
+#pragma unroll
+  for (int k = 0; k < RW_CH / 128; k++) {
+    const int q = k * 32 + lane;
+    if (4 * q < len) reinterpret_cast<int4*>(dst)[q] = v[k];
+  }
+}
+
 __global__ void __launch_bounds__(256) k_small_copy(const __grid_constant__ SmallBufs B,
                                                     const __grid_constant__ SmallEdit p) {
   const SmallStatus& st = *B.st;
-  const int lane = threadIdx.x & 31;
   const int nw = (gridDim.x * blockDim.x) >> 5, w0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   for (int d = 0; d < 2; d++) {
     if (!((p.dirs >> d) & 1) || st.skip[d]) continue;
     const int nc = st.chunks[d];
     for (int c = w0; c < nc; c += nw) {
       const int l = long_row(B.lpre[d], st.nlong[d], c), j = B.lrow[d][l];
-      const int32_t x0 = (c - B.lpre[d][l]) * RW_CH, x1 = min(x0 + RW_CH, B.od[d][j]);
+      const int32_t x0 = (c - B.lpre[d][l]) * RW_CH;
       const int32_t* row = p.col[d] + p.off[d][B.rows[d][j]];
-      int32_t* S = p.S[d] + (int64_t)B.lpre[d][l] * RW_CH;
-      for (int32_t x = x0 + lane; x < x1; x += 32) S[x] = row[x];
+      copy_chunk(row + x0, min(B.od[d][j] - x0, RW_CH), p.S[d] + (int64_t)c * RW_CH);
     }
   }
 }
@@ -1001,12 +1021,12 @@ __device__ __forceinline__ int32_t lower_i32(const int32_t* a, int32_t lo, int32
   return lo;
 }
 
-// one warp: positions [x0, x1) of a touched row (old elements S[0..d_old), the
-// padding after them included) and its insertions [k0, k1) written to their
-// new places: a survivor x goes to x - (deletions below it) + (insertions below
+// one warp: positions [x0, x1) of a touched row (its old elements from x0 on in
+// shared memory at T, all of them at S; the padding after them included) and its
+// insertions [k0, k1) written to their new places: a survivor x goes to x - (deletions below it) + (insertions below
 // it), an insertion to its rank among the insertions + old elements below it -
 // deletions below it
-__device__ __forceinline__ void edit_row_part(const int32_t* S, int32_t x0, int32_t x1, int k0, int k1, int32_t r, int4 pl,
+__device__ __forceinline__ void edit_row_part(const int32_t* T, const int32_t* S, int32_t x0, int32_t x1, int k0, int k1, int32_t r, int4 pl,
                                               int32_t d_old, int32_t cap, const uint64_t* __restrict__ dl,
                                               const uint64_t* __restrict__ il, uint64_t mask, int bits,
                                               int32_t* __restrict__ row, int32_t sent) {
@@ -1019,7 +1039,7 @@ __device__ __forceinline__ void edit_row_part(const int32_t* S, int32_t x0, int3
   for (int32_t xb = x0; xb < x1; xb += 32) {
     const int32_t x = xb + lane;
     const bool old = x < x1 && x < d_old;
-    const int32_t v = old ? S[x] : 0;
+    const int32_t v = old ? T[x - x0] : 0;
     int dlt = 0, ilt = 0;
     bool dead = false;
     if (few) {
@@ -1050,7 +1070,7 @@ __device__ __forceinline__ void edit_row_part(const int32_t* S, int32_t x0, int3
 
 __global__ void __launch_bounds__(256) k_small_edit(const __grid_constant__ SmallBufs B,
                                                     const __grid_constant__ SmallEdit p, int bits) {
-  __shared__ int32_t stage[8][RW_CH];
+  __shared__ __align__(16) int32_t stage[8][RW_CH];
   const SmallStatus& st = *B.st;
   const int lane = threadIdx.x & 31;
   const int nw = (gridDim.x * blockDim.x) >> 5;
@@ -1073,21 +1093,18 @@ __global__ void __launch_bounds__(256) k_small_edit(const __grid_constant__ Smal
     const int64_t cap64 = p.off[d][r + 1] - base;
     const int32_t cap = (int32_t)(cap64 < INT32_MAX ? cap64 : INT32_MAX), end = (int32_t)round4(len);
     int32_t* const row = p.col[d] + base;
-    if (!chunk) {
-      if (len > RW_CH) continue;   // a long row: its chunks are items of their own
-      int32_t* const S = stage[threadIdx.x >> 5];
-      __syncwarp();
-      for (int32_t x = lane; x < d_old; x += 32) S[x] = row[x];
-      __syncwarp();
-      edit_row_part(S, 0, end, pl.z, pl.w, r, pl, d_old, cap, B.dl[d], B.il[d], mask, bits, row, p.sent);
-    } else {
-      const int part = item - B.lpre[d][l], parts = B.lpre[d][l + 1] - B.lpre[d][l];
-      const int per = (pl.w - pl.z + parts - 1) / parts;
-      const int k0 = min(pl.z + part * per, pl.w), k1 = min(k0 + per, pl.w);
-      edit_row_part(p.S[d] + (int64_t)B.lpre[d][l] * RW_CH, part * RW_CH, min((part + 1) * RW_CH, end), k0, k1, r, pl,
-                    d_old, cap, B.dl[d], B.il[d], mask, bits, row, p.sent);
-      if (part > 0) continue;
-    }
+    if (!chunk && len > RW_CH) continue;   // a long row: its chunks are items of their own
+    int32_t* const T = stage[threadIdx.x >> 5];
+    const int part = chunk ? item - B.lpre[d][l] : 0, parts = chunk ? B.lpre[d][l + 1] - B.lpre[d][l] : 1;
+    const int32_t x0 = part * RW_CH;
+    const int32_t* const S = chunk ? p.S[d] + (int64_t)B.lpre[d][l] * RW_CH : T;
+    __syncwarp();
+    copy_chunk(chunk ? S + x0 : row, min(d_old - x0, RW_CH), T);
+    __syncwarp();
+    const int per = (pl.w - pl.z + parts - 1) / parts;
+    const int k0 = min(pl.z + part * per, pl.w), k1 = min(k0 + per, pl.w);
+    edit_row_part(T, S, x0, min(x0 + RW_CH, end), k0, k1, r, pl, d_old, cap, B.dl[d], B.il[d], mask, bits, row, p.sent);
+    if (part > 0) continue;
     if (lane == 0) {
       p.deg[d][r] = d_new;
       if (d == 0 && p.R) {   // the source's contribution with its new out-degree
