@@ -120,7 +120,7 @@ __global__ void k_row_copy_out(int64_t count, const int64_t* __restrict__ base, 
 // the others.  Bound by reading r once; the block adds its threads' sums with
 // warp shuffles and makes one atomic each, because atomics of every thread on
 // one address run one after another (~1.5 ns each: 0.93 ms whatever n above
-// 600K vertices; 0.045 ms at 33.5M vertices this way).
+// 600K vertices; 0.015 ms at 2.6M and 0.077 at 33.5M this way).
 __global__ void __launch_bounds__(256) k_check_ranks(const double* __restrict__ r, int32_t n, unsigned long long* bad,
                                                      double* sum) {
   __shared__ double ws[8];
@@ -174,6 +174,7 @@ static pr_status alloc_state(pr_graph* h) {
   TRY(dalloc(g, (void**)&g->aux, sizeof(uint32_t) * words));
   TRY(dalloc(g, (void**)&g->aux2, sizeof(uint32_t) * words));
   TRY(dalloc(g, (void**)&g->anyb, sizeof(uint32_t) * words));
+  TRY(cudaMemsetAsync(g->anyb, 0, sizeof(uint32_t) * words, g->stream));
   TRY(dalloc(g, (void**)&g->xl, sizeof(int32_t) * n));
   TRY(dalloc(g, (void**)&g->rnew, sizeof(double) * n));
   TRY(dalloc(g, (void**)&g->qs, sizeof(int64_t) * (n + 1)));
@@ -190,13 +191,14 @@ static pr_status alloc_state(pr_graph* h) {
   TRY(dalloc(g, (void**)&g->tab_ab, sizeof(double2) * TAB));
   TRY(dalloc(g, (void**)&g->ctl, sizeof(Ctl)));
   TRY(cudaMemsetAsync(g->ctl, 0, sizeof(Ctl), g->stream));
-  TRY(cudaMallocHost((void**)&g->ctl_h, sizeof(Ctl)));
+  TRY(cudaMallocHost((void**)&g->ctl_h, sizeof(Ctl) * 3));   // the last one read, and two under way
   TRY(dalloc(g, (void**)&h->lbits_tmp, sizeof(int32_t) * bits_to_list_tmp(n)));
   TRY(dalloc(g, (void**)&h->ls_tmp, sizeof(int64_t) * list_scan_tmp(n)));
   TRY(dalloc(g, (void**)&h->vec_tmp, sizeof(double) * (n > 4 ? n : 4)));
   TRY(launch_tables(g->tab_sc, g->tab_ab, 0.85, g->n, g->stream));
   g->tab_alpha = 0.85;
   for (int i = 0; i < 6; i++) TRY(cudaEventCreate(&h->ev[i]));
+  for (cudaEvent_t& e : h->ev_ahead) TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   return PR_OK;
 }
 
@@ -242,6 +244,8 @@ static void destroy_handle(pr_graph* h) {
   if (g->stage_h) cudaFreeHost(g->stage_h);
   for (int i = 0; i < 6; i++)
     if (h->ev[i]) cudaEventDestroy(h->ev[i]);
+  for (cudaEvent_t e : h->ev_ahead)
+    if (e) cudaEventDestroy(e);
   for (cudaEvent_t e : h->saux.ev)
     if (e) cudaEventDestroy(e);
   if (h->saux.stream) cudaStreamDestroy(h->saux.stream);
@@ -268,7 +272,7 @@ cudaError_t dfpr::sweep_aux(pr_graph* h, const GatherCfg& c, const SweepAux** ou
 // ------------------------------------------------------------------ drivers
 
 static pr_status read_ctl(Graph* g) {
-  TRY(cudaMemcpyAsync(g->ctl_h, g->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, g->stream));
+  TRY(launch_snapshot(g->ctl, g->ctl_h, g->stream));
   TRY(cudaStreamSynchronize(g->stream));
   if (g->ctl_h->status) return (pr_status)set_error(g, ECUDA_, "device reported an inconsistent tile table");
   return PR_OK;
@@ -402,7 +406,6 @@ struct SweepTimer {
   pr_graph* h;
   bool on;
   double ms = 0.0;
-  int32_t launches = 0;
   int last_mode = 0;
   long long edges0 = 0, verts0 = 0;   // the control block's totals at the previous record
   // asynchronous order: every-vertex sweeps over ASYNC_RANGES vertex ranges in
@@ -434,7 +437,6 @@ struct SweepTimer {
       e = launch_sweep(mode, p, s);
     }
     if (on) cudaEventRecord(h->ev[5], s);
-    launches++;
     return e;
   }
   // after read_ctl: the sweep's time and, from the control block's running
@@ -456,6 +458,37 @@ struct SweepTimer {
     h->sweep_log.push_back(r);
   }
 };
+
+// Every-vertex sweeps from iteration `from` until one sets ctl->stop or max_iter
+// is reached; enqueue(it, snap) launches one with p.close set, which leaves the
+// control block at snap.  The next sweep is
+// queued before the host waits for the outcome of this one (it does nothing if
+// this one stops), so the device does not idle for the readback and the
+// launches: 25 to 35 us per iteration otherwise, against sweeps of 90 us at
+// 17M in-edges.  Timed sweeps are read back one by one.  *iters: iterations run;
+// ctl_h holds the control block after the last.
+template <class Enqueue>
+static pr_status run_sweeps(pr_graph* h, SweepTimer& timer, int32_t from, int32_t max_iter, Enqueue enqueue,
+                            int32_t* iters) {
+  Graph* g = &h->g;
+  cudaStream_t s = g->stream;
+  const int32_t ahead = timer.on ? 1 : 2;
+  int32_t q = from;
+  for (int32_t it = from; it < max_iter; it++) {
+    for (; q < max_iter && q < it + ahead; q++) {
+      pr_status st = enqueue(q, g->ctl_h + 1 + (q & 1));
+      if (st != PR_OK) return st;
+      TRY(cudaEventRecord(h->ev_ahead[q & 1], s));
+    }
+    TRY(cudaEventSynchronize(h->ev_ahead[it & 1]));
+    *g->ctl_h = g->ctl_h[1 + (it & 1)];
+    if (g->ctl_h->status) return (pr_status)set_error(g, ECUDA_, "device reported an inconsistent tile table");
+    timer.collect();
+    *iters = it + 1;
+    if (g->ctl_h->stop) break;
+  }
+  return PR_OK;
+}
 
 pr_status dfpr::run_update(pr_graph* h, int method, double alpha, double tau, double tau_f, double tau_p,
                            int32_t max_iter, int32_t flags, pr_stats* out) {
@@ -483,27 +516,34 @@ pr_status dfpr::run_update(pr_graph* h, int method, double alpha, double tau, do
   int32_t iters = 0;
   double dR = 0.0;
   bool conv = false;
+  // with the gather and the epilogue in separate launches over one range, the
+  // epilogue updates the contributions in place (the gather that reads them has
+  // finished; one buffer instead of two in L2); otherwise into the other
+  // buffer.  Asynchronous order: in place after every range, on purpose
+  const bool inplace = async || (!h->gcfg.fused && h->gcfg.parts == 1);
+  memset(g->ctl_h, 0, sizeof(Ctl));
+  // every-vertex sweeps leave anyb zero; a failed update may not have
+  TRY(cudaMemsetAsync(g->anyb, 0, sizeof(uint32_t) * (size_t)(cdiv(n, 32) + 1), s));
   if (method == PR_STATIC || method == PR_NAIVE_DYNAMIC) {
     TRY(cudaMemsetAsync(g->ctl, 0, sizeof(Ctl), s));
     if (method == PR_STATIC) TRY(launch_init_uniform(g->R, g->C[g->ccur], g->out.deg, g->tab_sc, n, s));
     p.tfirst = g->full_tfirst;
     p.ntiles_host = g->full_ntiles;
-    for (int32_t it = 0; it < max_iter; it++) {
-      p.Ccur = g->C[g->ccur];
-      p.Cnext = g->C[async ? g->ccur : 1 - g->ccur];   // one vector, updated in place, when asynchronous
+    p.close.mode = 1;
+    p.close.tau = tau;
+    const int c0 = g->ccur;
+    pr_status st = run_sweeps(h, timer, 0, max_iter, [&](int32_t it, Ctl* snap) -> pr_status {
+      p.close.snap = snap;
+      const int c = inplace ? c0 : c0 ^ (it & 1);
+      p.Ccur = g->C[c];
+      p.Cnext = g->C[inplace ? c : c ^ 1];
       TRY(timer.launch(SWEEP_FULL, p, s));
-      TRY(launch_control(g->ctl, 0, s));
-      if (!async) g->ccur ^= 1;
-      pr_status st = read_ctl(g);
-      if (st != PR_OK) return st;
-      timer.collect();
-      iters = it + 1;
-      dR = ctl_dR(g->ctl_h);
-      if (dR <= tau) {
-        conv = true;
-        break;
-      }
-    }
+      return PR_OK;
+    }, &iters);
+    if (st != PR_OK) return st;
+    if (!inplace) g->ccur = c0 ^ (iters & 1);
+    dR = iters ? ctl_dR(g->ctl_h) : 0.0;
+    conv = iters > 0 && dR <= tau;
     ever = iters > 0 ? n : 0;
   } else if (method == PR_DYNAMIC_TRAVERSAL) {
     pr_status st = dt_affected(h);
@@ -528,35 +568,34 @@ pr_status dfpr::run_update(pr_graph* h, int method, double alpha, double tau, do
       for (uint32_t* b : {g->bits[1], g->aux, g->aux2, g->ever}) TRY(cudaMemsetAsync(b, 0, wbytes, s));
       p.tau_f = HUGE_VAL;
       p.tau_p = HUGE_VAL;
-      int cur = 0;
-      for (int32_t it = 0; it < max_iter; it++) {
-        p.list = nullptr;
-        p.tfirst = g->full_tfirst;
-        p.ntiles_host = g->full_ntiles;
-        p.Ccur = g->C[g->ccur];
-        p.Cnext = g->C[1 - g->ccur];
+      p.list = nullptr;
+      p.tfirst = g->full_tfirst;
+      p.ntiles_host = g->full_ntiles;
+      p.gany = g->gany;
+      p.ever = g->ever;
+      p.cnt_x = &g->ctl->nexp;
+      p.close.mode = 2;
+      p.close.tau = tau;
+      p.close.push_below = -1.0;
+      TRY(cudaMemsetAsync(&g->ctl->stop, 0, sizeof(int32_t), s));
+      const int c0 = g->ccur;
+      st = run_sweeps(h, timer, 0, max_iter, [&](int32_t it, Ctl* snap) -> pr_status {
+        p.close.snap = snap;
+        const int cur = it & 1, c = inplace ? c0 : c0 ^ (it & 1);
+        p.Ccur = g->C[c];
+        p.Cnext = g->C[inplace ? c : c ^ 1];
         p.S_cur = g->bits[cur];
         p.X_cur = xb[cur];
         p.S_next = g->bits[1 - cur];
         p.X_next = xb[1 - cur];
-        p.gany = g->gany;
-        p.ever = g->ever;
         p.cnt_next = &g->ctl->count[1 - cur];
-        p.cnt_x = &g->ctl->nexp;
         TRY(timer.launch(SWEEP_PULL_DF, p, s));
-        TRY(launch_control(g->ctl, 1, s));
-        g->ccur ^= 1;
-        cur ^= 1;
-        st = read_ctl(g);
-        if (st != PR_OK) return st;
-        timer.collect();
-        iters = it + 1;
-        dR = ctl_dR(g->ctl_h);
-        if (dR <= tau) {
-          conv = true;
-          break;
-        }
-      }
+        return PR_OK;
+      }, &iters);
+      if (st != PR_OK) return st;
+      if (!inplace) g->ccur = c0 ^ (iters & 1);
+      dR = iters ? ctl_dR(g->ctl_h) : 0.0;
+      conv = iters > 0 && dR <= tau;
       ever = iters > 0 ? n_aff : 0;
     } else {
       p.list = g->wl[0];
@@ -602,63 +641,60 @@ pr_status dfpr::run_update(pr_graph* h, int method, double alpha, double tau, do
                          &g->ctl->ntiles, h->ls_tmp, s));
     st = read_ctl(g);
     if (st != PR_OK) return st;
-    for (int32_t it = 0; it < max_iter; it++) {
-      const bool want_pull = (flags & PR_OPT_FORCE_PULL) ||
-                             (!(flags & PR_OPT_FORCE_PUSH) && (double)(4 * g->ctl_h->qtot) > PULL_EDGE_FRACTION * (double)g->m);
-      if (!pull && want_pull) {
+    p.gany = g->gany;
+    p.ever = g->ever;
+    p.cnt_x = &g->ctl->nexp;
+    p.close.tau = tau;
+    p.close.dbar = dbar;
+    p.close.push_below = (flags & PR_OPT_FORCE_PULL) ? -1.0 : PUSH_VERTEX_FRACTION * (double)n;
+    for (int32_t it = 0; it < max_iter;) {
+      if ((flags & PR_OPT_FORCE_PULL) ||
+          (!(flags & PR_OPT_FORCE_PUSH) && (double)(4 * g->ctl_h->qtot) > PULL_EDGE_FRACTION * (double)g->m)) {
         // large frontier: sweep every vertex and test membership (F_i = S u out(X),
-        // S = bits[cur] holds F_i, X empty)
-        pull = true;
+        // S = bits[cur] holds F_i, X empty), until it converges or shrinks; the
+        // pull epilogue writes every word of S_next and X_next
         TRY(cudaMemsetAsync(xb[cur], 0, wbytes, s));
-      }
-      if (pull) {
-        // the pull epilogue writes every word of S_next and X_next
+        TRY(cudaMemsetAsync(&g->ctl->stop, 0, sizeof(int32_t), s));
         p.list = nullptr;
         p.tfirst = g->full_tfirst;
         p.ntiles_host = g->full_ntiles;
-        // with the gather and the epilogue in separate launches over one
-        // range, the epilogue updates the contributions in place (the gather
-        // that reads them has finished); otherwise into the other buffer.
-        // Asynchronous order: in place after every range, on purpose
-        const bool inplace = async || (!h->gcfg.fused && h->gcfg.parts == 1);
-        p.Ccur = g->C[g->ccur];
-        p.Cnext = g->C[inplace ? g->ccur : 1 - g->ccur];
-        p.S_cur = g->bits[cur];
-        p.X_cur = xb[cur];
-        p.S_next = g->bits[1 - cur];
-        p.X_next = xb[1 - cur];
-        p.gany = g->gany;
-        p.ever = g->ever;
-        p.cnt_next = &g->ctl->count[1 - cur];
-        p.cnt_x = &g->ctl->nexp;
-        TRY(timer.launch(pull_mode, p, s));
-        TRY(launch_control(g->ctl, 1, s));
-        if (!inplace) g->ccur ^= 1;
-        cur ^= 1;
-        st = read_ctl(g);
+        p.close.mode = 2;
+        const int c0 = g->ccur, cur0 = cur, it0 = it;
+        st = run_sweeps(h, timer, it0, max_iter, [&](int32_t k, Ctl* snap) -> pr_status {
+          p.close.snap = snap;
+          const int b = cur0 ^ ((k - it0) & 1), c = inplace ? c0 : c0 ^ ((k - it0) & 1);
+          p.Ccur = g->C[c];
+          p.Cnext = g->C[inplace ? c : c ^ 1];
+          p.S_cur = g->bits[b];
+          p.X_cur = xb[b];
+          p.S_next = g->bits[1 - b];
+          p.X_next = xb[1 - b];
+          p.cnt_next = &g->ctl->count[1 - b];
+          TRY(timer.launch(pull_mode, p, s));
+          return PR_OK;
+        }, &iters);
         if (st != PR_OK) return st;
-        timer.collect();
-        iters = it + 1;
+        cur = cur0 ^ ((iters - it0) & 1);
+        if (!inplace) g->ccur = c0 ^ ((iters - it0) & 1);
+        it = iters;
         dR = ctl_dR(g->ctl_h);
         if (dR <= tau) {
           conv = true;
           break;
         }
-        double est = (double)g->ctl_h->count[cur] + dbar * (double)g->ctl_h->nexp_last;
-        if (!(flags & PR_OPT_FORCE_PULL) && est < PUSH_VERTEX_FRACTION * (double)n) {
-          // the frontier shrank: materialise F_{i+1} = S u out(X) as a list
-          pull = false;
-          TRY(launch_bits_to_list(g->bits[cur], nullptr, n, g->wl[cur], &g->ctl->count[cur], h->lbits_tmp, s));
-          TRY(launch_bits_to_list(xb[cur], nullptr, n, g->xl, &g->ctl->nexp, h->lbits_tmp, s));
-          st = run_expand(h, g->xl, &g->ctl->nexp, g->bits[cur], nullptr, g->wl[cur], &g->ctl->count[cur], nullptr);
-          if (st != PR_OK) return st;
-          TRY(cudaMemsetAsync(&g->ctl->nexp, 0, sizeof(int32_t), s));
-          TRY(cudaMemsetAsync(g->bits[1 - cur], 0, wbytes, s));
-          TRY(launch_list_scan(g->wl[cur], &g->ctl->count[cur], g->in.deg, n, g->qs, g->tfirst, &g->ctl->qtot,
-                               &g->ctl->ntiles, h->ls_tmp, s));
-          st = read_ctl(g);
-          if (st != PR_OK) return st;
-        }
+        if (g->ctl_h->stop != 2 || it >= max_iter) break;
+        // the frontier shrank: materialise F_{i+1} = S u out(X) as a list, whose
+        // edge volume picks the form of the next sweep
+        TRY(launch_bits_to_list(g->bits[cur], nullptr, n, g->wl[cur], &g->ctl->count[cur], h->lbits_tmp, s));
+        TRY(launch_bits_to_list(xb[cur], nullptr, n, g->xl, &g->ctl->nexp, h->lbits_tmp, s));
+        st = run_expand(h, g->xl, &g->ctl->nexp, g->bits[cur], nullptr, g->wl[cur], &g->ctl->count[cur], nullptr);
+        if (st != PR_OK) return st;
+        TRY(cudaMemsetAsync(&g->ctl->nexp, 0, sizeof(int32_t), s));
+        TRY(cudaMemsetAsync(g->bits[1 - cur], 0, wbytes, s));
+        TRY(launch_list_scan(g->wl[cur], &g->ctl->count[cur], g->in.deg, n, g->qs, g->tfirst, &g->ctl->qtot,
+                             &g->ctl->ntiles, h->ls_tmp, s));
+        st = read_ctl(g);
+        if (st != PR_OK) return st;
         continue;
       }
       p.list = g->wl[cur];
@@ -686,7 +722,7 @@ pr_status dfpr::run_update(pr_graph* h, int method, double alpha, double tau, do
       st = read_ctl(g);
       if (st != PR_OK) return st;
       timer.collect();
-      iters = it + 1;
+      iters = ++it;
       dR = ctl_dR(g->ctl_h);
       if (dR <= tau) {
         conv = true;
@@ -721,7 +757,7 @@ pr_status dfpr::run_update(pr_graph* h, int method, double alpha, double tau, do
     out->ms_apply = h->ms_apply;
     out->ms_update = ms;
     out->ms_sweep = timer.ms;
-    out->sweeps = timer.launches;
+    out->sweeps = iters;
     out->reserved = 0;
   }
   return PR_OK;
@@ -1155,7 +1191,7 @@ pr_status pr_ranks(const pr_graph* hc, double* out) {
 static pr_status set_ranks_from_device(pr_graph* h, const double* dev) {
   Graph* g = &h->g;
   cudaStream_t s = g->stream;
-  TRY(launch_import_ranks(dev, g->iperm, g->R, g->C[g->ccur], g->out.deg, g->tab_sc, g->n, s));
+  TRY(launch_import_ranks(dev, g->perm, g->iperm, g->R, g->C[g->ccur], g->out.deg, g->tab_sc, g->n, s));
   TRY(cudaStreamSynchronize(s));
   g->has_ranks = true;
   return PR_OK;

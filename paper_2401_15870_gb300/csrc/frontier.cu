@@ -192,6 +192,19 @@ cudaError_t launch_control(Ctl* ctl, int frontier, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// the control block written to the host's pinned copy by a kernel: the copy
+// engine takes about 10 us to take over from the kernel before it
+__global__ void k_snapshot(const Ctl* ctl, Ctl* host) {
+  const int i = threadIdx.x;
+  if (i < (int)(sizeof(Ctl) / 8))
+    reinterpret_cast<volatile unsigned long long*>(host)[i] = reinterpret_cast<const volatile unsigned long long*>(ctl)[i];
+}
+
+cudaError_t launch_snapshot(const Ctl* ctl, Ctl* host, cudaStream_t s) {
+  note_launch(); k_snapshot<<<1, 32, 0, s>>>(ctl, host);
+  return cudaGetLastError();
+}
+
 __global__ void k_tables(double* tab_sc, double2* tab_ab, double alpha, int32_t n) {
   GRID_STRIDE(d, TAB) {
     if (d == 0) {
@@ -259,28 +272,54 @@ __global__ void k_gather_f64(const double* __restrict__ in, const int32_t* __res
                              int32_t n) {
   GRID_STRIDE(i, n) out[i] = in[idx[i]];
 }
-// ranks given in the caller's order: rank and contribution of every vertex in
-// one pass.  Read through iperm (the random side is the 8-byte load; R and C
-// are written in order) instead of scattering R through perm and reading it
-// back for C: two passes over R and the scattered stores went, 0.37 -> 0.19 ms
-// at 33.5M vertices.
+// Ranks given in the caller's order: rank and contribution of every vertex in
+// one pass, read through iperm (the random side is an 8-byte load; R and C are
+// written in order).  Bound by the sectors of those loads: 28 us at 2.6M
+// vertices, 90 at 8.4M.  Once the vectors are larger than L2 a loaded sector is
+// gone before its other ranks are wanted, and scattering R through perm first
+// is the faster way: 374 against 413 us at 33.5M.
 __global__ void k_import_ranks(const double* __restrict__ in, const int32_t* __restrict__ iperm, double* __restrict__ R,
                                long long* __restrict__ C, const int32_t* __restrict__ odeg,
                                const double* __restrict__ tab_sc, int32_t n) {
-  GRID_STRIDE(v, n) {
-    const double r = in[iperm[v]];
-    R[v] = r;
-    C[v] = contrib_of(r, odeg[v], tab_sc);
+  constexpr int U = 4;   // vertices per thread whose chain of loads is in flight together
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t v0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v0 < n; v0 += U * stride) {
+    double r[U];
+    int32_t d[U];
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const int64_t v = v0 + u * stride;
+      r[u] = v < n ? in[iperm[v]] : 0.0;
+      d[u] = v < n ? odeg[v] : 1;
+    }
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const int64_t v = v0 + u * stride;
+      if (v >= n) break;
+      R[v] = r[u];
+      C[v] = contrib_of(r[u], d[u], tab_sc);
+    }
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) C[n] = 0;
+}
+
+__global__ void k_scatter_f64(const double* __restrict__ in, const int32_t* __restrict__ idx, double* __restrict__ out,
+                              int32_t n) {
+  GRID_STRIDE(i, n) out[idx[i]] = in[i];
 }
 
 cudaError_t launch_gather_f64(const double* in, const int32_t* idx, double* out, int32_t n, cudaStream_t s) {
   note_launch(); k_gather_f64<<<grid_for(n, 256), 256, 0, s>>>(in, idx, out, n);
   return cudaGetLastError();
 }
-cudaError_t launch_import_ranks(const double* in, const int32_t* iperm, double* R, long long* C, const int32_t* odeg,
-                                const double* tab_sc, int32_t n, cudaStream_t s) {
+constexpr int32_t IMPORT_SCATTER_N = 1 << 24;   // 134 MB per vector, against an L2 of 126 MB
+
+cudaError_t launch_import_ranks(const double* in, const int32_t* perm, const int32_t* iperm, double* R, long long* C,
+                                const int32_t* odeg, const double* tab_sc, int32_t n, cudaStream_t s) {
+  if (n > IMPORT_SCATTER_N) {
+    note_launch(); k_scatter_f64<<<grid_for(n, 256), 256, 0, s>>>(in, perm, R, n);
+    return launch_contrib_all(R, C, odeg, tab_sc, n, s);
+  }
   note_launch(); k_import_ranks<<<grid_for(n, 256), 256, 0, s>>>(in, iperm, R, C, odeg, tab_sc, n);
   return cudaGetLastError();
 }

@@ -28,6 +28,9 @@ cudaError_t launch_bits_or(const uint32_t* a, const uint32_t* b, uint32_t* out, 
 // end-of-iteration bookkeeping (one thread); frontier != 0 swaps the worklists
 cudaError_t launch_control(Ctl* ctl, int frontier, cudaStream_t s);
 
+// the control block to pinned host memory
+cudaError_t launch_snapshot(const Ctl* ctl, Ctl* host, cudaStream_t s);
+
 // tables for d in [1, TAB): tab_sc[d] = 2^61 / d and, unless tab_ab is NULL,
 // tab_ab[d] = closed_coeffs(alpha, n, d) (the coefficients of Eq. 2 as one FMA)
 cudaError_t launch_tables(double* tab_sc, double2* tab_ab, double alpha, int32_t n, cudaStream_t s);
@@ -43,8 +46,8 @@ cudaError_t launch_contrib_list(const int32_t* list, const int32_t* count, const
 
 // a vector from internal to user order, and ranks from user to internal order
 cudaError_t launch_gather_f64(const double* in, const int32_t* idx, double* out, int32_t n, cudaStream_t s);
-// R[v] = in[iperm[v]] and C[v] from it for all v (C[n] = 0)
-cudaError_t launch_import_ranks(const double* in, const int32_t* iperm, double* R, long long* C, const int32_t* odeg,
-                                const double* tab_sc, int32_t n, cudaStream_t s);
+// R[v] = in[iperm[v]] and C[v] from it for all v (C[n] = 0); perm the inverse of iperm
+cudaError_t launch_import_ranks(const double* in, const int32_t* perm, const int32_t* iperm, double* R, long long* C,
+                                const int32_t* odeg, const double* tab_sc, int32_t n, cudaStream_t s);
 
 }  // namespace dfpr

@@ -16,7 +16,7 @@ struct Csr {
 };
 
 // Per-iteration control block, device resident; the host reads a copy.
-struct Ctl {
+struct alignas(8) Ctl {
   int32_t count[2];             // worklist sizes
   int32_t nexp;                 // expander list size
   int32_t cur;                  // current worklist / bitset index
@@ -31,7 +31,8 @@ struct Ctl {
   int64_t verts;                // vertices processed (all iterations)
   int32_t status;               // device-detected error (0 = none)
   int32_t nexp_last;            // expander count of the last finished iteration
-  int32_t nbig;                 // rows deferred to the long-row pass of a full sweep
+  int32_t stop;                 // every-vertex sweeps: 1 the iteration converged, 2 it left a small frontier; sweeps
+                                // queued behind it return at once
   int32_t pad;
 };
 

@@ -9,6 +9,7 @@
 struct pr_graph {
   dfpr::Graph g;
   cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+  cudaEvent_t ev_ahead[2] = {nullptr, nullptr};   // control-block copies of sweeps queued ahead (run_sweeps)
   double ms_apply = 0.0;
   int32_t* lbits_tmp = nullptr;   // bits_to_list scratch
   int64_t* ls_tmp = nullptr;      // list scan scratch

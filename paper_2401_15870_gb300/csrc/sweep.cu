@@ -83,6 +83,50 @@ __device__ __forceinline__ void block_flush_stats(double dmax, long long edges, 
   }
 }
 
+// ------------------------------------------------------------------ closing an iteration
+
+// (an ordinary load: the flag is set by an earlier launch, and warp after warp
+// reading one address past L1 would queue at its L2 slice)
+__device__ __forceinline__ bool stopped(const SweepParams& p) { return p.close.mode && p.ctl->stop; }
+
+// One warp: the control block is read whole, a word per lane, changed and
+// written back to the device and to the host's pinned copy (a copy engine
+// between two sweeps costs the stream about 10 us, this kernel 2).  In the
+// epilogue's last block instead (fence, ticket) it cost the epilogue more:
+// 110 against 93 us per sweep at 8.4M vertices.
+__global__ void __launch_bounds__(32, 1) k_close(Ctl* ctl, SweepClose c) {
+  constexpr int W = sizeof(Ctl) / 8;
+  static_assert(sizeof(Ctl) % 8 == 0 && W <= 32, "a word per lane");
+  __shared__ unsigned long long w[W];
+  const int lane = threadIdx.x;
+  unsigned long long* const m = reinterpret_cast<unsigned long long*>(ctl);
+  if (lane < W) w[lane] = m[lane];
+  __syncwarp();
+  Ctl& v = *reinterpret_cast<Ctl*>(w);
+  if (v.stop) return;
+  __syncwarp();
+  if (lane == 0) {
+    v.dR_last = v.dR;
+    v.dR = 0ull;
+    v.iter += 1;
+    v.stop = __longlong_as_double((long long)v.dR_last) <= c.tau ? 1 : 0;
+    if (c.mode == 2) {
+      const int cur = v.cur;
+      v.count[cur] = 0;
+      v.cur = 1 - cur;
+      v.nexp_last = v.nexp;
+      v.nexp = 0;
+      if (!v.stop && c.push_below >= 0.0 && (double)v.count[1 - cur] + c.dbar * (double)v.nexp_last < c.push_below)
+        v.stop = 2;
+    }
+  }
+  __syncwarp();
+  if (lane < W) {
+    m[lane] = w[lane];
+    reinterpret_cast<volatile unsigned long long*>(c.snap)[lane] = w[lane];
+  }
+}
+
 // ------------------------------------------------------------------ tiles
 
 // Shared-memory view of one tile: for every item (list entry) touching the
@@ -364,8 +408,9 @@ __global__ void __launch_bounds__(1024, QPT == 2 ? 2 : 1) k_gather_rows(const in
                                                       const int32_t* __restrict__ rowbase, int64_t nquads, int32_t sent,
                                                       long long* __restrict__ acc, uint32_t* __restrict__ anyb,
                                                       int32_t hub_k, int32_t hub_kx, const int64_t* __restrict__ ioff,
-                                                      int32_t v_lo, int32_t v_hi) {
+                                                      int32_t v_lo, int32_t v_hi, const int32_t* stop) {
   extern __shared__ __align__(16) unsigned char hub_smem[];
+  if (stop && *stop) return;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const uint64_t pol_stream = policy_evict_first();
@@ -397,6 +442,7 @@ __global__ void __launch_bounds__(1024, QPT == 2 ? 2 : 1) k_gather_rows(const in
 template <bool CLOSED, bool REL, bool SAME = false>
 __global__ void __launch_bounds__(256, 3) k_finish_pull(SweepParams p, long long* __restrict__ acc,
                                                         uint32_t* __restrict__ anyb, int64_t ch_lo, int64_t ch_hi) {
+  if (stopped(p)) return;
   const int lane = threadIdx.x & 31;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   PullTotals t;
@@ -415,6 +461,7 @@ __global__ void __launch_bounds__(256, 3) k_finish_pull(SweepParams p, long long
 // (vertices [v_lo, v_hi))
 __global__ void __launch_bounds__(256, 4) k_finish_full(SweepParams p, long long* __restrict__ acc, int64_t v_lo,
                                                         int64_t v_hi) {
+  if (stopped(p)) return;
   constexpr int U = 4;
   const double alpha_fix = p.alpha * FIX_INV;
   unsigned long long dmax = 0ull;
@@ -538,6 +585,7 @@ template <int MODE, int QPT, bool HUB>
 __global__ void __launch_bounds__(1024) k_sweep_rows(SweepParams p, const uint32_t* __restrict__ rowbits,
                                                      const int32_t* __restrict__ rowbase, uint32_t* __restrict__ anyb,
                                                      int32_t* __restrict__ done, int32_t hub_k, int32_t hub_kx) {
+  if (stopped(p)) return;
   constexpr bool PULL = MODE != SWEEP_FULL;
   constexpr int64_t UQ = 32 * QPT;          // quads per gather step
   constexpr int CV = FIN_U * 32;            // vertices per epilogue chunk
@@ -671,7 +719,8 @@ static cudaError_t gather_launch(const SweepParams& p, const uint32_t* rowbits, 
   note_launch();
   k_gather_rows<PULL, QPT, HUB><<<grid, threads, smem, s>>>(p.icol, p.Ccur, PULL ? p.X_cur : nullptr,
                                                           PULL ? p.S_cur : nullptr, rowbits, rowbase, nquads, p.n,
-                                                          p.gacc, anyb, hub_k, hub_kx, p.ioff, v_lo, v_hi);
+                                                          p.gacc, anyb, hub_k, hub_kx, p.ioff, v_lo, v_hi,
+                                                          p.close.mode ? &p.ctl->stop : nullptr);
   return cudaGetLastError();
 }
 
@@ -790,23 +839,28 @@ cudaError_t async_range_bounds(const int32_t* ideg, int32_t n, int P, int64_t* s
   return cudaGetLastError();
 }
 
+static cudaError_t launch_close(const SweepParams& p, cudaStream_t s) {
+  if (!p.close.mode) return cudaSuccess;
+  note_launch();
+  k_close<<<1, 32, 0, s>>>(p.ctl, p.close);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_full_sweep(int mode, const SweepParams& p, const GatherCfg& cfg, const uint32_t* rowbits,
                               const int32_t* rowbase, uint32_t* anyb, int32_t* done, const SweepAux* aux,
                               cudaStream_t s, bool ordered, const int32_t* bounds) {
   const int64_t nquads = p.ntiles_host;   // quads of the in-CSR capacity
   const bool pull = mode == SWEEP_PULL_DF || mode == SWEEP_PULL_DFP;
-  if (pull) {
-    cudaError_t e = cudaMemsetAsync(anyb, 0, sizeof(uint32_t) * (size_t)(cdiv(p.n, 32) + 1), s);
-    if (e != cudaSuccess) return e;
-  }
   if (cfg.fused && !ordered) {
     if (!gather_cfg_valid(cfg)) return cudaErrorInvalidValue;
+    cudaError_t e;
     switch (mode) {
-      case SWEEP_FULL: return sweep_rows_dispatch<SWEEP_FULL>(p, cfg, rowbits, rowbase, anyb, done, s);
-      case SWEEP_PULL_DF: return sweep_rows_dispatch<SWEEP_PULL_DF>(p, cfg, rowbits, rowbase, anyb, done, s);
-      case SWEEP_PULL_DFP: return sweep_rows_dispatch<SWEEP_PULL_DFP>(p, cfg, rowbits, rowbase, anyb, done, s);
+      case SWEEP_FULL: e = sweep_rows_dispatch<SWEEP_FULL>(p, cfg, rowbits, rowbase, anyb, done, s); break;
+      case SWEEP_PULL_DF: e = sweep_rows_dispatch<SWEEP_PULL_DF>(p, cfg, rowbits, rowbase, anyb, done, s); break;
+      case SWEEP_PULL_DFP: e = sweep_rows_dispatch<SWEEP_PULL_DFP>(p, cfg, rowbits, rowbase, anyb, done, s); break;
       default: return cudaErrorInvalidValue;
     }
+    return e == cudaSuccess ? launch_close(p, s) : e;
   }
   if (!ordered && !gather_cfg_valid(cfg)) return cudaErrorInvalidValue;
   // P vertex ranges cut at multiples of 128: the gather of range k + 1 runs on
@@ -868,7 +922,8 @@ cudaError_t launch_full_sweep(int mode, const SweepParams& p, const GatherCfg& c
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, aux->ev[P], 0);
     if (e != cudaSuccess) return e;
   }
-  return cudaGetLastError();
+  const cudaError_t ec = launch_close(p, s);
+  return ec != cudaSuccess ? ec : cudaGetLastError();
 }
 
 // bitmap of the quads where an in-CSR row starts, and per 32-quad word the

@@ -46,6 +46,18 @@ __device__ __forceinline__ double2 closed_coeffs(double alpha, int32_t n, int32_
   return make_double2(f * (alpha * FIX_INV), f * C0);
 }
 
+// How an every-vertex sweep closes its iteration: a last small kernel moves the
+// L-inf change and the frontier counts on (as launch_control does) and sets
+// ctl->stop, so that the host can queue the next sweep before it has seen this
+// one's outcome (a sweep queued behind a stop does nothing).
+struct SweepClose {
+  int32_t mode;        // 0: not closed here, 1: Static / ND, 2: with a frontier
+  double tau;          // stop = 1 when the change is at most tau
+  double dbar;         // mean degree, and the frontier size below which a pull
+  double push_below;   // sweep hands over to lists (stop = 2; negative: never)
+  Ctl* snap;           // pinned host copy of the control block, written by the device
+};
+
 struct SweepParams {
   int32_t n;
   const int64_t* ioff;
@@ -90,6 +102,7 @@ struct SweepParams {
   uint32_t* X_next;
   int32_t* gany;             // per split item: an in-neighbour expanded (n)
   Ctl* ctl;
+  SweepClose close;
 };
 
 cudaError_t launch_sweep(int mode, const SweepParams& p, cudaStream_t s);
@@ -127,8 +140,9 @@ cudaError_t launch_gather(bool pull, const SweepParams& p, const GatherCfg& cfg,
 // every-vertex sweep (FULL, PULL_DF, PULL_DFP); p.ntiles_host is the number of
 // quads of the in-CSR capacity, p.gacc the all-zero per-vertex accumulators
 // (left zero), rowbits / rowbase the row-start index of the in-CSR
-// (launch_row_start_index), anyb an n-bit scratch bitset, done the all-zero
-// per-chunk unit counts of the one-launch form (cdiv(n, 128) int32, left zero)
+// (launch_row_start_index), anyb an all-zero n-bit bitset (left zero), done the
+// all-zero per-chunk unit counts of the one-launch form (cdiv(n, 128) int32,
+// left zero)
 // aux: the second stream of a sweep in several ranges (NULL: one range)
 // ordered: the asynchronous order -- the cfg.parts vertex ranges are swept one
 // after another on s, each gather followed by its epilogue, and the epilogue
@@ -136,6 +150,7 @@ cudaError_t launch_gather(bool pull, const SweepParams& p, const GatherCfg& cfg,
 // gathers the contributions of the ranges before it as updated in this sweep
 // bounds (ordered only): the P + 1 range bounds on the host (P = cfg.parts;
 // async_range_bounds below)
+// p.close: the iteration is closed after the sweep
 cudaError_t launch_full_sweep(int mode, const SweepParams& p, const GatherCfg& cfg, const uint32_t* rowbits,
                               const int32_t* rowbase, uint32_t* anyb, int32_t* done, const SweepAux* aux,
                               cudaStream_t s, bool ordered = false, const int32_t* bounds = nullptr);
