@@ -521,6 +521,8 @@ pr_status dfpr::run_update(pr_graph* h, int method, double alpha, double tau, do
   // finished; one buffer instead of two in L2); otherwise into the other
   // buffer.  Asynchronous order: in place after every range, on purpose
   const bool inplace = async || (!h->gcfg.fused && h->gcfg.parts == 1);
+  // the one-launch form has no variant without X: it gets an empty one
+  const bool with_x = h->gcfg.fused && !async;
   memset(g->ctl_h, 0, sizeof(Ctl));
   // every-vertex sweeps leave anyb zero; a failed update may not have
   TRY(cudaMemsetAsync(g->anyb, 0, sizeof(uint32_t) * (size_t)(cdiv(n, 32) + 1), s));
@@ -585,7 +587,7 @@ pr_status dfpr::run_update(pr_graph* h, int method, double alpha, double tau, do
         p.Ccur = g->C[c];
         p.Cnext = g->C[inplace ? c : c ^ 1];
         p.S_cur = g->bits[cur];
-        p.X_cur = xb[cur];
+        p.X_cur = with_x ? xb[cur] : nullptr;   // nothing expands
         p.S_next = g->bits[1 - cur];
         p.X_next = xb[1 - cur];
         p.cnt_next = &g->ctl->count[1 - cur];
@@ -651,9 +653,9 @@ pr_status dfpr::run_update(pr_graph* h, int method, double alpha, double tau, do
       if ((flags & PR_OPT_FORCE_PULL) ||
           (!(flags & PR_OPT_FORCE_PUSH) && (double)(4 * g->ctl_h->qtot) > PULL_EDGE_FRACTION * (double)g->m)) {
         // large frontier: sweep every vertex and test membership (F_i = S u out(X),
-        // S = bits[cur] holds F_i, X empty), until it converges or shrinks; the
-        // pull epilogue writes every word of S_next and X_next
-        TRY(cudaMemsetAsync(xb[cur], 0, wbytes, s));
+        // S = bits[cur] holds F_i, X empty at first), until it converges or
+        // shrinks; the pull epilogue writes every word of S_next and X_next
+        if (with_x) TRY(cudaMemsetAsync(xb[cur], 0, wbytes, s));
         TRY(cudaMemsetAsync(&g->ctl->stop, 0, sizeof(int32_t), s));
         p.list = nullptr;
         p.tfirst = g->full_tfirst;
@@ -666,7 +668,7 @@ pr_status dfpr::run_update(pr_graph* h, int method, double alpha, double tau, do
           p.Ccur = g->C[c];
           p.Cnext = g->C[inplace ? c : c ^ 1];
           p.S_cur = g->bits[b];
-          p.X_cur = xb[b];
+          p.X_cur = k > it0 || with_x ? xb[b] : nullptr;
           p.S_next = g->bits[1 - b];
           p.X_next = xb[1 - b];
           p.cnt_next = &g->ctl->count[1 - b];

@@ -138,7 +138,13 @@ struct GatherSpan {
 // COH: the contributions and the S / X words were written earlier in the same
 // launch (a kernel that runs the whole iteration loop): they are read with
 // ordinary loads, not through the read-only path
-template <bool PULL, int QPT = SW_QPT, bool HUB = false, bool SPAN = false, bool COH = false>
+// NOX: no vertex expanded before this sweep, so the frontier is S alone (pull
+// form): a row outside it is not processed, and neither its sum nor its sources'
+// bits are loaded.  The loads then wait for the S word, which costs sweeps whose
+// frontier holds nearly every edge about as much as it saves them (0.161 against
+// 0.163 ms at 97% of 34M edges) and halves one that holds 46% of 1.08e9 (4.36 ->
+// 2.37 ms).
+template <bool PULL, int QPT = SW_QPT, bool HUB = false, bool SPAN = false, bool COH = false, bool NOX = false>
 __device__ __forceinline__ GatherSpan gather_step(const int32_t* __restrict__ icol, const long long* __restrict__ C,
                                                   const uint32_t* __restrict__ X, const uint32_t* __restrict__ S,
                                                   const uint32_t* __restrict__ rowbits,
@@ -205,12 +211,15 @@ __device__ __forceinline__ GatherSpan gather_step(const int32_t* __restrict__ ic
   unsigned x[QPT];
 #pragma unroll
   for (int j = 0; j < QPT; j++) {
-    s[j] = contrib(c[j].x) + contrib(c[j].y) + contrib(c[j].z) + contrib(c[j].w);
-    x[j] = 0;
     // a row whose vertex stays in the frontier is processed anyway: its
     // sources' expanded bits are not needed
-    if (PULL && owner[j] >= 0 &&
-        !(((COH ? ld_weak(S + (owner[j] >> 5)) : __ldg(S + (owner[j] >> 5))) >> (owner[j] & 31)) & 1u))
+    x[j] = 0u;
+    const auto stays = [&] {
+      return ((COH ? ld_weak(S + (owner[j] >> 5)) : __ldg(S + (owner[j] >> 5))) >> (owner[j] & 31)) & 1u;
+    };
+    if (NOX && (owner[j] < 0 || !stays())) c[j] = make_int4(sent, sent, sent, sent);
+    s[j] = contrib(c[j].x) + contrib(c[j].y) + contrib(c[j].z) + contrib(c[j].w);
+    if (PULL && !NOX && owner[j] >= 0 && !stays())
       x[j] = (expanded(c[j].x) | expanded(c[j].y) | expanded(c[j].z) | expanded(c[j].w)) & 1u;
   }
   GatherSpan span{0, 0, false};
@@ -231,24 +240,23 @@ __device__ __forceinline__ GatherSpan gather_step(const int32_t* __restrict__ ic
     const int own = owner[j];
     long long sum = s[j];
     // segment starts: lane 0, the row starts, and where the valid quads
-    // ([qlo, nquads), owner >= 0) begin and end
+    // ([qlo, nquads), owner >= 0) begin and end; this lane's row piece ends
+    // before lane `end`
     const unsigned vm = __ballot_sync(0xffffffffu, own >= 0);
-    const unsigned long long st = (unsigned long long)(wb[j] | 1u | (vm ^ (vm << 1)));
+    const unsigned st = wb[j] | 1u | (vm ^ (vm << 1));
+    const unsigned later = st & ~upto;
+    const int end = later ? __ffs(later) - 1 : 32;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const long long os = __shfl_down_sync(0xffffffffu, sum, o);
-      // lane + o holds the same row piece when no segment starts in (lane, lane + o]
-      if (lane + o < 32 && ((st >> (lane + 1)) & ((1ull << o) - 1ull)) == 0) sum += os;
+      if (lane + o < end) sum += os;
     }
     unsigned any = 0u;
-    if (PULL) {
+    if (PULL && !NOX) {
       const unsigned xm = __ballot_sync(0xffffffffu, x[j] != 0u);
-      const unsigned long long later = (st >> (lane + 1)) << (lane + 1);   // starts after this lane
-      const int end = later ? __ffsll((long long)later) - 1 : 32;         // this lane's segment ends before it
-      const unsigned seg = (unsigned)(((1ull << end) - 1ull) & ~((1ull << lane) - 1ull));
-      any = (xm & seg) != 0u;
+      any = xm & (unsigned)((1ull << end) - (1ull << lane));
     }
-    if (own >= 0 && ((st >> lane) & 1ull)) {
+    if (own >= 0 && ((st >> lane) & 1u)) {
       if (sum) atomicAdd(reinterpret_cast<unsigned long long*>(acc + own), (unsigned long long)sum);
       if (PULL && any) atomicOr(anyb + (own >> 5), 1u << (own & 31));
       if (SPAN) span.wrote = span.wrote || sum != 0 || (PULL && any);

@@ -401,7 +401,8 @@ __global__ void __launch_bounds__(SW_THREADS) k_sweep(SweepParams p) {
 //   shared memory; the grid is then one wave of resident blocks, so the
 //   staging is paid once per block and sweep.
 // (2 quads per lane: held to 32 registers, two 1024-thread blocks per SM)
-template <bool PULL, int QPT, bool HUB>
+// (PULL without X: no vertex expanded, see gather_step's NOX)
+template <bool PULL, int QPT, bool HUB, bool NOX>
 __global__ void __launch_bounds__(1024, QPT == 2 ? 2 : 1) k_gather_rows(const int32_t* __restrict__ icol, const long long* __restrict__ C,
                                                       const uint32_t* __restrict__ X, const uint32_t* __restrict__ S,
                                                       const uint32_t* __restrict__ rowbits,
@@ -434,8 +435,8 @@ __global__ void __launch_bounds__(1024, QPT == 2 ? 2 : 1) k_gather_rows(const in
   const int64_t qhi = v_hi < sent ? __ldg(ioff + v_hi) >> 2 : nquads;
   const int64_t q0 = qlo / (32 * QPT) * (32 * QPT);
   for (int64_t base = q0 + warp * 32 * QPT; base < qhi; base += nw * 32 * QPT)
-    gather_step<PULL, QPT, HUB>(icol, C, X, S, rowbits, rowbase, qhi, sent, acc, anyb, base, pol_stream, pol_keep,
-                                hub, qlo);
+    gather_step<PULL, QPT, HUB, false, false, NOX>(icol, C, X, S, rowbits, rowbase, qhi, sent, acc, anyb, base, pol_stream,
+                                                   pol_keep, hub, qlo);
 }
 
 // (the 32-vertex chunks [ch_lo, ch_hi); ch_lo a multiple of FIN_U)
@@ -684,7 +685,7 @@ static cudaError_t sweep_rows_dispatch(const SweepParams& p, const GatherCfg& cf
                                        const int32_t* rowbase, uint32_t* anyb, int32_t* done, cudaStream_t s) {
   constexpr bool PULL = MODE != SWEEP_FULL;
   const int32_t hub_k = std::min<int32_t>(cfg.hub, p.n + 1);
-  const int32_t hub_kx = PULL ? (int32_t)cdiv(std::min<int32_t>(hub_k, p.n), 32) : 0;
+  const int32_t hub_kx = PULL && p.X_cur ? (int32_t)cdiv(std::min<int32_t>(hub_k, p.n), 32) : 0;
   const int t = cfg.threads;
   switch (cfg.qpt * 2 + (hub_k > 0 ? 1 : 0)) {
     case 4: return sweep_rows_launch<MODE, 2, false>(p, rowbits, rowbase, anyb, done, t, 0, 0, s);
@@ -701,7 +702,8 @@ template <bool PULL, int QPT, bool HUB>
 static cudaError_t gather_launch(const SweepParams& p, const uint32_t* rowbits, const int32_t* rowbase, uint32_t* anyb,
                                  int64_t nquads, int threads, int32_t hub_k, int32_t hub_kx, int32_t v_lo, int32_t v_hi,
                                  bool one_wave, cudaStream_t s) {
-  const void* fn = (const void*)k_gather_rows<PULL, QPT, HUB>;
+  const auto kernel = PULL && !p.X_cur ? k_gather_rows<PULL, QPT, HUB, PULL> : k_gather_rows<PULL, QPT, HUB, false>;
+  const void* fn = (const void*)kernel;
   const size_t smem = HUB ? gather_hub_bytes(hub_k, hub_kx) : 0;
   int bps = 1;
   cudaError_t e = gather_occupancy(fn, threads, smem, &bps);
@@ -717,10 +719,9 @@ static cudaError_t gather_launch(const SweepParams& p, const uint32_t* rowbits, 
   const int64_t cap = HUB || one_wave ? (int64_t)num_sms() * bps : (int64_t)num_sms() * 64 * 256 / threads;
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(cdiv(units, threads / 32), cap));
   note_launch();
-  k_gather_rows<PULL, QPT, HUB><<<grid, threads, smem, s>>>(p.icol, p.Ccur, PULL ? p.X_cur : nullptr,
-                                                          PULL ? p.S_cur : nullptr, rowbits, rowbase, nquads, p.n,
-                                                          p.gacc, anyb, hub_k, hub_kx, p.ioff, v_lo, v_hi,
-                                                          p.close.mode ? &p.ctl->stop : nullptr);
+  kernel<<<grid, threads, smem, s>>>(p.icol, p.Ccur, PULL ? p.X_cur : nullptr, PULL ? p.S_cur : nullptr, rowbits,
+                                     rowbase, nquads, p.n, p.gacc, anyb, hub_k, hub_kx, p.ioff, v_lo, v_hi,
+                                     p.close.mode ? &p.ctl->stop : nullptr);
   return cudaGetLastError();
 }
 
@@ -730,7 +731,7 @@ static cudaError_t gather_dispatch(const SweepParams& p, const GatherCfg& cfg, c
                                    cudaStream_t s) {
   const bool ow = cfg.parts > 1;
   const int32_t hub_k = std::min<int32_t>(cfg.hub, p.n + 1);
-  const int32_t hub_kx = PULL ? (int32_t)cdiv(std::min<int32_t>(hub_k, p.n), 32) : 0;
+  const int32_t hub_kx = PULL && p.X_cur ? (int32_t)cdiv(std::min<int32_t>(hub_k, p.n), 32) : 0;
   const bool hub = hub_k > 0;
   const int t = cfg.threads;
   switch (cfg.qpt * 2 + (hub ? 1 : 0)) {

@@ -95,7 +95,7 @@ struct SweepParams {
   int32_t* cnt_x;
   // pull form of the frontier (PULL_*): F_i = S_cur u out(X_cur); the sweep
   // writes S_next (vertices that stay) and X_next (vertices that expand) and
-  // counts them in *cnt_next / *cnt_x
+  // counts them in *cnt_next / *cnt_x.  X_cur null: nothing expanded, F_i = S_cur
   const uint32_t* S_cur;
   const uint32_t* X_cur;
   uint32_t* S_next;
