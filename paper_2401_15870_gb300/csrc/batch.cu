@@ -8,12 +8,11 @@
 //
 // Steps: packed keys -> radix sort -> first occurrences -> effective flags by
 // binary search in the sorted rows -> compaction (Delta-, Delta+ sorted by
-// (src, dst)).  Each touched row is rewritten by one warp: the old row is
-// copied to scratch, every surviving element and every insertion computes its
-// output position by counting smaller deletions / insertions / old elements,
-// and is written back in place; padding slots get the sentinel.  A row whose
-// new degree exceeds its capacity triggers a repack of that direction (a full
-// rebuild with fresh slack).
+// (src, dst)) -> the same sorted by (dst, src) -> touched rows with their edit
+// plans -> the rows rewritten in place, padding slots set to the sentinel.  A
+// batch of at most SMALL_MAX edges does the steps up to the plans in two
+// kernels.  A row whose new degree exceeds its capacity triggers a repack of
+// that direction (a full rebuild with fresh slack).
 #include <algorithm>
 #include <climits>
 #include <cstring>
@@ -130,150 +129,6 @@ __global__ void k_flag_ins(const uint64_t* __restrict__ ik, int64_t ni, const in
 __global__ void k_swap_keys(const uint64_t* __restrict__ in, int64_t k, int bits, uint64_t* __restrict__ out) {
   uint64_t mask = (1ull << bits) - 1;
   GRID_STRIDE(i, k) out[i] = ((in[i] & mask) << bits) | (in[i] >> bits);
-}
-
-__global__ void k_row_keys(const uint64_t* __restrict__ a, int64_t na, const uint64_t* __restrict__ b, int64_t nb,
-                           int bits, uint64_t* __restrict__ out) {
-  GRID_STRIDE(i, na + nb) out[i] = (i < na ? a[i] : b[i - na]) >> bits;
-}
-
-// per touched row: ranges in the deletion / insertion lists, old degree,
-// chunk counts of the copy and write passes, overflow
-constexpr int RW_CH = 1024;   // row elements per chunk (one warp works on a chunk)
-
-__global__ void k_row_plan(const uint64_t* __restrict__ rows, int64_t nr, const uint64_t* __restrict__ dl, int64_t nd,
-                           const uint64_t* __restrict__ il, int64_t ni, int bits, const int64_t* __restrict__ off,
-                           const int32_t* __restrict__ deg, int64_t* __restrict__ plan, int64_t* __restrict__ olddeg,
-                           int64_t* __restrict__ cchunks, int64_t* __restrict__ wchunks, unsigned long long* overflow) {
-  GRID_STRIDE(j, nr) {
-    uint64_t r = rows[j];
-    int64_t d0 = lower_key(dl, 0, nd, r << bits), d1 = lower_key(dl, d0, nd, (r + 1) << bits);
-    int64_t i0 = lower_key(il, 0, ni, r << bits), i1 = lower_key(il, i0, ni, (r + 1) << bits);
-    int64_t dg = deg[r];
-    int64_t nd2 = dg - (d1 - d0) + (i1 - i0);
-    plan[4 * j + 0] = d0;
-    plan[4 * j + 1] = d1;
-    plan[4 * j + 2] = i0;
-    plan[4 * j + 3] = i1;
-    olddeg[j] = dg;
-    cchunks[j] = cdiv(dg, RW_CH);
-    wchunks[j] = cdiv(round4(dg > nd2 ? dg : nd2), RW_CH);
-    if (round4(nd2) > off[r + 1] - off[r]) atomicAdd(overflow, 1ull);
-  }
-}
-
-// row j of chunk c: largest j with pre[j] <= c
-__device__ __forceinline__ int64_t chunk_row(const int64_t* pre, int64_t nr, int64_t c) {
-  int64_t lo = 0, hi = nr - 1;
-  while (lo < hi) {
-    int64_t mid = (lo + hi + 1) >> 1;
-    if (pre[mid] <= c) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
-}
-
-// copy pass: the old elements of every touched row into scratch, one warp per chunk
-__global__ void k_row_copy(const uint64_t* __restrict__ rows, const int64_t* __restrict__ nrp,
-                           const int64_t* __restrict__ sofs, const int64_t* __restrict__ cpre,
-                           const int64_t* __restrict__ off, const int32_t* __restrict__ deg,
-                           const int32_t* __restrict__ col, int32_t* __restrict__ scratch) {
-  const int64_t nr = *nrp;
-  const int lane = threadIdx.x & 31;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t total = cpre[nr];
-  for (int64_t c = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; c < total; c += nw) {
-    const int64_t j = chunk_row(cpre, nr, c);
-    const int64_t r = (int64_t)rows[j];
-    const int64_t x0 = (c - cpre[j]) * RW_CH;
-    const int64_t x1 = min(x0 + (int64_t)RW_CH, (int64_t)deg[r]);
-    const int64_t base = off[r];
-    int32_t* S = scratch + sofs[j];
-    for (int64_t x = x0 + lane; x < x1; x += 32) S[x] = col[base + x];
-  }
-}
-
-// write pass over old positions: every surviving element moves to
-// x - (#deletions below it) + (#insertions below it); slots from the new degree
-// up to the old end get the sentinel
-__global__ void k_row_survivors(const uint64_t* __restrict__ rows, const int64_t* __restrict__ nrp,
-                                const int64_t* __restrict__ plan, const int64_t* __restrict__ sofs,
-                                const int64_t* __restrict__ wpre, const uint64_t* __restrict__ dl,
-                                const uint64_t* __restrict__ il, int bits, const int64_t* __restrict__ off,
-                                const int32_t* __restrict__ deg, int32_t* __restrict__ col,
-                                const int32_t* __restrict__ scratch, int32_t sent) {
-  const int64_t nr = *nrp;
-  const int lane = threadIdx.x & 31;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t total = wpre[nr];
-  for (int64_t c = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; c < total; c += nw) {
-    const int64_t j = chunk_row(wpre, nr, c);
-    const int64_t r = (int64_t)rows[j];
-    const int64_t d0 = plan[4 * j], d1 = plan[4 * j + 1], i0 = plan[4 * j + 2], i1 = plan[4 * j + 3];
-    const int64_t d_old = deg[r];
-    const int64_t d_new = d_old - (d1 - d0) + (i1 - i0);
-    const int64_t pad_end = round4(d_old > d_new ? d_old : d_new);
-    const int64_t base = off[r], cap = off[r + 1] - base;
-    const int32_t* S = scratch + sofs[j];
-    const int64_t x0 = (c - wpre[j]) * RW_CH;
-    const int64_t x1 = min(x0 + (int64_t)RW_CH, pad_end);
-    for (int64_t x = x0 + lane; x < x1; x += 32) {
-      if (x < d_old) {
-        const int32_t v = S[x];
-        const uint64_t key = ((uint64_t)r << bits) | (uint64_t)v;
-        const int64_t dl_lt = lower_key(dl, d0, d1, key);
-        if (!(dl_lt < d1 && dl[dl_lt] == key)) {
-          const int64_t pos = x - (dl_lt - d0) + (lower_key(il, i0, i1, key) - i0);
-          if (pos >= 0 && pos < cap) col[base + pos] = v;
-        }
-      }
-      if (x >= d_new && x < cap) col[base + x] = sent;
-    }
-  }
-}
-
-// write pass over insertions: insertion k of row r goes to
-// (#insertions below it) + (#old elements below it) - (#deletions below it)
-__global__ void k_row_insertions(const uint64_t* __restrict__ rows, const int64_t* __restrict__ nrp,
-                                 const int64_t* __restrict__ plan, const int64_t* __restrict__ sofs,
-                                 const uint64_t* __restrict__ dl, const uint64_t* __restrict__ il,
-                                 const int64_t* __restrict__ nip, int bits, const int64_t* __restrict__ off,
-                                 const int32_t* __restrict__ deg, int32_t* __restrict__ col,
-                                 const int32_t* __restrict__ scratch) {
-  const int64_t nr = *nrp, ni = *nip;
-  const uint64_t mask = (1ull << bits) - 1;
-  GRID_STRIDE(k, ni) {
-    const uint64_t r = il[k] >> bits;
-    int64_t lo = 0, hi = nr - 1;   // touched-row index of r
-    while (lo < hi) {
-      int64_t mid = (lo + hi) >> 1;
-      if (rows[mid] < r) lo = mid + 1;
-      else hi = mid;
-    }
-    const int64_t j = lo;
-    const int64_t d0 = plan[4 * j], d1 = plan[4 * j + 1], i0 = plan[4 * j + 2];
-    const int32_t y = (int32_t)(il[k] & mask);
-    const int32_t* S = scratch + sofs[j];
-    int32_t a = 0, b = deg[r];
-    while (a < b) {
-      int32_t mid = (a + b) >> 1;
-      if (S[mid] < y) a = mid + 1;
-      else b = mid;
-    }
-    const int64_t dl_lt = lower_key(dl, d0, d1, (r << bits) | (uint64_t)y);
-    const int64_t pos = (k - i0) + a - (dl_lt - d0);
-    const int64_t base = off[r], cap = off[r + 1] - base;
-    if (pos >= 0 && pos < cap) col[base + pos] = y;
-  }
-}
-
-__global__ void k_row_degrees(const uint64_t* __restrict__ rows, const int64_t* __restrict__ nrp,
-                              const int64_t* __restrict__ plan, int32_t* __restrict__ deg) {
-  const int64_t nr = *nrp;
-  GRID_STRIDE(j, nr) {
-    const uint64_t r = rows[j];
-    deg[r] = deg[r] - (int32_t)(plan[4 * j + 1] - plan[4 * j]) + (int32_t)(plan[4 * j + 3] - plan[4 * j + 2]);
-  }
 }
 
 constexpr int32_t REPACK_SHORT = 64;     // rows of at most this degree are rewritten by one thread
@@ -442,10 +297,6 @@ __global__ void k_repack_short(const int64_t* __restrict__ off, const int32_t* _
   }
 }
 
-__global__ void k_u64_to_i32_low(const uint64_t* __restrict__ in, int64_t k, int32_t* __restrict__ out) {
-  GRID_STRIDE(i, k) out[i] = (int32_t)in[i];
-}
-
 // ------------------------------------------------------------------ host
 
 // a direction whose new rows do not fit their capacity is rebuilt with fresh
@@ -530,92 +381,365 @@ static int repack_direction(Graph* g, Csr* c, const uint64_t* dl, int64_t nd, co
   return OK;
 }
 
-static int edit_direction(Graph* g, Csr* c, const uint64_t* dl, int64_t nd, const uint64_t* il, int64_t ni,
-                          const int64_t* ni_dev, bool* repacked) {
-  cudaStream_t s = g->stream;
-  int bits = g->id_bits;
-  *repacked = false;
-  int64_t nrk = nd + ni;
-  if (nrk == 0) return OK;
-  // touched rows: sorted distinct row ids
-  size_t need = 0;
-  {
-    Carve probe(nullptr);
-    probe.take<uint64_t>(nrk);
-    probe.take<uint64_t>(nrk);
-    probe.take<uint64_t>(nrk);
-    probe.take<uint8_t>(nrk);
-    probe.take<char>((int64_t)std::max(radix_tmp_bytes(nrk), compact_tmp_bytes(nrk)));
-    probe.take<int64_t>(1);
-    need = probe.used + 4096;
-  }
-  void* base;
-  TRY(scratch_get(g, 3, need, &base));
-  Carve cv(base);
-  uint64_t* rk = cv.take<uint64_t>(nrk);
-  uint64_t* alt = cv.take<uint64_t>(nrk);
-  uint64_t* rows = cv.take<uint64_t>(nrk);
-  uint8_t* flag = cv.take<uint8_t>(nrk);
-  void* tmp = cv.take<char>((int64_t)std::max(radix_tmp_bytes(nrk), compact_tmp_bytes(nrk)));
-  int64_t* cnt = cv.take<int64_t>(1);
-  note_launch(); k_row_keys<<<grid_for(nrk, 256), 256, 0, s>>>(dl, nd, il, ni, bits, rk);
-  TRY(radix_sort_u64(rk, alt, nrk, bits, tmp, s));
-  TRY(flag_unique_sorted(rk, nrk, flag, s));
-  TRY(compact_u64(rk, flag, nrk, rows, cnt, tmp, s));
-  int64_t nr = 0;
-  TRY(cudaMemcpyAsync(&nr, cnt, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  TRY(cudaStreamSynchronize(s));
+// ------------------------------------------------------------------ editing rows in place
+//
+// Touched rows of both directions with their plans, rewritten by two kernels:
+//   k_edit_short  rows of at most EDIT_SHORT slots, eight lanes per row, the
+//                 row in registers;
+//   k_edit_long   the others in chunks of RW_CH slots, one warp per chunk
+//                 staged in shared memory; a row of several chunks is copied to
+//                 scratch first (k_edit_copy), because its chunks move into one
+//                 another's places.
+// A survivor x goes to x - (deletions below it) + (insertions below it), an
+// insertion to its rank among the insertions + old elements below it -
+// deletions below it.  A chunk looks only at the changes that fall into it:
+// held one per lane when they are few, else counted into the places where they
+// take effect and summed over the chunk (a prefix sum per 32 elements), so an
+// element costs no search.  Bound by reading and writing the rows: 2.7M
+// changes of a graph of 271M edges touch rows that hold most of them, about
+// 2 GB per direction.  Before, a warp searched both lists of the row in global
+// memory for every element: 5.7 ms per direction there, with a scratch copy of
+// every touched row.
+constexpr int RW_CH = 1024;         // slots of a chunk
+constexpr int EDIT_SHORT = 64;      // rows of at most this many slots: eight lanes
+constexpr int EDIT_FEW = 8;         // changes of a chunk compared one by one
 
-  void* base2;
-  size_t need2 = 0;
-  {
-    Carve probe(nullptr);
-    probe.take<int64_t>(4 * nr);
-    for (int i = 0; i < 3; i++) probe.take<int64_t>(nr + 1);
-    probe.take<int64_t>(scan_tmp_elems(nr));
-    probe.take<unsigned long long>(1);
-    need2 = probe.used + 4096;
-  }
-  TRY(scratch_get(g, 4, need2, &base2));
-  Carve c2(base2);
-  int64_t* plan = c2.take<int64_t>(4 * nr);
-  int64_t* sofs = c2.take<int64_t>(nr + 1);
-  int64_t* cpre = c2.take<int64_t>(nr + 1);
-  int64_t* wpre = c2.take<int64_t>(nr + 1);
-  int64_t* sscr = c2.take<int64_t>(scan_tmp_elems(nr));
-  unsigned long long* ovf = c2.take<unsigned long long>(1);
-  TRY(cudaMemsetAsync(ovf, 0, sizeof(unsigned long long), s));
-  note_launch(); k_row_plan<<<grid_for(nr, 256), 256, 0, s>>>(rows, nr, dl, nd, il, ni, bits, c->off, c->deg, plan, sofs,
-                                                              cpre, wpre, ovf);
-  TRY(scan_excl<int64_t>(sofs, sofs, nr, sscr, s));
-  TRY(scan_excl<int64_t>(cpre, cpre, nr, sscr, s));
-  TRY(scan_excl<int64_t>(wpre, wpre, nr, sscr, s));
-  unsigned long long ovf_h = 0;
-  int64_t stot = 0;
-  TRY(cudaMemcpyAsync(&ovf_h, ovf, sizeof(ovf_h), cudaMemcpyDeviceToHost, s));
-  TRY(cudaMemcpyAsync(&stot, sofs + nr, sizeof(stot), cudaMemcpyDeviceToHost, s));
-  TRY(cudaStreamSynchronize(s));
+}  // namespace dfpr
 
-  if (ovf_h == 0) {
-    void* sp;
-    TRY(scratch_get(g, 5, sizeof(int32_t) * (size_t)(stot + 1), &sp));
-    int32_t* S = (int32_t*)sp;
-    const int wgrid = num_sms() * 16;
-    note_launch(); k_row_copy<<<wgrid, 256, 0, s>>>(rows, cnt, sofs, cpre, c->off, c->deg, c->col, S);
-    note_launch(); k_row_survivors<<<wgrid, 256, 0, s>>>(rows, cnt, plan, sofs, wpre, dl, il, bits, c->off, c->deg, c->col,
-                                                         S, g->n);
-    if (ni) {
-      note_launch(); k_row_insertions<<<grid_for(ni, 256), 256, 0, s>>>(rows, cnt, plan, sofs, dl, il, ni_dev, bits,
-                                                                        c->off, c->deg, c->col, S);
+struct dfpr::EditStatus {
+  int32_t n_del, n_ins;   // effective deletions / insertions
+  int32_t bad;            // an id out of range (nothing was changed)
+  // per direction (out 0, in 1): touched rows, those of more than EDIT_SHORT
+  // slots, their chunks, and the scratch chunks of rows of several; the device
+  // leaves the direction unchanged (skip), because rows overflow (ovf) or the
+  // scratch is too small (need)
+  int32_t nr[2], nlong[2], chunks[2], scratch[2], skip[2], ovf[2], need[2];
+};
+
+// device arrays of one batch's edit, in one scratch buffer
+struct dfpr::EditBufs {
+  uint64_t *dl[2], *il[2];   // Delta-, Delta+ sorted by (src, dst) and by (dst, src)
+  int32_t* rows[2];
+  int4* plan[2];             // per touched row: its deletions [x, y) and insertions [z, w)
+  int32_t* od[2];            // its degree before the batch
+  // rows of more than EDIT_SHORT slots: index into rows, chunks and scratch
+  // chunks before
+  int32_t *lrow[2], *lpre[2], *lsc[2];
+  EditStatus* st;
+  uint64_t* key;             // small batches: packed (src, dst, insertion, present)
+};
+
+namespace dfpr {
+
+struct EditArgs {
+  const int64_t* off[2];
+  int32_t* deg[2];
+  int32_t* col[2];
+  int32_t* S[2];          // scratch: chunk c at c x RW_CH
+  int32_t sent;
+  const double* R;        // ranks, or null: no contributions to refresh
+  long long* C;
+  const double* tab_sc;
+  int dirs;               // bit d: work on direction d
+};
+
+// the long row that chunk c belongs to
+__device__ __forceinline__ int long_row(const int32_t* pre, int nlong, int c) {
+  int lo = 0, hi = nlong - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (pre[mid] <= c) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
+// one warp: the first `len` (at most RW_CH) elements of src, a row position
+// that is a multiple of four, to dst, in whole quads (a row's slots are a
+// multiple of four), every load of a lane before its stores
+__device__ __forceinline__ void copy_chunk(const int32_t* src, int32_t len, int32_t* dst) {
+  const int lane = threadIdx.x & 31;
+  int4 v[RW_CH / 128];
+#pragma unroll
+  for (int k = 0; k < RW_CH / 128; k++) {
+    const int q = k * 32 + lane;
+    if (4 * q < len) v[k] = reinterpret_cast<const int4*>(src)[q];
+  }
+#pragma unroll
+  for (int k = 0; k < RW_CH / 128; k++) {
+    const int q = k * 32 + lane;
+    if (4 * q < len) reinterpret_cast<int4*>(dst)[q] = v[k];
+  }
+}
+
+__global__ void __launch_bounds__(256) k_edit_copy(const __grid_constant__ EditBufs B, const __grid_constant__ EditArgs p) {
+  const EditStatus& st = *B.st;
+  const int nw = (gridDim.x * blockDim.x) >> 5, w0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  for (int d = 0; d < 2; d++) {
+    if (!((p.dirs >> d) & 1) || st.skip[d] || st.scratch[d] == 0) continue;
+    const int nc = st.chunks[d];
+    for (int c = w0; c < nc; c += nw) {
+      const int l = long_row(B.lpre[d], st.nlong[d], c);
+      if (B.lpre[d][l + 1] - B.lpre[d][l] == 1) continue;   // edited straight from shared memory
+      const int part = c - B.lpre[d][l], j = B.lrow[d][l];
+      const int32_t x0 = part * RW_CH;
+      copy_chunk(p.col[d] + p.off[d][B.rows[d][j]] + x0, min(B.od[d][j] - x0, RW_CH),
+                 p.S[d] + (int64_t)(B.lsc[d][l] + part) * RW_CH);
     }
-    note_launch(); k_row_degrees<<<grid_for(nr, 256), 256, 0, s>>>(rows, cnt, plan, c->deg);
-    TRY(cudaGetLastError());
-    return OK;
   }
+}
 
-  // repack this direction: survivors + insertions, sorted, rebuilt with more slack
-  *repacked = true;
-  return repack_direction(g, c, dl, nd, il, ni);
+__device__ __forceinline__ int32_t lower_i32(const int32_t* a, int32_t lo, int32_t hi, int32_t x) {
+  while (lo < hi) {
+    const int32_t mid = (lo + hi) >> 1;
+    if (a[mid] < x) lo = mid + 1;
+    else hi = mid;
+  }
+  return lo;
+}
+
+// the row's new degree, and (out-rows) its source's contribution with it
+__device__ __forceinline__ void finish_row(const EditArgs& p, int d, int32_t r, int32_t d_new) {
+  p.deg[d][r] = d_new;
+  if (d == 0 && p.R) {
+    const double sc = d_new < TAB ? p.tab_sc[d_new] : FIX_ONE / (double)d_new;
+    p.C[r] = __double2ll_rn(p.R[r] * sc);
+  }
+}
+
+__global__ void __launch_bounds__(256) k_edit_short(const __grid_constant__ EditBufs B, const __grid_constant__ EditArgs p,
+                                                    int bits) {
+  const EditStatus& st = *B.st;
+  const int lane = threadIdx.x & 31, l = lane & 7;
+  const unsigned grp = 0xffu << (lane & 24);   // the eight lanes of this row
+  const uint64_t mask = (1ull << bits) - 1;
+  const int e0 = (p.dirs & 1) && !st.skip[0] ? st.nr[0] : 0, e1 = e0 + ((p.dirs & 2) && !st.skip[1] ? st.nr[1] : 0);
+  const int stride = (gridDim.x * blockDim.x) >> 3;
+  for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 3; w < e1; w += stride) {
+    const int d = w >= e0 ? 1 : 0, j = w - (d ? e0 : 0);
+    const int32_t r = B.rows[d][j], d_old = B.od[d][j];
+    const int4 pl = B.plan[d][j];
+    const int32_t d_new = d_old - (pl.y - pl.x) + (pl.w - pl.z);
+    const int32_t len = (int32_t)round4(d_old > d_new ? d_old : d_new);
+    if (len > EDIT_SHORT) continue;
+    const int64_t base = p.off[d][r];
+    const int32_t cap = (int32_t)min(p.off[d][r + 1] - base, (int64_t)INT32_MAX);
+    int32_t* const row = p.col[d] + base;
+    int32_t v[8];
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+      int4 q = make_int4(0, 0, 0, 0);
+      if (8 * l + 4 * h < d_old) q = reinterpret_cast<const int4*>(row)[2 * l + h];
+      v[4 * h] = q.x;
+      v[4 * h + 1] = q.y;
+      v[4 * h + 2] = q.z;
+      v[4 * h + 3] = q.w;
+    }
+    int pos[8];
+    unsigned keep = 0;
+#pragma unroll
+    for (int e = 0; e < 8; e++) {
+      pos[e] = 8 * l + e;
+      if (pos[e] < d_old) keep |= 1u << e;
+    }
+    const unsigned old = keep;
+    for (int k = pl.x; k < pl.y; k++) {
+      const int32_t y = (int32_t)(B.dl[d][k] & mask);
+#pragma unroll
+      for (int e = 0; e < 8; e++) {
+        pos[e] -= y < v[e];
+        if (y == v[e]) keep &= ~(1u << e);
+      }
+    }
+    __syncwarp(grp);   // every lane holds its elements before any is overwritten
+    for (int k = pl.z; k < pl.w; k++) {
+      const int32_t y = (int32_t)(B.il[d][k] & mask);
+      int below = 0;
+#pragma unroll
+      for (int e = 0; e < 8; e++) {
+        pos[e] += y < v[e];
+        below += ((old >> e) & 1u) && v[e] < y ? 1 : 0;
+      }
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) below += __shfl_xor_sync(grp, below, o);
+      if (((k - pl.z) & 7) == l) {
+        for (int i = pl.x; i < pl.y; i++) below -= (int32_t)(B.dl[d][i] & mask) < y;
+        const int at = k - pl.z + below;
+        if (at >= 0 && at < cap) row[at] = y;
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 8; e++) {
+      const int x = 8 * l + e;
+      if (((keep >> e) & 1u) && pos[e] != x && pos[e] >= 0 && pos[e] < cap) row[pos[e]] = v[e];
+      if (x >= d_new && x < len && x < cap) row[x] = p.sent;
+    }
+    if (l == 0) finish_row(p, d, r, d_new);
+  }
+}
+
+constexpr int EDIT_WARPS = 4;   // warps of a k_edit_long block
+
+__global__ void __launch_bounds__(EDIT_WARPS * 32) k_edit_long(const __grid_constant__ EditBufs B,
+                                                               const __grid_constant__ EditArgs p, int bits) {
+  __shared__ __align__(16) int32_t stage[EDIT_WARPS][RW_CH];
+  __shared__ int32_t delta[EDIT_WARPS][RW_CH + 1];   // change of the shift at an element, + DEAD where it is deleted
+  constexpr int32_t DEAD = 1 << 30;                  // (a row gets fewer than 2^29 insertions)
+  const EditStatus& st = *B.st;
+  const int lane = threadIdx.x & 31;
+  const int nw = gridDim.x * EDIT_WARPS;
+  const uint64_t mask = (1ull << bits) - 1;
+  int32_t* const T = stage[threadIdx.x >> 5];
+  int32_t* const D = delta[threadIdx.x >> 5];
+  const int e0 = (p.dirs & 1) && !st.skip[0] ? st.chunks[0] : 0;
+  const int e1 = e0 + ((p.dirs & 2) && !st.skip[1] ? st.chunks[1] : 0);
+  for (int w = blockIdx.x * EDIT_WARPS + (threadIdx.x >> 5); w < e1; w += nw) {
+    const int d = w >= e0 ? 1 : 0, c = w - (d ? e0 : 0);
+    const int li = long_row(B.lpre[d], st.nlong[d], c);
+    const int j = B.lrow[d][li], part = c - B.lpre[d][li];
+    const bool one = B.lpre[d][li + 1] - B.lpre[d][li] == 1;
+    const int32_t r = B.rows[d][j], d_old = B.od[d][j];
+    const int4 pl = B.plan[d][j];
+    const int nd = pl.y - pl.x, ni = pl.w - pl.z;
+    const int32_t d_new = d_old - nd + ni;
+    const int32_t len = (int32_t)round4(d_old > d_new ? d_old : d_new);
+    const int64_t base = p.off[d][r];
+    const int32_t cap = (int32_t)min(p.off[d][r + 1] - base, (int64_t)INT32_MAX);
+    int32_t* const row = p.col[d] + base;
+    const int32_t x0 = part * RW_CH, no = max(0, min(d_old - x0, RW_CH));   // old elements of the chunk
+    const uint64_t *dl = B.dl[d], *il = B.il[d];
+    __syncwarp();
+    copy_chunk(one ? row : p.S[d] + (int64_t)(B.lsc[d][li] + part) * RW_CH, no, T);
+    int32_t before = 0;   // the element before the chunk
+    if (part > 0 && no > 0) before = p.S[d][(int64_t)(B.lsc[d][li] + part) * RW_CH - 1];
+    __syncwarp();
+    // the chunk's changes: deletions [da, db) are those of its elements;
+    // insertions [ia, ib) those above the element before it and below its last
+    // one (the last chunk with elements: all that are left)
+    int da = pl.x, db = pl.y, ia = pl.z, ib = pl.w;
+    int32_t mine = 0;
+    const bool few = nd + ni <= 32;
+    if (few && lane < nd + ni) mine = (int32_t)((lane < nd ? dl[pl.x + lane] : il[pl.z + lane - nd]) & mask);
+    if (no == 0) {
+      da = db;
+      ia = ib;
+    } else if (!one) {
+      const bool last = x0 + RW_CH >= d_old;
+      const int32_t lo = T[0], hi = T[no - 1];
+      if (few) {
+        const bool del = lane < nd, ins = lane >= nd && lane < nd + ni;
+        da = pl.x + __popc(__ballot_sync(0xffffffffu, del && mine < lo));
+        db = pl.x + __popc(__ballot_sync(0xffffffffu, del && mine <= hi));
+        const int bi = __popc(__ballot_sync(0xffffffffu, ins && part > 0 && mine < before));
+        const int ei = __popc(__ballot_sync(0xffffffffu, ins && (last || mine < hi)));
+        ia = pl.z + bi;
+        ib = pl.z + ei;
+      } else {
+        const uint64_t rk = (uint64_t)r << bits;
+        int at = 0;   // lanes 0 to 3 search one bound each
+        if (lane == 0) at = (int)lower_key(dl, pl.x, pl.y, rk | (uint64_t)lo);
+        if (lane == 1) at = (int)lower_key(dl, pl.x, pl.y, (rk | (uint64_t)hi) + 1);
+        if (lane == 2) at = part > 0 ? (int)lower_key(il, pl.z, pl.w, rk | (uint64_t)before) : pl.z;
+        if (lane == 3) at = last ? pl.w : (int)lower_key(il, pl.z, pl.w, rk | (uint64_t)hi);
+        da = __shfl_sync(0xffffffffu, at, 0);
+        db = __shfl_sync(0xffffffffu, at, 1);
+        ia = __shfl_sync(0xffffffffu, at, 2);
+        ib = __shfl_sync(0xffffffffu, at, 3);
+      }
+    }
+    const int shift = (ia - pl.z) - (da - pl.x);   // of the chunk's first element
+    const int cd = db - da, ci = ib - ia;
+    if (cd + ci <= EDIT_FEW) {
+      // one change per lane, compared with every element
+      int32_t y = 0;
+      if (lane < cd + ci) y = (int32_t)((lane < cd ? dl[da + lane] : il[ia + lane - cd]) & mask);
+      for (int32_t b = 0; b < no; b += 32) {
+        const int32_t i = b + lane, v = i < no ? T[i] : 0;
+        int sh = shift;
+        bool dead = false;
+        for (int k = 0; k < cd; k++) {
+          const int32_t z = __shfl_sync(0xffffffffu, y, k);
+          sh -= z < v;
+          dead |= z == v;
+        }
+        for (int k = cd; k < cd + ci; k++) sh += __shfl_sync(0xffffffffu, y, k) < v;
+        const int32_t at = x0 + i + sh;
+        if (i < no && !dead && sh != 0 && at >= 0 && at < cap) row[at] = v;
+      }
+      if (lane >= cd && lane < cd + ci) {
+        int below = da - pl.x;
+        for (int k = 0; k < cd; k++) below += (int32_t)(dl[da + k] & mask) < y;
+        const int32_t at = (ia + lane - cd - pl.z) + x0 + lower_i32(T, 0, no, y) - below;
+        if (at >= 0 && at < cap) row[at] = y;
+      }
+    } else {
+      for (int32_t i = lane; i <= no; i += 32) D[i] = 0;
+      __syncwarp();
+      for (int k = da + lane; k < db; k += 32) {
+        const int32_t i = lower_i32(T, 0, no, (int32_t)(dl[k] & mask));   // its element (present)
+        atomicAdd(&D[i], DEAD);
+        atomicAdd(&D[i + 1], -1);
+      }
+      for (int k = ia + lane; k < ib; k += 32) {
+        const int32_t y = (int32_t)(il[k] & mask);
+        const int32_t i = lower_i32(T, 0, no, y);
+        atomicAdd(&D[i], 1);
+        const int below = (int)(lower_key(dl, da, db, ((uint64_t)r << bits) | (uint64_t)y) - pl.x);
+        const int32_t at = (k - pl.z) + x0 + i - below;
+        if (at >= 0 && at < cap) row[at] = y;
+      }
+      __syncwarp();
+      int run = shift;
+      for (int32_t b = 0; b < no; b += 32) {
+        const int32_t i = b + lane, m = i < no ? D[i] : 0;
+        const bool dead = m > DEAD / 2;
+        int sh = dead ? m - DEAD : m;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(0xffffffffu, sh, o);
+          if (lane >= o) sh += y;
+        }
+        const int all = __shfl_sync(0xffffffffu, sh, 31);
+        sh += run;
+        run += all;
+        const int32_t at = x0 + i + sh;
+        if (i < no && !dead && sh != 0 && at >= 0 && at < cap) row[at] = T[i];
+      }
+    }
+    for (int32_t x = x0 + lane; x < min(x0 + RW_CH, len); x += 32)
+      if (x >= d_new && x < cap) row[x] = p.sent;
+    if (part == 0 && lane == 0) finish_row(p, d, r, d_new);
+  }
+}
+
+// queue the edit of the directions in `dirs`; rows: touched rows of both, at most
+static void launch_edit(Graph* g, const EditBufs& B, int32_t* const* S, int dirs, int64_t rows) {
+  cudaStream_t s = g->stream;
+  EditArgs p;
+  const Csr* c[2] = {&g->out, &g->in};
+  for (int d = 0; d < 2; d++) {
+    p.off[d] = c[d]->off;
+    p.deg[d] = c[d]->deg;
+    p.col[d] = c[d]->col;
+    p.S[d] = S[d];
+  }
+  p.sent = g->n;
+  p.R = g->has_ranks ? g->R : nullptr;
+  p.C = g->C[g->ccur];
+  p.tab_sc = g->tab_sc;
+  p.dirs = dirs;
+  note_launch(); k_edit_copy<<<num_sms() * 4, 256, 0, s>>>(B, p);
+  note_launch(); k_edit_short<<<grid_for(8 * rows, 256), 256, 0, s>>>(B, p, g->id_bits);
+  note_launch(); k_edit_long<<<num_sms() * 6, EDIT_WARPS * 32, 0, s>>>(B, p, g->id_bits);
+}
+
+// what a row of `len` slots adds to the lists of long rows: one entry, its
+// chunks, and its scratch chunks (20 + 22 + 22 bits: at most SMALL_MAX entries
+// here, and a direction holds fewer than 2^31 slots)
+__device__ __forceinline__ uint64_t long_counts(int64_t len) {
+  if (len <= EDIT_SHORT) return 0;
+  const uint64_t c = (uint64_t)cdiv(len, RW_CH);
+  return 1ull << 44 | c << 22 | (c > 1 ? c : 0);
 }
 
 // ------------------------------------------------------------------ small batches
@@ -630,49 +754,21 @@ static int edit_direction(Graph* g, Csr* c, const uint64_t* dl, int64_t nd, cons
 //                   (src, dst) and as (dst, src) in registers (bitonic: strides
 //                   within a thread and a warp need no barrier), effective
 //                   flags, compaction, touched rows with their edit plans;
-//   k_small_copy    the old elements of touched rows longer than a chunk into
-//                   scratch (a row is edited in place, by many warps);
-//   k_small_edit    one warp per touched row, staged in shared memory, or per
-//                   chunk of a longer row; both directions at once, with the
-//                   new degrees and the contributions of the sources.
+// and then the row edit above, both directions at once, with the new degrees
+// and the contributions of the sources.
 // Device time of a batch: 50 us for 168 edges on a graph of 2^20 vertices, 115
 // for 4000 and 145 for 6300 on one of 2.6M (k_small_keys 4 to 8, k_small_ingest
-// 9 / 37 / 63, k_small_copy 6 to 8, k_small_edit 12 to 37).  Before, one block
-// ran both directions in turn with the sort in shared memory (53 us at 168
-// edges, 143 at 1300, 312 at 4000) and five kernels per direction followed: 166
-// us in all for 168 edges, 450 for 4000; above 4096 edges the path below, 930
-// us for 6300.
+// 9 / 37 / 63).  Before, one block ran both directions in turn with the sort in
+// shared memory (53 us at 168 edges, 143 at 1300, 312 at 4000) and five kernels
+// per direction followed: 166 us in all for 168 edges, 450 for 4000; above 4096
+// edges the path below, 930 us for 6300.
 // A direction whose rows overflow their capacity, or whose scratch is too
 // small, is left alone by the device and finished by the host.
 constexpr int SMALL_MAX = 16384;                // edges of a batch (deletions + insertions)
 constexpr int SMALL_THREADS = 1024;
 constexpr uint64_t BAD = ~1ull;                  // key of an edge with an id out of range (no packed key: ids are below 2^31)
 
-}  // namespace dfpr
-
-struct dfpr::SmallStatus {
-  int32_t n_del, n_ins;   // effective deletions / insertions
-  int32_t bad;
-  // per direction (out 0, in 1): touched rows, those longer than a chunk and
-  // their chunks; the device left the direction unchanged (skip), because rows
-  // overflow (ovf) or the scratch is too small (need)
-  int32_t nr[2], nlong[2], chunks[2], skip[2], ovf[2], need[2];
-};
-
-// device arrays of one small batch, all in one scratch buffer
-struct dfpr::SmallBufs {
-  uint64_t* key;           // packed (src, dst, insertion, present)
-  uint64_t *dl[2], *il[2];   // Delta-, Delta+ sorted by (src, dst) and by (dst, src)
-  int32_t* rows[2];
-  int4* plan[2];           // per touched row: its deletions [x, y) and insertions [z, w)
-  int32_t* od[2];          // its degree before the batch
-  int32_t *lrow[2], *lpre[2];   // rows longer than a chunk: index into rows, chunks before
-  SmallStatus* st;
-};
-
-namespace dfpr {
-
-static size_t small_carve(void* base, int64_t cap, SmallBufs* B) {
+static size_t small_carve(void* base, int64_t cap, EditBufs* B) {
   Carve c(base);
   B->key = c.take<uint64_t>(cap);
   B->dl[0] = B->il[0] = nullptr;   // the graph's own buffers
@@ -684,8 +780,9 @@ static size_t small_carve(void* base, int64_t cap, SmallBufs* B) {
     B->od[d] = c.take<int32_t>(cap);
     B->lrow[d] = c.take<int32_t>(cap);
     B->lpre[d] = c.take<int32_t>(cap + 1);
+    B->lsc[d] = c.take<int32_t>(cap);
   }
-  B->st = c.take<SmallStatus>(1);
+  B->st = c.take<EditStatus>(1);
   return c.used;
 }
 
@@ -824,7 +921,7 @@ constexpr size_t small_smem() {
 template <int E>
 __global__ void __launch_bounds__(SMALL_THREADS, 1)
     k_small_ingest(int N, int bits, const __grid_constant__ SmallCsr out, const __grid_constant__ SmallCsr in,
-                   const __grid_constant__ SmallBufs B) {
+                   const __grid_constant__ EditBufs B) {
   extern __shared__ uint64_t K[];   // the sorted keys, then the effective changes (row, col, insertion)
   uint16_t* const DP = reinterpret_cast<uint16_t*>(K + SMALL_THREADS * E + 8);
   uint16_t* const RS = DP + SMALL_THREADS * E + 8;
@@ -832,7 +929,7 @@ __global__ void __launch_bounds__(SMALL_THREADS, 1)
   const int dir = blockIdx.x, t = threadIdx.x;
   const SmallCsr& c = dir == 0 ? out : in;
   const uint64_t mask = (1ull << bits) - 1;
-  SmallStatus& st = *B.st;
+  EditStatus& st = *B.st;
   uint64_t k[E];
   bool bad = false;
 #pragma unroll
@@ -848,7 +945,7 @@ __global__ void __launch_bounds__(SMALL_THREADS, 1)
   if (__syncthreads_or(bad)) {
     if (t == 0) {
       st.bad = 1;
-      st.nr[dir] = st.nlong[dir] = st.chunks[dir] = 0;
+      st.nr[dir] = st.nlong[dir] = st.chunks[dir] = st.scratch[dir] = 0;
       st.skip[dir] = 1;
     }
     return;
@@ -927,211 +1024,34 @@ __global__ void __launch_bounds__(SMALL_THREADS, 1)
       B.plan[dir][j] = make_int4(d0, d1, i0, i1);
       B.od[dir][j] = dg;
       ovf |= round4(dn) > c.off[r + 1] - c.off[r];
-      const int32_t len = dg > dn ? dg : dn;
-      if (len > RW_CH) longs = 1ull << 32 | (uint64_t)cdiv(round4(len), RW_CH);
+      longs = long_counts(round4(dg > dn ? dg : dn));
     }
     if (__syncthreads_or(longs != 0)) {
       const uint64_t before = carry + block_excl(longs, wsum, &tot);
       if (longs) {
-        B.lrow[dir][before >> 32] = j;
-        B.lpre[dir][before >> 32] = (int32_t)(uint32_t)before;
+        const int at = (int)(before >> 44);
+        B.lrow[dir][at] = j;
+        B.lpre[dir][at] = (int32_t)(before >> 22 & 0x3fffff);
+        B.lsc[dir][at] = (int32_t)(before & 0x3fffff);
       }
       carry += tot;
     }
   }
   const int any_ovf = __syncthreads_or(ovf);
   if (t == 0) {
-    const int64_t chunks = (int64_t)(uint32_t)carry;
+    const int nlong = (int)(carry >> 44), chunks = (int)(carry >> 22 & 0x3fffff), scratch = (int)(carry & 0x3fffff);
     st.bad = 0;
     st.n_del = nde;
     st.n_ins = nie;
     st.nr[dir] = nr;
-    st.nlong[dir] = (int32_t)(carry >> 32);
-    st.chunks[dir] = (int32_t)chunks;
-    B.lpre[dir][carry >> 32] = (int32_t)chunks;
+    st.nlong[dir] = nlong;
+    st.chunks[dir] = chunks;
+    st.scratch[dir] = scratch;
+    B.lpre[dir][nlong] = chunks;
     st.ovf[dir] = any_ovf ? 1 : 0;
-    st.need[dir] = chunks * RW_CH > c.scap ? 1 : 0;
+    st.need[dir] = (int64_t)scratch * RW_CH > c.scap ? 1 : 0;
     st.skip[dir] = st.ovf[dir] | st.need[dir];
   }
-}
-
-struct SmallEdit {
-  const int64_t* off[2];
-  int32_t* deg[2];
-  int32_t* col[2];
-  int32_t* S[2];          // scratch of rows longer than a chunk: chunk c of the direction at c x RW_CH
-  int32_t sent;
-  const double* R;        // ranks, or null: no contributions to refresh
-  long long* C;
-  const double* tab_sc;
-  int dirs;               // bit d: work on direction d
-};
-
-// the long row that chunk c belongs to
-__device__ __forceinline__ int long_row(const int32_t* pre, int nlong, int c) {
-  int lo = 0, hi = nlong - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (pre[mid] <= c) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
-}
-
-// one warp: the first `len` (at most RW_CH) elements of src, a row position
-// that is a multiple of four, to dst, in whole quads (a row's slots are a
-// multiple of four), every load of a lane before its stores
-__device__ __forceinline__ void copy_chunk(const int32_t* src, int32_t len, int32_t* dst) {
-  const int lane = threadIdx.x & 31;
-  int4 v[RW_CH / 128];
-#pragma unroll
-  for (int k = 0; k < RW_CH / 128; k++) {
-    const int q = k * 32 + lane;
-    if (4 * q < len) v[k] = reinterpret_cast<const int4*>(src)[q];
-  }
-#pragma unroll
-  for (int k = 0; k < RW_CH / 128; k++) {
-    const int q = k * 32 + lane;
-    if (4 * q < len) reinterpret_cast<int4*>(dst)[q] = v[k];
-  }
-}
-
-__global__ void __launch_bounds__(256) k_small_copy(const __grid_constant__ SmallBufs B,
-                                                    const __grid_constant__ SmallEdit p) {
-  const SmallStatus& st = *B.st;
-  const int nw = (gridDim.x * blockDim.x) >> 5, w0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  for (int d = 0; d < 2; d++) {
-    if (!((p.dirs >> d) & 1) || st.skip[d]) continue;
-    const int nc = st.chunks[d];
-    for (int c = w0; c < nc; c += nw) {
-      const int l = long_row(B.lpre[d], st.nlong[d], c), j = B.lrow[d][l];
-      const int32_t x0 = (c - B.lpre[d][l]) * RW_CH;
-      const int32_t* row = p.col[d] + p.off[d][B.rows[d][j]];
-      copy_chunk(row + x0, min(B.od[d][j] - x0, RW_CH), p.S[d] + (int64_t)c * RW_CH);
-    }
-  }
-}
-
-__device__ __forceinline__ int32_t lower_i32(const int32_t* a, int32_t lo, int32_t hi, int32_t x) {
-  while (lo < hi) {
-    const int32_t mid = (lo + hi) >> 1;
-    if (a[mid] < x) lo = mid + 1;
-    else hi = mid;
-  }
-  return lo;
-}
-
-// one warp: positions [x0, x1) of a touched row (its old elements from x0 on in
-// shared memory at T, all of them at S; the padding after them included) and its
-// insertions [k0, k1) written to their new places: a survivor x goes to x - (deletions below it) + (insertions below
-// it), an insertion to its rank among the insertions + old elements below it -
-// deletions below it
-__device__ __forceinline__ void edit_row_part(const int32_t* T, const int32_t* S, int32_t x0, int32_t x1, int k0, int k1, int32_t r, int4 pl,
-                                              int32_t d_old, int32_t cap, const uint64_t* __restrict__ dl,
-                                              const uint64_t* __restrict__ il, uint64_t mask, int bits,
-                                              int32_t* __restrict__ row, int32_t sent) {
-  const int lane = threadIdx.x & 31;
-  const int nd = pl.y - pl.x, ni = pl.w - pl.z;
-  const int32_t d_new = d_old - nd + ni;
-  const bool few = nd + ni <= 32;   // the row's changes in registers, one per lane
-  const int32_t mine = few && lane < nd + ni ? (int32_t)((lane < nd ? dl[pl.x + lane] : il[pl.z + lane - nd]) & mask) : 0;
-  const uint64_t rk = (uint64_t)r << bits;
-  for (int32_t xb = x0; xb < x1; xb += 32) {
-    const int32_t x = xb + lane;
-    const bool old = x < x1 && x < d_old;
-    const int32_t v = old ? T[x - x0] : 0;
-    int dlt = 0, ilt = 0;
-    bool dead = false;
-    if (few) {
-      for (int k = 0; k < nd; k++) {
-        const int32_t y = __shfl_sync(0xffffffffu, mine, k);
-        dlt += y < v;
-        dead |= y == v;
-      }
-      for (int k = nd; k < nd + ni; k++) ilt += __shfl_sync(0xffffffffu, mine, k) < v;
-    } else if (old) {
-      const int64_t a = lower_key(dl, pl.x, pl.y, rk | (uint64_t)v);
-      dead = a < pl.y && dl[a] == (rk | (uint64_t)v);
-      dlt = (int)(a - pl.x);
-      ilt = (int)(lower_key(il, pl.z, pl.w, rk | (uint64_t)v) - pl.z);
-    }
-    if (old && !dead) {
-      const int32_t pos = x - dlt + ilt;
-      if (pos >= 0 && pos < cap) row[pos] = v;
-    }
-    if (x < x1 && x >= d_new && x < cap) row[x] = sent;
-  }
-  for (int k = k0 + lane; k < k1; k += 32) {
-    const int32_t y = (int32_t)(il[k] & mask);
-    const int32_t pos = (k - pl.z) + lower_i32(S, 0, d_old, y) - (int32_t)(lower_key(dl, pl.x, pl.y, rk | (uint64_t)y) - pl.x);
-    if (pos >= 0 && pos < cap) row[pos] = y;
-  }
-}
-
-__global__ void __launch_bounds__(256) k_small_edit(const __grid_constant__ SmallBufs B,
-                                                    const __grid_constant__ SmallEdit p, int bits) {
-  __shared__ __align__(16) int32_t stage[8][RW_CH];
-  const SmallStatus& st = *B.st;
-  const int lane = threadIdx.x & 31;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  const uint64_t mask = (1ull << bits) - 1;
-  // the work: touched rows of both directions, then chunks of both
-  const bool on0 = (p.dirs & 1) && !st.skip[0], on1 = (p.dirs & 2) && !st.skip[1];
-  const int e0 = on0 ? st.nr[0] : 0, e1 = e0 + (on1 ? st.nr[1] : 0);
-  const int e2 = e1 + (on0 ? st.chunks[0] : 0), e3 = e2 + (on1 ? st.chunks[1] : 0);
-  for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < e3; w += nw) {
-    const bool chunk = w >= e1;
-    const int d = chunk ? (w >= e2 ? 1 : 0) : (w >= e0 ? 1 : 0);
-    const int item = chunk ? w - (d ? e2 : e1) : w - (d ? e0 : 0);
-    const int l = chunk ? long_row(B.lpre[d], st.nlong[d], item) : 0;
-    const int j = chunk ? B.lrow[d][l] : item;
-    const int32_t r = B.rows[d][j], d_old = B.od[d][j];
-    const int4 pl = B.plan[d][j];
-    const int32_t d_new = d_old - (pl.y - pl.x) + (pl.w - pl.z);
-    const int32_t len = d_old > d_new ? d_old : d_new;
-    const int64_t base = p.off[d][r];
-    const int64_t cap64 = p.off[d][r + 1] - base;
-    const int32_t cap = (int32_t)(cap64 < INT32_MAX ? cap64 : INT32_MAX), end = (int32_t)round4(len);
-    int32_t* const row = p.col[d] + base;
-    if (!chunk && len > RW_CH) continue;   // a long row: its chunks are items of their own
-    int32_t* const T = stage[threadIdx.x >> 5];
-    const int part = chunk ? item - B.lpre[d][l] : 0, parts = chunk ? B.lpre[d][l + 1] - B.lpre[d][l] : 1;
-    const int32_t x0 = part * RW_CH;
-    const int32_t* const S = chunk ? p.S[d] + (int64_t)B.lpre[d][l] * RW_CH : T;
-    __syncwarp();
-    copy_chunk(chunk ? S + x0 : row, min(d_old - x0, RW_CH), T);
-    __syncwarp();
-    const int per = (pl.w - pl.z + parts - 1) / parts;
-    const int k0 = min(pl.z + part * per, pl.w), k1 = min(k0 + per, pl.w);
-    edit_row_part(T, S, x0, min(x0 + RW_CH, end), k0, k1, r, pl, d_old, cap, B.dl[d], B.il[d], mask, bits, row, p.sent);
-    if (part > 0) continue;
-    if (lane == 0) {
-      p.deg[d][r] = d_new;
-      if (d == 0 && p.R) {   // the source's contribution with its new out-degree
-        const double sc = d_new < TAB ? p.tab_sc[d_new] : FIX_ONE / (double)d_new;
-        p.C[r] = __double2ll_rn(p.R[r] * sc);
-      }
-    }
-  }
-}
-
-static void launch_small_edit(Graph* g, const SmallApply* A, int dirs) {
-  cudaStream_t s = g->stream;
-  SmallEdit p;
-  const Csr* c[2] = {&g->out, &g->in};
-  for (int d = 0; d < 2; d++) {
-    p.off[d] = c[d]->off;
-    p.deg[d] = c[d]->deg;
-    p.col[d] = c[d]->col;
-    p.S[d] = A->S[d];
-  }
-  p.sent = g->n;
-  p.R = g->has_ranks ? g->R : nullptr;
-  p.C = g->C[g->ccur];
-  p.tab_sc = g->tab_sc;
-  p.dirs = dirs;
-  note_launch(); k_small_copy<<<num_sms() * 2, 256, 0, s>>>(*A->B, p);
-  note_launch(); k_small_edit<<<num_sms() * 4, 256, 0, s>>>(*A->B, p, g->id_bits);
 }
 
 // grow-only scratch of one direction's long rows (scratch slot 5: out, 7: in)
@@ -1167,7 +1087,7 @@ static cudaError_t grow_delta(Graph* g, uint64_t** list, int64_t* cap, int64_t u
 }
 
 template <int E>
-static cudaError_t launch_ingest(Graph* g, int N, const SmallCsr& out, const SmallCsr& in, const SmallBufs& B) {
+static cudaError_t launch_ingest(Graph* g, int N, const SmallCsr& out, const SmallCsr& in, const EditBufs& B) {
   int bps;   // (raises the kernel's shared memory limit once)
   cudaError_t e = gather_occupancy((const void*)k_small_ingest<E>, SMALL_THREADS, small_smem<E>(), &bps);
   if (e != cudaSuccess) return e;
@@ -1183,11 +1103,11 @@ static int small_launch(Graph* g, const int32_t* ds, const int32_t* dd, int64_t 
   cudaStream_t s = g->stream;
   const int N = (int)(nd + ni);
   const int64_t cap = std::max(1024, pow2_at_least(N));
-  SmallBufs B;
+  EditBufs B;
   void* bp;
   TRY(scratch_get(g, 6, small_carve(nullptr, cap, &B) + 256, &bp));
   small_carve(bp, cap, &B);
-  if (!g->small_h) TRY(cudaMallocHost(&g->small_h, sizeof(SmallStatus)));
+  if (!g->small_h) TRY(cudaMallocHost(&g->small_h, sizeof(EditStatus)));
   TRY(grow_delta(g, &g->dmin, &g->cap_dmin, g->n_dmin, nd));
   TRY(grow_delta(g, &g->dplus, &g->cap_dplus, g->n_dplus, ni));
   B.dl[0] = g->dmin;
@@ -1200,7 +1120,7 @@ static int small_launch(Graph* g, const int32_t* ds, const int32_t* dd, int64_t 
     csr[d].off = c.off;
     csr[d].deg = c.deg;
   }
-  A->B = new (std::nothrow) SmallBufs(B);
+  A->B = new (std::nothrow) EditBufs(B);
   if (!A->B) return set_error(g, ENOMEM_, "pr_apply_batch: host memory");
   note_launch();
   k_small_keys<<<grid_for(N, 256), 256, 0, s>>>(ds, dd, (int)nd, is, id, (int)ni, g->n, g->id_bits, g->perm, g->out.off,
@@ -1211,10 +1131,10 @@ static int small_launch(Graph* g, const int32_t* ds, const int32_t* dd, int64_t 
                   : N <= 8 * SMALL_THREADS ? launch_ingest<8>(g, N, csr[0], csr[1], B)
                                            : launch_ingest<16>(g, N, csr[0], csr[1], B);
   if (e == cudaSuccess) {
-    launch_small_edit(g, A, 3);
+    launch_edit(g, B, A->S, 3, 2 * (int64_t)N);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(g->small_h, B.st, sizeof(SmallStatus), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(g->small_h, B.st, sizeof(EditStatus), cudaMemcpyDeviceToHost, s);
   if (e != cudaSuccess) {
     delete A->B;
     A->B = nullptr;
@@ -1228,7 +1148,7 @@ static int small_launch(Graph* g, const int32_t* ds, const int32_t* dd, int64_t 
 static int small_complete(Graph* g, SmallApply* A) {
   cudaStream_t s = g->stream;
   const int32_t n = g->n;
-  const SmallBufs B = *A->B;
+  const EditBufs B = *A->B;
   struct Release {
     SmallApply* a;
     ~Release() {
@@ -1238,7 +1158,7 @@ static int small_complete(Graph* g, SmallApply* A) {
   } release{A};
   TRY(cudaStreamSynchronize(s));
   g->stage_busy = false;
-  const SmallStatus h = *(SmallStatus*)g->small_h;
+  const EditStatus h = *(EditStatus*)g->small_h;
   if (h.bad) return set_error(g, ERANGE_, "pr_apply_batch: vertex id out of range");
   const int64_t a = h.n_del, b = h.n_ins;
   g->n_dmin = a;
@@ -1254,9 +1174,9 @@ static int small_complete(Graph* g, SmallApply* A) {
       rep[dir] = true;
     } else {
       int64_t cap;
-      TRY(small_staging(g, dir, (int64_t)h.chunks[dir] * RW_CH, &A->S[dir], &cap));
+      TRY(small_staging(g, dir, (int64_t)h.scratch[dir] * RW_CH, &A->S[dir], &cap));
       TRY(cudaMemsetAsync(&B.st->skip[dir], 0, sizeof(int32_t), s));
-      launch_small_edit(g, A, 1 << dir);
+      launch_edit(g, B, A->S, 1 << dir, a + b);
     }
   }
   if (rep[1]) {
@@ -1323,6 +1243,59 @@ int apply_batch_complete(Graph* g, SmallApply* pending) {
   return small_complete(g, pending);
 }
 
+// the touched rows' plans (row j of *nrp, zero counts for the rest up to mr):
+// changes, old degree, whether the row overflows, and what it adds to the lists
+// of long rows: ca entries << 32 | chunks, cb scratch chunks
+__global__ void k_edit_plan(const __grid_constant__ EditBufs B, int d, const int32_t* nrp, int64_t mr, int64_t nd,
+                            int64_t ni, int bits, const int64_t* __restrict__ off, const int32_t* __restrict__ deg,
+                            int64_t* __restrict__ ca, int64_t* __restrict__ cb) {
+  const int nr = *nrp;
+  const uint64_t *dl = B.dl[d], *il = B.il[d];
+  if (blockIdx.x == 0 && threadIdx.x == 0) B.st->nr[d] = nr;
+  GRID_STRIDE(j, mr) {
+    int64_t long_chunks = 0, scratch = 0;
+    if (j < nr) {
+      const int32_t r = B.rows[d][j];
+      const uint64_t lo = (uint64_t)r << bits, hi = (uint64_t)(r + 1) << bits;
+      const int64_t d0 = lower_key(dl, 0, nd, lo), d1 = lower_key(dl, d0, nd, hi);
+      const int64_t i0 = lower_key(il, 0, ni, lo), i1 = lower_key(il, i0, ni, hi);
+      const int32_t dg = deg[r];
+      const int32_t dn = dg - (int32_t)(d1 - d0) + (int32_t)(i1 - i0);
+      B.plan[d][j] = make_int4((int)d0, (int)d1, (int)i0, (int)i1);
+      B.od[d][j] = dg;
+      if (round4(dn) > off[r + 1] - off[r]) B.st->ovf[d] = 1;
+      const int64_t len = round4(dg > dn ? dg : dn);
+      if (len > EDIT_SHORT) {
+        const int64_t c = cdiv(len, RW_CH);
+        long_chunks = (1ll << 32) | c;
+        scratch = c > 1 ? c : 0;
+      }
+    }
+    ca[j] = long_chunks;
+    cb[j] = scratch;
+  }
+}
+
+// ca, cb: exclusive prefixes of what k_edit_plan wrote, totals at [mr]
+__global__ void k_edit_lists(const __grid_constant__ EditBufs B, int d, int64_t mr, const int64_t* __restrict__ ca,
+                             const int64_t* __restrict__ cb) {
+  GRID_STRIDE(j, mr) {
+    if (ca[j + 1] == ca[j]) continue;
+    const int64_t at = ca[j] >> 32;
+    B.lrow[d][at] = (int32_t)j;
+    B.lpre[d][at] = (int32_t)(uint32_t)ca[j];
+    B.lsc[d][at] = (int32_t)cb[j];
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    EditStatus& st = *B.st;
+    st.nlong[d] = (int32_t)(ca[mr] >> 32);
+    st.chunks[d] = (int32_t)(uint32_t)ca[mr];
+    st.scratch[d] = (int32_t)cb[mr];
+    B.lpre[d][ca[mr] >> 32] = (int32_t)(uint32_t)ca[mr];
+    st.skip[d] = st.ovf[d];
+  }
+}
+
 int apply_batch_device(Graph* g, const int32_t* ds, const int32_t* dd, int64_t nd, const int32_t* is,
                        const int32_t* id, int64_t ni, bool validated) {
   cudaStream_t s = g->stream;
@@ -1380,11 +1353,11 @@ int apply_batch_device(Graph* g, const int32_t* ds, const int32_t* dd, int64_t n
   }
   if (nd) {
     note_launch(); k_make_keys<<<grid_for(nd, 256), 256, 0, s>>>(ds, dd, nd, g->perm, bits, dk);
-    TRY(radix_sort_u64(dk, alt, nd, 2 * bits, tmp, s));
+    TRY(radix_sort_u64(dk, alt, nd, 0, 2 * bits, tmp, s));
   }
   if (ni) {
     note_launch(); k_make_keys<<<grid_for(ni, 256), 256, 0, s>>>(is, id, ni, g->perm, bits, ik);
-    TRY(radix_sort_u64(ik, alt, ni, 2 * bits, tmp, s));
+    TRY(radix_sort_u64(ik, alt, ni, 0, 2 * bits, tmp, s));
   }
   int64_t* cnts = (int64_t*)(small + 1);
   TRY(cudaMemsetAsync(cnts, 0, 2 * sizeof(int64_t), s));
@@ -1403,50 +1376,97 @@ int apply_batch_device(Graph* g, const int32_t* ds, const int32_t* dd, int64_t n
   g->n_dplus = hc[1];
   if (hc[0] + hc[1] == 0) return OK;
 
-  // out-CSR: lists are sorted by (src, dst)
-  bool rep_out = false, rep_in = false;
-  int rc = edit_direction(g, &g->out, g->dmin, hc[0], g->dplus, hc[1], cnts + 1, &rep_out);
-  if (rc) return rc;
-  // in-CSR: the same lists keyed (dst, src)
-  {
-    int64_t a = hc[0], b = hc[1];
-    void* base2;
-    size_t need2;
-    {
-      Carve probe(nullptr);
-      probe.take<uint64_t>(a);
-      probe.take<uint64_t>(b);
-      probe.take<uint64_t>(a + b);
-      probe.take<char>((int64_t)radix_tmp_bytes(a + b));
-      need2 = probe.used + 4096;
+  // both directions: the lists (in-CSR: the same keyed (dst, src); the lists are
+  // sorted by (src, dst), so a stable sort by dst alone orders them), touched
+  // rows from a bitmap, plans, long rows
+  const int64_t a = hc[0], b = hc[1];
+  const int64_t mr = std::min<int64_t>(a + b, n);   // touched rows, at most
+  const int64_t tmp_bytes = (int64_t)std::max(radix_tmp_bytes(a + b), sizeof(int64_t) * (size_t)scan_tmp_elems(mr));
+  auto carve = [&](void* at, EditBufs* B, uint64_t** alt2, void** tmp2, uint32_t** rbits, int32_t** btmp, int64_t** ca,
+                   int64_t** cb, int32_t** cnt) {
+    Carve c(at);
+    B->key = nullptr;
+    B->dl[0] = g->dmin;
+    B->il[0] = g->dplus;
+    B->dl[1] = c.take<uint64_t>(a);
+    B->il[1] = c.take<uint64_t>(b);
+    *alt2 = c.take<uint64_t>(std::max(a, b));
+    *tmp2 = c.take<char>(tmp_bytes);
+    *rbits = c.take<uint32_t>(cdiv(n, 32) + 1);
+    *btmp = c.take<int32_t>(bits_to_list_tmp(n));
+    *ca = c.take<int64_t>(mr + 1);
+    *cb = c.take<int64_t>(mr + 1);
+    *cnt = c.take<int32_t>(2);
+    for (int d = 0; d < 2; d++) {
+      B->rows[d] = c.take<int32_t>(mr);
+      B->plan[d] = c.take<int4>(mr);
+      B->od[d] = c.take<int32_t>(mr);
+      B->lrow[d] = c.take<int32_t>(mr);
+      B->lpre[d] = c.take<int32_t>(mr + 1);
+      B->lsc[d] = c.take<int32_t>(mr);
     }
-    TRY(scratch_get(g, 1, need2, &base2));
-    Carve c2(base2);
-    uint64_t* sd = c2.take<uint64_t>(a);
-    uint64_t* si = c2.take<uint64_t>(b);
-    uint64_t* alt2 = c2.take<uint64_t>(a + b);
-    void* tmp2 = c2.take<char>((int64_t)radix_tmp_bytes(a + b));
-    if (a) {
-      note_launch(); k_swap_keys<<<grid_for(a, 256), 256, 0, s>>>(g->dmin, a, bits, sd);
-      TRY(radix_sort_u64(sd, alt2, a, 2 * bits, tmp2, s));
-    }
-    if (b) {
-      note_launch(); k_swap_keys<<<grid_for(b, 256), 256, 0, s>>>(g->dplus, b, bits, si);
-      TRY(radix_sort_u64(si, alt2, b, 2 * bits, tmp2, s));
-    }
-    rc = edit_direction(g, &g->in, sd, a, si, b, cnts + 1, &rep_in);
-    if (rc) return rc;
+    B->st = c.take<EditStatus>(1);
+    return c.used;
+  };
+  EditBufs B;
+  uint64_t* alt2;
+  void *tmp2, *ebase;
+  uint32_t* rbits;
+  int32_t *btmp, *rcnt;
+  int64_t *ca, *cb;
+  TRY(scratch_get(g, 1, carve(nullptr, &B, &alt2, &tmp2, &rbits, &btmp, &ca, &cb, &rcnt) + 256, &ebase));
+  carve(ebase, &B, &alt2, &tmp2, &rbits, &btmp, &ca, &cb, &rcnt);
+  if (a) {
+    note_launch(); k_swap_keys<<<grid_for(a, 256), 256, 0, s>>>(g->dmin, a, bits, B.dl[1]);
+    TRY(radix_sort_u64(B.dl[1], alt2, a, bits, 2 * bits, tmp2, s));
   }
-  if (rep_in) {
-    rc = refresh_full_tiles(g);
-    if (rc) return rc;
+  if (b) {
+    note_launch(); k_swap_keys<<<grid_for(b, 256), 256, 0, s>>>(g->dplus, b, bits, B.il[1]);
+    TRY(radix_sort_u64(B.il[1], alt2, b, bits, 2 * bits, tmp2, s));
   }
-  // contributions of sources whose out-degree changed (a3)
-  if (g->has_ranks) {
-    // the sources: reuse worklist 0 and the aux bitset
+  TRY(cudaMemsetAsync(B.st, 0, sizeof(EditStatus), s));
+  Csr* dirs[2] = {&g->out, &g->in};
+  for (int d = 0; d < 2; d++) {
+    const Csr* c = dirs[d];
+    TRY(cudaMemsetAsync(rbits, 0, sizeof(uint32_t) * (size_t)(cdiv(n, 32) + 1), s));
+    TRY(launch_source_bits(B.dl[d], a, bits, rbits, s));
+    TRY(launch_source_bits(B.il[d], b, bits, rbits, s));
+    TRY(launch_bits_to_list(rbits, nullptr, n, B.rows[d], rcnt, btmp, s));
+    note_launch();
+    k_edit_plan<<<grid_for(mr, 256), 256, 0, s>>>(B, d, rcnt, mr, a, b, bits, c->off, c->deg, ca, cb);
+    TRY(scan_excl<int64_t>(ca, ca, mr, (int64_t*)tmp2, s));
+    TRY(scan_excl<int64_t>(cb, cb, mr, (int64_t*)tmp2, s));
+    note_launch(); k_edit_lists<<<grid_for(mr, 256), 256, 0, s>>>(B, d, mr, ca, cb);
+  }
+  if (!g->small_h) TRY(cudaMallocHost(&g->small_h, sizeof(EditStatus)));
+  TRY(cudaMemcpyAsync(g->small_h, B.st, sizeof(EditStatus), cudaMemcpyDeviceToHost, s));
+  TRY(cudaStreamSynchronize(s));
+  const EditStatus h = *(EditStatus*)g->small_h;
+  int32_t* S[2] = {nullptr, nullptr};
+  int todo = 0;
+  for (int d = 0; d < 2; d++) {
+    if (h.ovf[d]) continue;
+    int64_t cap;
+    TRY(small_staging(g, d, (int64_t)h.scratch[d] * RW_CH, &S[d], &cap));
+    todo |= 1 << d;
+  }
+  if (todo) launch_edit(g, B, S, todo, 2 * mr);
+  TRY(cudaGetLastError());
+  for (int d = 0; d < 2; d++)
+    if (h.ovf[d]) {
+      int rc = repack_direction(g, dirs[d], B.dl[d], a, B.il[d], b);
+      if (rc) return rc;
+      if (d == 1) {
+        rc = refresh_full_tiles(g);
+        if (rc) return rc;
+      }
+    }
+  // contributions of sources whose out-degree changed (a3); the edit in place
+  // has refreshed them
+  if (h.ovf[0] && g->has_ranks) {
     TRY(cudaMemsetAsync(g->aux, 0, sizeof(uint32_t) * (size_t)(cdiv(n, 32) + 1), s));
     TRY(cudaMemsetAsync(&g->ctl->count[0], 0, sizeof(int32_t), s));
-    TRY(launch_mark_sources(g->dmin, hc[0], g->dplus, hc[1], bits, g->aux, g->wl[0], &g->ctl->count[0], s));
+    TRY(launch_mark_sources(g->dmin, a, g->dplus, b, bits, g->aux, g->wl[0], &g->ctl->count[0], s));
     TRY(launch_contrib_list(g->wl[0], &g->ctl->count[0], g->R, g->C[g->ccur], g->out.deg, g->tab_sc, n, s));
     TRY(cudaMemsetAsync(&g->ctl->count[0], 0, sizeof(int32_t), s));
   }

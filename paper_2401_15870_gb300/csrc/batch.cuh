@@ -12,10 +12,10 @@ int apply_batch_device(Graph* g, const int32_t* ds, const int32_t* dd, int64_t n
 // the host waits for any: a small batch (at most 16384 edges) is queued by
 // apply_batch_launch and finished by apply_batch_complete (which waits for the
 // graph's stream); a larger one is applied whole by apply_batch_launch.
-struct SmallStatus;
-struct SmallBufs;
+struct EditStatus;
+struct EditBufs;
 struct SmallApply {
-  SmallBufs* B = nullptr;   // set while a small batch is pending
+  EditBufs* B = nullptr;   // set while a small batch is pending
   int32_t* S[2] = {nullptr, nullptr};
 };
 // a host batch's endpoint arrays copied to the device, queued on the graph's

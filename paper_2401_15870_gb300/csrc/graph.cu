@@ -254,7 +254,7 @@ int build_graph_from_user_keys(Graph* g, uint64_t* keys, int64_t nkeys) {
   int64_t* cnt;
   TRY(t.get(&alt, nkeys));
   TRY(t.get((char**)&rtmp, radix_tmp_bytes(nkeys)));
-  TRY(radix_sort_u64(keys, alt, nkeys, 2 * bits, rtmp, s));
+  TRY(radix_sort_u64(keys, alt, nkeys, 0, 2 * bits, rtmp, s));
   TRY(t.get(&flag, nkeys));
   TRY(flag_unique_sorted(keys, nkeys, flag, s));
   ukeys = alt;   // alt is free again after the sort
@@ -278,7 +278,7 @@ int build_graph_from_user_keys(Graph* g, uint64_t* keys, int64_t nkeys) {
     TRY(t.get((char**)&vtmp, radix_tmp_bytes(n)));
     note_launch(); k_row_starts<<<grid_for(m, 256), 256, 0, s>>>(ukeys, m, bits, rowstart, n);
     note_launch(); k_relabel_keys<<<grid_for(n, 256), 256, 0, s>>>(rowstart, n, bits, vk);
-    TRY(radix_sort_u64(vk, vk_alt, n, 32 + bits, vtmp, s));
+    TRY(radix_sort_u64(vk, vk_alt, n, 0, 32 + bits, vtmp, s));
     note_launch(); k_perm_from_sorted<<<grid_for(n, 256), 256, 0, s>>>(vk, n, bits, g->perm, g->iperm);
   } else {
     TRY(iota_i32(g->perm, n, s));
@@ -289,12 +289,12 @@ int build_graph_from_user_keys(Graph* g, uint64_t* keys, int64_t nkeys) {
   {
     uint64_t* alt2;
     TRY(t.get(&alt2, m));
-    TRY(radix_sort_u64(keys, alt2, m, 2 * bits, rtmp, s));
+    TRY(radix_sort_u64(keys, alt2, m, 0, 2 * bits, rtmp, s));
     int rc = build_csr_from_sorted(g, &g->out, keys, m, false, 1);
     if (rc) return rc;
     // in-CSR: swapped keys
     note_launch(); k_remap_keys<<<grid_for(m, 256), 256, 0, s>>>(ukeys, m, bits, g->perm, true, keys);
-    TRY(radix_sort_u64(keys, alt2, m, 2 * bits, rtmp, s));
+    TRY(radix_sort_u64(keys, alt2, m, 0, 2 * bits, rtmp, s));
     rc = build_csr_from_sorted(g, &g->in, keys, m, true, 1);
     if (rc) return rc;
   }

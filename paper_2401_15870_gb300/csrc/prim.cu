@@ -262,8 +262,9 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const uint64_t* __res
   }
 }
 
-cudaError_t radix_sort_u64(uint64_t* keys, uint64_t* alt, int64_t n, int nbits, void* tmp, cudaStream_t s) {
-  if (n <= 1 || nbits <= 0) return cudaSuccess;
+cudaError_t radix_sort_u64(uint64_t* keys, uint64_t* alt, int64_t n, int lo_bit, int hi_bit, void* tmp,
+                           cudaStream_t s) {
+  if (n <= 1 || hi_bit <= lo_bit) return cudaSuccess;
   if (n >= (int64_t(1) << 31)) return cudaErrorInvalidValue;
   static std::once_flag smem_set;
   static cudaError_t smem_err = cudaSuccess;
@@ -277,7 +278,7 @@ cudaError_t radix_sort_u64(uint64_t* keys, uint64_t* alt, int64_t n, int nbits, 
   int32_t* scratch = counts + cnt + 1;
   uint64_t* src = keys;
   uint64_t* dst = alt;
-  for (int shift = 0; shift < nbits; shift += RS_BITS) {
+  for (int shift = lo_bit; shift < hi_bit; shift += RS_BITS) {
     note_launch(); k_rs_hist<<<(unsigned)ntiles, RS_THREADS, 0, s>>>(src, n, shift, counts, ntiles);
     cudaError_t e = scan_excl<int32_t>(counts, counts, cnt, scratch, s);
     if (e != cudaSuccess) return e;

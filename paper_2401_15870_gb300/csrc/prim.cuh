@@ -13,10 +13,10 @@ template <typename T>
 cudaError_t scan_excl(const T* in, T* out, int64_t n, T* tmp, cudaStream_t s);
 
 // ------------------------------------------------------------------ radix sort
-// Sorts keys[0..n) ascending on bits [0, nbits); alt is a same-size buffer.
-// The result ends in keys.  n < 2^31.  tmp: radix_tmp_bytes(n) bytes.
+// Sorts keys[0..n) ascending on bits [lo_bit, hi_bit), stable; alt is a
+// same-size buffer.  The result ends in keys.  n < 2^31.  tmp: radix_tmp_bytes(n) bytes.
 size_t radix_tmp_bytes(int64_t n);
-cudaError_t radix_sort_u64(uint64_t* keys, uint64_t* alt, int64_t n, int nbits, void* tmp, cudaStream_t s);
+cudaError_t radix_sort_u64(uint64_t* keys, uint64_t* alt, int64_t n, int lo_bit, int hi_bit, void* tmp, cudaStream_t s);
 
 // ------------------------------------------------------------------ compaction
 // out[0..c) = in[i] for which flag[i] != 0, in order; *count_dev = c.
