@@ -112,8 +112,8 @@ template <bool CLOSED, bool REL>
 __device__ __forceinline__ void row_update(const LoopParams& p, double alpha_fix, bool same_tau, long long sum,
                                            long long cself, double Rv, int32_t d, double sc, double2 ab, double& r,
                                            long long& c, unsigned long long& drb, bool& stay, bool& expand) {
-  if (CLOSED) r = fma(ab.x, (double)(sum - cself), ab.y);
-  else r = fma(alpha_fix, (double)sum, p.C0);
+  if (CLOSED) r = fma(ab.x, fixconv::i64_to_f64_rn(sum - cself), ab.y);
+  else r = fma(alpha_fix, fixconv::i64_to_f64_rn(sum), p.C0);
   drb = dbits(fabs(r - Rv));
   c = fixconv::f64_to_i64_rn(r * sc);
   const double mx = dbits(r) > dbits(Rv) ? r : Rv;

@@ -332,9 +332,9 @@ __device__ __forceinline__ void finish_pull_step(const P& p, long long* __restri
         // Eq. 2, the self term removed exactly in fixed point, as one FMA
         const long long K = sum[u] - cself[u];
         const double2 ab = d[u] < TAB ? p.tab_ab[d[u]] : closed_coeffs(p.alpha, p.n, d[u]);
-        r = fma(ab.x, (double)K, ab.y);
+        r = fma(ab.x, fixconv::i64_to_f64_rn(K), ab.y);
       } else {
-        r = fma(alpha_fix, (double)sum[u], p.C0);   // Eq. 1
+        r = fma(alpha_fix, fixconv::i64_to_f64_rn(sum[u]), p.C0);   // Eq. 1
       }
       const unsigned long long drb = dbits(fabs(r - Rv[u]));
       t.dmax = drb > t.dmax ? drb : t.dmax;

@@ -485,7 +485,7 @@ __global__ void __launch_bounds__(256, 4) k_finish_full(SweepParams p, long long
       const int64_t v = v0 + u * stride;
       if (v >= v_hi) continue;
       acc[v] = 0;
-      const double r = fma(alpha_fix, (double)sum[u], p.C0);   // Eq. 1
+      const double r = fma(alpha_fix, fixconv::i64_to_f64_rn(sum[u]), p.C0);   // Eq. 1
       const unsigned long long drb = dbits(fabs(r - Rv[u]));
       dmax = drb > dmax ? drb : dmax;
       edges += p.ideg[v];
@@ -533,7 +533,7 @@ __device__ __forceinline__ void finish_full_step(const SweepParams& p, long long
     const int64_t v = (ch0 + u) * 32 + lane;
     if (v >= p.n) continue;
     acc[v] = 0;
-    const double r = fma(alpha_fix, (double)sum[u], p.C0);   // Eq. 1
+    const double r = fma(alpha_fix, fixconv::i64_to_f64_rn(sum[u]), p.C0);   // Eq. 1
     const unsigned long long drb = dbits(fabs(r - Rv[u]));
     t.dmax = drb > t.dmax ? drb : t.dmax;
     t.edges += p.ideg[v];
