@@ -316,8 +316,8 @@ SweepParams dfpr::base_params(Graph* g, double alpha, double tau_f, double tau_p
   return p;
 }
 
-static ExpandParams expand_params(Graph* g, const int32_t* list, const int32_t* count, uint32_t* bits, uint32_t* ever,
-                                  int32_t* wl, int32_t* cnt) {
+static ExpandParams expand_params(Graph* g, const int32_t* list, const int32_t* count, uint32_t* bits, int32_t* wl,
+                                  int32_t* cnt) {
   ExpandParams e;
   memset(&e, 0, sizeof(e));
   e.n = g->n;
@@ -329,7 +329,6 @@ static ExpandParams expand_params(Graph* g, const int32_t* list, const int32_t* 
   e.tfirst = g->xtfirst;
   e.ntiles_dev = &g->ctl->xntiles;
   e.bits = bits;
-  e.ever = ever;
   e.wl = wl;
   e.cnt = cnt;
   e.id_bits = g->id_bits;
@@ -337,12 +336,12 @@ static ExpandParams expand_params(Graph* g, const int32_t* list, const int32_t* 
 }
 
 // expand the listed vertices' out-rows (expander tables)
-static pr_status run_expand(pr_graph* h, const int32_t* list, const int32_t* count, uint32_t* bits, uint32_t* ever,
-                            int32_t* wl, int32_t* cnt, const uint32_t* ins_src_bits) {
+static pr_status run_expand(pr_graph* h, const int32_t* list, const int32_t* count, uint32_t* bits, int32_t* wl,
+                            int32_t* cnt, const uint32_t* ins_src_bits) {
   Graph* g = &h->g;
   TRY(launch_list_scan(list, count, g->out.deg, g->n, g->xqs, g->xtfirst, &g->ctl->xqtot, &g->ctl->xntiles, h->ls_tmp,
                        g->stream));
-  ExpandParams e = expand_params(g, list, count, bits, ever, wl, cnt);
+  ExpandParams e = expand_params(g, list, count, bits, wl, cnt);
   e.ins_src_bits = ins_src_bits;
   e.dplus = g->dplus;
   e.n_dplus = g->n_dplus;
@@ -361,7 +360,7 @@ static pr_status initial_marking(pr_graph* h) {
   // sources of the effective change, each once
   TRY(launch_mark_sources(g->dmin, g->n_dmin, g->dplus, g->n_dplus, g->id_bits, g->aux, g->xl, &g->ctl->nexp, s));
   // G_t.out(u) for every source u ...
-  pr_status st = run_expand(h, g->xl, &g->ctl->nexp, g->bits[0], nullptr, g->wl[0], &g->ctl->count[0], nullptr);
+  pr_status st = run_expand(h, g->xl, &g->ctl->nexp, g->bits[0], g->wl[0], &g->ctl->count[0], nullptr);
   if (st != PR_OK) return st;
   // ... and the targets of deleted edges, which complete G_{t-1}.out(u)
   TRY(launch_mark_targets(g->dmin, g->n_dmin, g->id_bits, g->bits[0], nullptr, g->wl[0], &g->ctl->count[0], s));
@@ -383,7 +382,7 @@ static pr_status dt_affected(pr_graph* h) {
     TRY(launch_mark_sources(g->dmin, g->n_dmin, g->dplus, g->n_dplus, g->id_bits, vis, g->wl[0], &g->ctl->count[0], s));
     int c = 0;
     for (;;) {
-      pr_status st = run_expand(h, g->wl[c], &g->ctl->count[c], vis, nullptr, g->wl[1 - c], &g->ctl->count[1 - c],
+      pr_status st = run_expand(h, g->wl[c], &g->ctl->count[c], vis, g->wl[1 - c], &g->ctl->count[1 - c],
                                 which == 1 ? g->bits[1] : nullptr);
       if (st != PR_OK) return st;
       if (which == 1)
@@ -689,7 +688,7 @@ pr_status dfpr::run_update(pr_graph* h, int method, double alpha, double tau, do
         // edge volume picks the form of the next sweep
         TRY(launch_bits_to_list(g->bits[cur], nullptr, n, g->wl[cur], &g->ctl->count[cur], h->lbits_tmp, s));
         TRY(launch_bits_to_list(xb[cur], nullptr, n, g->xl, &g->ctl->nexp, h->lbits_tmp, s));
-        st = run_expand(h, g->xl, &g->ctl->nexp, g->bits[cur], nullptr, g->wl[cur], &g->ctl->count[cur], nullptr);
+        st = run_expand(h, g->xl, &g->ctl->nexp, g->bits[cur], g->wl[cur], &g->ctl->count[cur], nullptr);
         if (st != PR_OK) return st;
         TRY(cudaMemsetAsync(&g->ctl->nexp, 0, sizeof(int32_t), s));
         TRY(cudaMemsetAsync(g->bits[1 - cur], 0, wbytes, s));
@@ -712,7 +711,7 @@ pr_status dfpr::run_update(pr_graph* h, int method, double alpha, double tau, do
       p.xl = g->xl;
       p.cnt_x = &g->ctl->nexp;
       TRY(timer.launch(push_mode, p, s));
-      st = run_expand(h, g->xl, &g->ctl->nexp, g->bits[1 - cur], nullptr, g->wl[1 - cur], &g->ctl->count[1 - cur],
+      st = run_expand(h, g->xl, &g->ctl->nexp, g->bits[1 - cur], g->wl[1 - cur], &g->ctl->count[1 - cur],
                       nullptr);
       if (st != PR_OK) return st;
       TRY(launch_commit(g->wl[cur], &g->ctl->count[cur], g->rnew, g->R, g->C[g->ccur], g->out.deg, g->tab_sc,

@@ -188,7 +188,6 @@ struct ExpandParams {
   const int32_t* tfirst;
   const int64_t* ntiles_dev;
   uint32_t* bits;            // marks (test-and-set)
-  uint32_t* ever;            // nullable
   int32_t* wl;               // appended newly marked vertices
   int32_t* cnt;
   // previous-snapshot traversal (Dynamic Traversal on G_{t-1}): skip inserted edges
