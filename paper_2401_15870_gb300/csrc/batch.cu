@@ -126,11 +126,6 @@ __global__ void k_flag_ins(const uint64_t* __restrict__ ik, int64_t ni, const in
   }
 }
 
-__global__ void k_swap_keys(const uint64_t* __restrict__ in, int64_t k, int bits, uint64_t* __restrict__ out) {
-  uint64_t mask = (1ull << bits) - 1;
-  GRID_STRIDE(i, k) out[i] = ((in[i] & mask) << bits) | (in[i] >> bits);
-}
-
 constexpr int32_t REPACK_SHORT = 64;     // rows of at most this degree are rewritten by one thread
 constexpr int32_t REPACK_HUB = 16384;    // rows above this degree are spread over many blocks
 constexpr int64_t REPACK_CHUNK = 8192;   // elements of a hub row per block
@@ -1417,11 +1412,11 @@ int apply_batch_device(Graph* g, const int32_t* ds, const int32_t* dd, int64_t n
   TRY(scratch_get(g, 1, carve(nullptr, &B, &alt2, &tmp2, &rbits, &btmp, &ca, &cb, &rcnt) + 256, &ebase));
   carve(ebase, &B, &alt2, &tmp2, &rbits, &btmp, &ca, &cb, &rcnt);
   if (a) {
-    note_launch(); k_swap_keys<<<grid_for(a, 256), 256, 0, s>>>(g->dmin, a, bits, B.dl[1]);
+    TRY(swap_keys_u64(g->dmin, a, bits, B.dl[1], s));
     TRY(radix_sort_u64(B.dl[1], alt2, a, bits, 2 * bits, tmp2, s));
   }
   if (b) {
-    note_launch(); k_swap_keys<<<grid_for(b, 256), 256, 0, s>>>(g->dplus, b, bits, B.il[1]);
+    TRY(swap_keys_u64(g->dplus, b, bits, B.il[1], s));
     TRY(radix_sort_u64(B.il[1], alt2, b, bits, 2 * bits, tmp2, s));
   }
   TRY(cudaMemsetAsync(B.st, 0, sizeof(EditStatus), s));

@@ -118,14 +118,12 @@ __global__ void k_perm_from_sorted(const uint64_t* __restrict__ vk, int32_t n, i
   }
 }
 
-// keys_out[i] = (perm[u] << bits | perm[v]) or, if swap, (perm[v] << bits | perm[u])
+// keys_out[i] = perm[u] << bits | perm[v]
 __global__ void k_remap_keys(const uint64_t* __restrict__ in, int64_t m, int bits, const int32_t* __restrict__ perm,
-                             bool swap, uint64_t* __restrict__ out) {
+                             uint64_t* __restrict__ out) {
   uint64_t mask = (1ull << bits) - 1;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-    uint64_t u = (uint64_t)perm[in[i] >> bits], v = (uint64_t)perm[in[i] & mask];
-    out[i] = swap ? (v << bits | u) : (u << bits | v);
-  }
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x)
+    out[i] = (uint64_t)perm[in[i] >> bits] << bits | (uint64_t)perm[in[i] & mask];
 }
 
 // tile starts of the identity list over capacity quads
@@ -285,17 +283,17 @@ int build_graph_from_user_keys(Graph* g, uint64_t* keys, int64_t nkeys) {
     TRY(iota_i32(g->iperm, n, s));
   }
   // out-CSR on internal ids
-  note_launch(); k_remap_keys<<<grid_for(m, 256), 256, 0, s>>>(ukeys, m, bits, g->perm, false, keys);
+  note_launch(); k_remap_keys<<<grid_for(m, 256), 256, 0, s>>>(ukeys, m, bits, g->perm, keys);
   {
     uint64_t* alt2;
     TRY(t.get(&alt2, m));
     TRY(radix_sort_u64(keys, alt2, m, 0, 2 * bits, rtmp, s));
     int rc = build_csr_from_sorted(g, &g->out, keys, m, false, 1);
     if (rc) return rc;
-    // in-CSR: swapped keys
-    note_launch(); k_remap_keys<<<grid_for(m, 256), 256, 0, s>>>(ukeys, m, bits, g->perm, true, keys);
-    TRY(radix_sort_u64(keys, alt2, m, 0, 2 * bits, rtmp, s));
-    rc = build_csr_from_sorted(g, &g->in, keys, m, true, 1);
+    // in-CSR: the sorted edges exchanged, and a stable sort by target alone
+    TRY(swap_keys_u64(keys, m, bits, ukeys, s));
+    TRY(radix_sort_u64(ukeys, alt2, m, bits, 2 * bits, rtmp, s));
+    rc = build_csr_from_sorted(g, &g->in, ukeys, m, true, 1);
     if (rc) return rc;
   }
   TRY(cudaGetLastError());

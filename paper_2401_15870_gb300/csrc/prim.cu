@@ -149,8 +149,10 @@ constexpr int RS_WARPS = RS_THREADS / WARP;
 constexpr int RS_ITEMS = 16;
 constexpr int RS_KPW = WARP * RS_ITEMS;       // keys per warp
 constexpr int RS_TILE = RS_WARPS * RS_KPW;    // 8192 keys per tile
-// digits of RS_BITS bits: the 2 x 25-bit edge keys of a 2^25-vertex graph
-// take 5 passes instead of the 7 of 8-bit digits
+// digits of at most RS_BITS bits: the 2 x 25-bit edge keys of a 2^25-vertex
+// graph take 5 passes instead of the 7 of 8-bit digits.  A sort takes the
+// narrowest digits that need no more passes: the fewer digits, the longer the
+// runs of a tile's keys that go to one place (8 keys on average with 10 bits)
 constexpr int RS_BITS = 10;
 constexpr int RS_BINS = 1 << RS_BITS;
 
@@ -161,18 +163,26 @@ size_t radix_tmp_bytes(int64_t n) {
   return sizeof(int32_t) * (size_t)(cnt + 1 + scan_tmp_elems(cnt));
 }
 
-__global__ void __launch_bounds__(RS_THREADS) k_rs_hist(const uint64_t* __restrict__ keys, int64_t n, int shift,
-                                                        int32_t* __restrict__ counts, int64_t ntiles) {
+// (both kernels load a thread's RS_ITEMS keys before they use the first: one
+// memory latency per tile, not RS_ITEMS)
+__global__ void __launch_bounds__(RS_THREADS, 2) k_rs_hist(const uint64_t* __restrict__ keys, int64_t n, int shift, int bits,
+                                                           int32_t* __restrict__ counts, int64_t ntiles) {
   __shared__ int hist[RS_BINS];
-  for (int i = threadIdx.x; i < RS_BINS; i += RS_THREADS) hist[i] = 0;
-  __syncthreads();
-  int64_t base = (int64_t)blockIdx.x * RS_TILE;
-  for (int i = threadIdx.x; i < RS_TILE; i += RS_THREADS) {
-    int64_t j = base + i;
-    if (j < n) atomicAdd(&hist[(int)((keys[j] >> shift) & (RS_BINS - 1))], 1);
+  const int bins = 1 << bits;
+  const int64_t base = (int64_t)blockIdx.x * RS_TILE + threadIdx.x;
+  uint64_t k[RS_ITEMS];
+#pragma unroll
+  for (int i = 0; i < RS_ITEMS; i++) {
+    const int64_t j = base + (int64_t)i * RS_THREADS;
+    k[i] = j < n ? keys[j] : 0;
   }
+  for (int i = threadIdx.x; i < bins; i += RS_THREADS) hist[i] = 0;
   __syncthreads();
-  for (int d = threadIdx.x; d < RS_BINS; d += RS_THREADS) counts[(int64_t)d * ntiles + blockIdx.x] = hist[d];
+#pragma unroll
+  for (int i = 0; i < RS_ITEMS; i++)
+    if (base + (int64_t)i * RS_THREADS < n) atomicAdd(&hist[(int)((k[i] >> shift) & (bins - 1))], 1);
+  __syncthreads();
+  for (int d = threadIdx.x; d < bins; d += RS_THREADS) counts[(int64_t)d * ntiles + blockIdx.x] = hist[d];
 }
 
 // stable scatter: a warp owns a contiguous run of RS_KPW keys of the tile and
@@ -181,85 +191,119 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_hist(const uint64_t* __restri
 // its position among the tile's keys of its digit), then written out by
 // consecutive threads, so the keys of one digit leave as one coalesced run
 // instead of each warp's 32 keys going to up to 32 places.
-// dynamic shared memory of k_rs_scatter: the staged tile, the per-warp digit
-// counts and the digit starts
+// Dynamic shared memory: the staged tile, the per-warp digit counts (16 bits: a
+// tile holds 8192 keys) and two words per digit, 104 KB, so two blocks share an SM
+// (32-bit counts: 132 KB and one block).  A pass over 35.6M keys of 42 bits took
+// 336 us for the scatter and 91 for the counts with 10-bit digits, one block and
+// the loads one by one; 259 and 52 now (0.57 and 0.28 GB moved).  What is left is
+// instructions (60% of the issue slots: the ballots) and shared memory.
 constexpr size_t RS_STAGE_BYTES =
-    sizeof(uint64_t) * RS_TILE + sizeof(int) * (size_t)RS_WARPS * RS_BINS + sizeof(int) * (size_t)RS_BINS;
+    sizeof(uint64_t) * RS_TILE + sizeof(uint16_t) * (size_t)RS_WARPS * RS_BINS + 2 * sizeof(int) * (size_t)RS_BINS;
 
-__global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const uint64_t* __restrict__ keys, uint64_t* __restrict__ out,
-                                                           int64_t n, int shift, const int32_t* __restrict__ offs,
-                                                           int64_t ntiles) {
-  extern __shared__ uint64_t stage[];   // RS_TILE keys, then wcnt and dstart
-  int (*wcnt)[RS_BINS] = reinterpret_cast<int (*)[RS_BINS]>(stage + RS_TILE);
-  int* dstart = reinterpret_cast<int*>(stage + RS_TILE) + RS_WARPS * RS_BINS;   // first position of each digit
-  int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int i = threadIdx.x; i < RS_WARPS * RS_BINS; i += RS_THREADS) (&wcnt[0][0])[i] = 0;
-  __syncthreads();
+__global__ void __launch_bounds__(RS_THREADS, 2) k_rs_scatter(const uint64_t* __restrict__ keys, uint64_t* __restrict__ out,
+                                                              int64_t n, int shift, int bits,
+                                                              const int32_t* __restrict__ offs,
+                                                              int64_t ntiles) {
+  extern __shared__ uint64_t stage[];   // RS_TILE keys, then dstart, gofs and wcnt
+  int* dstart = reinterpret_cast<int*>(stage + RS_TILE);   // first position of each digit
+  int* gofs = dstart + RS_BINS;                            // its place in the output, less that position
+  uint16_t (*wcnt)[RS_BINS] = reinterpret_cast<uint16_t (*)[RS_BINS]>(gofs + RS_BINS);
+  __shared__ int wtot[RS_WARPS];
+  const int bins = 1 << bits;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t tile0 = (int64_t)blockIdx.x * RS_TILE;
-  int64_t base = tile0 + (int64_t)w * RS_KPW;
+  const int64_t base = tile0 + (int64_t)w * RS_KPW;
   uint64_t k[RS_ITEMS];
-  int rank[RS_ITEMS];
-  unsigned lt = lanemask_lt();
 #pragma unroll
   for (int i = 0; i < RS_ITEMS; i++) {
-    int64_t j = base + i * WARP + lane;
-    bool valid = j < n;
-    k[i] = valid ? keys[j] : 0;
-    int d = valid ? (int)((k[i] >> shift) & (RS_BINS - 1)) : RS_BINS;
-    unsigned peers = __match_any_sync(0xffffffffu, d);
-    int before = valid ? wcnt[w][d] : 0;
-    rank[i] = before + __popc(peers & lt);
-    __syncwarp();
-    if (valid && lane == __ffs(peers) - 1) wcnt[w][d] = before + __popc(peers);
-    __syncwarp();
+    const int64_t j = base + i * WARP + lane;
+    k[i] = j < n ? keys[j] : 0;
   }
-  __syncthreads();
-  // per digit: the warps' counts turned into offsets within the digit, and
-  // the digit's total
-  for (int d = threadIdx.x; d < RS_BINS; d += RS_THREADS) {
-    int run = 0;
-    for (int ww = 0; ww < RS_WARPS; ww++) {
-      int t = wcnt[ww][d];
-      wcnt[ww][d] = run;
-      run += t;
-    }
-    dstart[d] = run;
+  int32_t goff[2] = {0, 0};
+  if (2 * threadIdx.x < bins) {   // (bins: at least two)
+    goff[0] = offs[(int64_t)(2 * threadIdx.x) * ntiles + blockIdx.x];
+    goff[1] = offs[(int64_t)(2 * threadIdx.x + 1) * ntiles + blockIdx.x];
   }
+  for (int i = threadIdx.x; i < RS_WARPS * RS_BINS / 2; i += RS_THREADS) reinterpret_cast<uint32_t*>(wcnt)[i] = 0u;
   __syncthreads();
-  // exclusive scan of the digit totals by warp 0 (RS_BINS / 32 digits per lane)
-  if (w == 0) {
-    constexpr int PER = RS_BINS / WARP;
-    int sum = 0;
-    for (int q = 0; q < PER; q++) sum += dstart[lane * PER + q];
-    int incl = sum;
+  uint32_t rank[RS_ITEMS / 2] = {};   // two ranks of 16 bits each
+  const unsigned lt = lanemask_lt();
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int t = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += t;
+  for (int i = 0; i < RS_ITEMS; i++) {
+    const bool valid = base + i * WARP + lane < n;
+    const int d = (int)((k[i] >> shift) & (bins - 1));
+    // lanes of the same digit, from a ballot per bit (__match_any_sync takes
+    // longer than the ten of them)
+    unsigned peers = __ballot_sync(0xffffffffu, valid);
+#pragma unroll
+    for (int b = 0; b < RS_BITS; b++) {   // (bits past the digit's are zero in every lane)
+      const bool bit = (d >> b) & 1;
+      const unsigned m = __ballot_sync(0xffffffffu, bit);
+      peers &= bit ? m : ~m;
     }
-    int run = incl - sum;
-    for (int q = 0; q < PER; q++) {
-      const int v = dstart[lane * PER + q];
-      dstart[lane * PER + q] = run;
-      run += v;
-    }
+    const int before = valid ? wcnt[w][d] : 0;
+    rank[i / 2] |= (uint32_t)(before + __popc(peers & lt)) << (16 * (i & 1));
+    __syncwarp();
+    if (valid && lane == __ffs(peers) - 1) wcnt[w][d] = (uint16_t)(before + __popc(peers));
+    __syncwarp();
   }
+  __syncthreads();
+  // per digit (thread t: digits 2 t and 2 t + 1): the warps' counts turned into
+  // offsets within the digit, the totals into the digits' first positions, and
+  // the place of the tile's run of the digit in the output less that position
+  static_assert(RS_BINS == 2 * RS_THREADS, "two digits per thread");
+  int run[2] = {0, 0};
+  uint32_t* const col = reinterpret_cast<uint32_t*>(&wcnt[0][2 * threadIdx.x]);
+#pragma unroll
+  for (int ww = 0; ww < RS_WARPS; ww++) {
+    const uint32_t t = col[ww * (RS_BINS / 2)];
+    col[ww * (RS_BINS / 2)] = (uint32_t)run[0] | (uint32_t)run[1] << 16;
+    run[0] += (int)(t & 0xffffu);
+    run[1] += (int)(t >> 16);
+  }
+  int incl = run[0] + run[1];
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  if (lane == 31) wtot[w] = incl;
+  __syncthreads();
+  int first = incl - run[0] - run[1];
+  for (int ww = 0; ww < w; ww++) first += wtot[ww];
+  dstart[2 * threadIdx.x] = first;
+  dstart[2 * threadIdx.x + 1] = first + run[0];
+  gofs[2 * threadIdx.x] = goff[0] - first;
+  gofs[2 * threadIdx.x + 1] = goff[1] - first - run[0];
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < RS_ITEMS; i++) {
-    int64_t j = base + i * WARP + lane;
-    if (j < n) {
-      int d = (int)((k[i] >> shift) & (RS_BINS - 1));
-      stage[dstart[d] + wcnt[w][d] + rank[i]] = k[i];
+    if (base + i * WARP + lane < n) {
+      const int d = (int)((k[i] >> shift) & (bins - 1));
+      stage[dstart[d] + wcnt[w][d] + (rank[i / 2] >> (16 * (i & 1)) & 0xffffu)] = k[i];
     }
   }
   __syncthreads();
   const int valid_keys = (int)(n - tile0 < RS_TILE ? n - tile0 : RS_TILE);
+#pragma unroll 4
   for (int t = threadIdx.x; t < valid_keys; t += RS_THREADS) {
     const uint64_t key = stage[t];
-    const int d = (int)((key >> shift) & (RS_BINS - 1));
-    out[(int64_t)offs[(int64_t)d * ntiles + blockIdx.x] + (t - dstart[d])] = key;
+    const int d = (int)((key >> shift) & (bins - 1));
+    out[(int64_t)gofs[d] + t] = key;
   }
+}
+
+// packed pairs (a, b) as (b, a)
+__global__ void k_swap_keys(const uint64_t* __restrict__ in, int64_t n, int bits, uint64_t* __restrict__ out) {
+  const uint64_t mask = (1ull << bits) - 1;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    out[i] = ((in[i] & mask) << bits) | (in[i] >> bits);
+}
+
+cudaError_t swap_keys_u64(const uint64_t* in, int64_t n, int bits, uint64_t* out, cudaStream_t s) {
+  if (n == 0) return cudaSuccess;
+  note_launch(); k_swap_keys<<<grid_for(n, 256), 256, 0, s>>>(in, n, bits, out);
+  return cudaGetLastError();
 }
 
 cudaError_t radix_sort_u64(uint64_t* keys, uint64_t* alt, int64_t n, int lo_bit, int hi_bit, void* tmp,
@@ -273,16 +317,19 @@ cudaError_t radix_sort_u64(uint64_t* keys, uint64_t* alt, int64_t n, int lo_bit,
   });
   if (smem_err != cudaSuccess) return smem_err;
   int64_t ntiles = rs_tiles(n);
-  int64_t cnt = (int64_t)RS_BINS * ntiles;
+  const int passes = (hi_bit - lo_bit + RS_BITS - 1) / RS_BITS;
+  const int bits = (hi_bit - lo_bit + passes - 1) / passes;
+  const int64_t cnt = ((int64_t)1 << bits) * ntiles;
   int32_t* counts = (int32_t*)tmp;
-  int32_t* scratch = counts + cnt + 1;
+  int32_t* scratch = counts + (int64_t)RS_BINS * ntiles + 1;
   uint64_t* src = keys;
   uint64_t* dst = alt;
-  for (int shift = lo_bit; shift < hi_bit; shift += RS_BITS) {
-    note_launch(); k_rs_hist<<<(unsigned)ntiles, RS_THREADS, 0, s>>>(src, n, shift, counts, ntiles);
+  for (int p = 0; p < passes; p++) {
+    const int shift = lo_bit + p * bits;
+    note_launch(); k_rs_hist<<<(unsigned)ntiles, RS_THREADS, 0, s>>>(src, n, shift, bits, counts, ntiles);
     cudaError_t e = scan_excl<int32_t>(counts, counts, cnt, scratch, s);
     if (e != cudaSuccess) return e;
-    note_launch(); k_rs_scatter<<<(unsigned)ntiles, RS_THREADS, RS_STAGE_BYTES, s>>>(src, dst, n, shift, counts, ntiles);
+    note_launch(); k_rs_scatter<<<(unsigned)ntiles, RS_THREADS, RS_STAGE_BYTES, s>>>(src, dst, n, shift, bits, counts, ntiles);
     uint64_t* t = src;
     src = dst;
     dst = t;

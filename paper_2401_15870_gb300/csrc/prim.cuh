@@ -18,6 +18,10 @@ cudaError_t scan_excl(const T* in, T* out, int64_t n, T* tmp, cudaStream_t s);
 size_t radix_tmp_bytes(int64_t n);
 cudaError_t radix_sort_u64(uint64_t* keys, uint64_t* alt, int64_t n, int lo_bit, int hi_bit, void* tmp, cudaStream_t s);
 
+// out[i] = in[i] with its two `bits`-bit halves exchanged: pairs sorted by
+// (a, b), exchanged and sorted by their new high half, are sorted by (b, a)
+cudaError_t swap_keys_u64(const uint64_t* in, int64_t n, int bits, uint64_t* out, cudaStream_t s);
+
 // ------------------------------------------------------------------ compaction
 // out[0..c) = in[i] for which flag[i] != 0, in order; *count_dev = c.
 // tmp: compact_tmp_bytes(n) bytes.
