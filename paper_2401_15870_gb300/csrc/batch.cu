@@ -421,6 +421,7 @@ struct dfpr::EditBufs {
   // chunks before
   int32_t *lrow[2], *lpre[2], *lsc[2];
   EditStatus* st;
+  EditStatus* st_h;          // small batches: the pinned host copy the ingest writes
   uint64_t* key;             // small batches: packed (src, dst, insertion, present)
 };
 
@@ -942,6 +943,7 @@ __global__ void __launch_bounds__(SMALL_THREADS, 1)
       st.bad = 1;
       st.nr[dir] = st.nlong[dir] = st.chunks[dir] = st.scratch[dir] = 0;
       st.skip[dir] = 1;
+      *(volatile int32_t*)&B.st_h->bad = 1;
     }
     return;
   }
@@ -1046,6 +1048,14 @@ __global__ void __launch_bounds__(SMALL_THREADS, 1)
     st.ovf[dir] = any_ovf ? 1 : 0;
     st.need[dir] = (int64_t)scratch * RW_CH > c.scap ? 1 : 0;
     st.skip[dir] = st.ovf[dir] | st.need[dir];
+    // the same to the host, which a copy engine after the edit would reach
+    // about 10 us later
+    volatile EditStatus& h = *B.st_h;
+    h.n_del = nde;
+    h.n_ins = nie;
+    h.skip[dir] = st.skip[dir];
+    h.ovf[dir] = st.ovf[dir];
+    h.scratch[dir] = scratch;
   }
 }
 
@@ -1103,6 +1113,8 @@ static int small_launch(Graph* g, const int32_t* ds, const int32_t* dd, int64_t 
   TRY(scratch_get(g, 6, small_carve(nullptr, cap, &B) + 256, &bp));
   small_carve(bp, cap, &B);
   if (!g->small_h) TRY(cudaMallocHost(&g->small_h, sizeof(EditStatus)));
+  B.st_h = (EditStatus*)g->small_h;
+  B.st_h->bad = 0;
   TRY(grow_delta(g, &g->dmin, &g->cap_dmin, g->n_dmin, nd));
   TRY(grow_delta(g, &g->dplus, &g->cap_dplus, g->n_dplus, ni));
   B.dl[0] = g->dmin;
@@ -1129,7 +1141,6 @@ static int small_launch(Graph* g, const int32_t* ds, const int32_t* dd, int64_t 
     launch_edit(g, B, A->S, 3, 2 * (int64_t)N);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(g->small_h, B.st, sizeof(EditStatus), cudaMemcpyDeviceToHost, s);
   if (e != cudaSuccess) {
     delete A->B;
     A->B = nullptr;
@@ -1189,34 +1200,32 @@ static int small_complete(Graph* g, SmallApply* A) {
   return OK;
 }
 
-// the endpoint arrays of a host batch on the device (scratch slot 0): deletion
+// the endpoint arrays of a host batch where the device can read them: deletion
 // sources and targets, insertion sources and targets, one after another.  A
-// small batch goes through the graph's pinned buffer in one copy: four copies
-// from pageable memory take about 8 us of host time each.
+// small batch's are read once, by k_small_keys, straight from the graph's
+// pinned buffer; a larger one's are copied (scratch slot 0).
 int stage_host_batch(Graph* g, const int32_t* ds, const int32_t* dd, int64_t nd, const int32_t* is, const int32_t* id,
                      int64_t ni, int32_t** out) {
   cudaStream_t s = g->stream;
-  void* stage;
-  TRY(scratch_get(g, 0, sizeof(int32_t) * (size_t)(2 * (nd + ni) + 4) + 1024, &stage));
-  int32_t* b = (int32_t*)stage;
-  *out = b;
   const int32_t* src[4] = {ds, dd, is, id};
   const int64_t len[4] = {nd, nd, ni, ni};
   if (nd + ni <= SMALL_MAX) {
     if (!g->stage_h) TRY(cudaMallocHost(&g->stage_h, sizeof(int32_t) * 2 * SMALL_MAX));
-    if (g->stage_busy) TRY(cudaDeviceSynchronize());   // the copy of a call that failed after it
+    if (g->stage_busy) TRY(cudaDeviceSynchronize());   // the read of a call that failed after it
     int32_t* h = (int32_t*)g->stage_h;
+    *out = h;
+    g->stage_busy = nd + ni > 0;
     for (int k = 0; k < 4; k++)
       if (len[k]) {
         memcpy(h, src[k], sizeof(int32_t) * (size_t)len[k]);
         h += len[k];
       }
-    if (nd + ni > 0) {
-      g->stage_busy = true;
-      TRY(cudaMemcpyAsync(b, g->stage_h, sizeof(int32_t) * 2 * (size_t)(nd + ni), cudaMemcpyHostToDevice, s));
-    }
     return OK;
   }
+  void* stage;
+  TRY(scratch_get(g, 0, sizeof(int32_t) * (size_t)(2 * (nd + ni) + 4) + 1024, &stage));
+  int32_t* b = (int32_t*)stage;
+  *out = b;
   for (int k = 0; k < 4; k++)
     if (len[k]) {
       TRY(cudaMemcpyAsync(b, src[k], sizeof(int32_t) * (size_t)len[k], cudaMemcpyHostToDevice, s));

@@ -98,7 +98,7 @@ struct Graph {
 
   Scratch scr[8];
   void* small_h = nullptr;  // pinned host copy of the small-batch status (batch.cu)
-  void* stage_h = nullptr;  // pinned endpoint arrays of a small host batch, and whether their copy may be under way
+  void* stage_h = nullptr;  // pinned endpoint arrays of a small host batch, and whether the device may be reading them
   bool stage_busy = false;
   std::vector<void*> allocs;
   std::string err;

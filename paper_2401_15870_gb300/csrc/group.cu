@@ -563,9 +563,9 @@ struct pr_group {
   cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
   // resident blocks per SM of the one-kernel loop [form][relative measure], 0 until asked
   int loop_bps[2][2] = {{0, 0}, {0, 0}};
-  // an update of one graph in the one-barrier loop (loop.cu): its barrier and
-  // outcome on the device, the outcome on the host, and whether the update in
-  // flight is one
+  // an update of one graph in the one-barrier loop (loop.cu): its barrier on the
+  // device, its outcome in pinned host memory, and whether the update in flight
+  // is one
   LoopState* d_loop = nullptr;
   LoopOut* h_loop = nullptr;
   bool loop_clean = false, one_barrier = false;
@@ -827,9 +827,9 @@ static cudaError_t launch_one_barrier(pr_group* q, Graph* g, pr_method method, d
   p.tab_sc = q->tab_sc;
   p.tab_ab = g->tab_ab;
   p.st = q->d_loop;
-  cudaError_t e = one_after_another(q, [&] { return launch_loop(g, p, s); });
-  if (e != cudaSuccess) return e;
-  return cudaMemcpyAsync(q->h_loop, &q->d_loop->out, sizeof(LoopOut), cudaMemcpyDeviceToHost, s);
+  p.out = q->h_loop;
+  q->h_loop->err = 0;
+  return one_after_another(q, [&] { return launch_loop(g, p, s); });
 }
 
 // the same kernels launched one by one, the loop condition read back after

@@ -75,19 +75,20 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long x)
 // an arrival counter plus a release word 2.1; a slot per block polled by 152
 // threads of every block (no atomics) 3.9 to 5.2, the polls contending for a
 // few L2 lines.
-__device__ __forceinline__ bool grid_wait(LoopState* st, unsigned long long target) {
+__device__ __forceinline__ bool grid_wait(LoopState* st, LoopOut* out, unsigned long long target) {
   fence_acq_rel();   // this block's writes before its arrival
   atomicAdd(&st->count, 1ull);
   long long spins = 0;
   bool good = true;
   while (ld_relaxed_u64(&st->count) < target) {
     spins++;
-    if ((spins & 255) == 0 && *(volatile int32_t*)&st->out.err) {
+    if ((spins & 255) == 0 && *(volatile int32_t*)&st->err) {
       good = false;
       break;
     }
     if (spins > LOOP_SPINS) {
-      atomicExch(&st->out.err, 1);
+      atomicExch(&st->err, 1);
+      *(volatile int32_t*)&out->err = 1;
       good = false;
       break;
     }
@@ -146,11 +147,11 @@ __global__ void __launch_bounds__(LT, 1) k_loop(const __grid_constant__ LoopPara
   const int NB = gridDim.x;
   const uint64_t pol_stream = policy_evict_first(), pol_keep = policy_evict_last();
   // barriers of the launches before (block 0 wrote it at the end of the last one)
-  unsigned long long k = ld_relaxed_u64(&st->out.barriers);
+  unsigned long long k = ld_relaxed_u64(&st->barriers);
   auto barrier = [&]() -> bool {
     __syncthreads();
     bool good = true;
-    if (tid == 0) good = grid_wait(st, (k + 1) * NB);
+    if (tid == 0) good = grid_wait(st, p.out, (k + 1) * NB);
     k++;
     return __syncthreads_and(good) != 0;
   };
@@ -416,7 +417,7 @@ __global__ void __launch_bounds__(LT, 1) k_loop(const __grid_constant__ LoopPara
       if (lane == 0) {
         if (blockIdx.x == 0) st_relaxed_u64(&st->dR[(it + 1) % 3], 0ull);
         if (m) atomicMax(&st->dR[it % 3], m);
-        good = grid_wait(st, (k + 1) * NB);
+        good = grid_wait(st, p.out, (k + 1) * NB);
         next_dR = ld_relaxed_u64(&st->dR[it % 3]);
         if (!REGS) red[LW] = next_dR;
       }
@@ -446,14 +447,14 @@ __global__ void __launch_bounds__(LT, 1) k_loop(const __grid_constant__ LoopPara
   if (tid < 3) {
     long long s = 0;
     for (int i = 0; i < LW; i++) s += tot[tid][i];
-    st->out.part[blockIdx.x][tid] = s;
+    p.out->part[blockIdx.x][tid] = s;
   }
   if (blockIdx.x == 0 && tid == 0) {
-    st->out.iter = it;
-    st->out.converged = conv;
-    st->out.cur = cur;
-    st->out.dR_last = dR;
-    st->out.barriers = k;
+    st->barriers = k;
+    p.out->iter = it;
+    p.out->converged = conv;
+    p.out->cur = cur;
+    p.out->dR_last = dR;
   }
 }
 

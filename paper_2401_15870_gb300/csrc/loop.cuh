@@ -7,20 +7,21 @@
 namespace dfpr {
 
 constexpr int LOOP_MAX_BLOCKS = 256;
-// what a launch leaves on the device: the barrier's counter (kept between
-// launches), and the outcome, copied to the host as one piece
+// the outcome of an update, written by the kernel to pinned host memory (a
+// copy engine after the kernel adds about 10 us)
 struct LoopOut {
   int32_t iter, converged, err, cur;
   unsigned long long dR_last;
-  unsigned long long barriers;                // grid barriers completed, over all launches
   long long part[LOOP_MAX_BLOCKS][3];         // per block: in-edges, vertices, vertices ever affected
 };
+// what a launch leaves on the device for the next one
 struct LoopState {
-  unsigned long long count;   // arrivals at the grid barrier, over all launches
+  unsigned long long count;      // arrivals at the grid barrier, over all launches
   unsigned long long pad0[15];
-  unsigned long long dR[3];   // L-inf change of an iteration (mod 3), the bits of a non-negative double
-  unsigned long long pad1[13];
-  LoopOut out;
+  unsigned long long dR[3];      // L-inf change of an iteration (mod 3), the bits of a non-negative double
+  unsigned long long barriers;   // grid barriers completed, over all launches
+  int32_t err;                   // 1: a wait ran out
+  int32_t pad1;
 };
 
 struct LoopParams {
@@ -43,6 +44,7 @@ struct LoopParams {
   const double* tab_sc;
   const double2* tab_ab;
   LoopState* st;
+  LoopOut* out;             // pinned host memory; err must be 0 on entry
   int32_t rows_cap, words_cap, staged;
   int32_t l1_hub;           // contributions of internal ids below it are kept in L1
 };
