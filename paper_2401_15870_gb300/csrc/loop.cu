@@ -5,7 +5,7 @@
 // microseconds, and the time of an update is the number of iterations times
 // the latency of one: launches (three kernels per iteration in the CUDA graph,
 // 18-21 us) or, in the group loop of group.cu, two grid barriers plus two
-// phases of dependent loads (12-13 us at 2^14 vertices; here 4.7, and 4.0 at
+// phases of dependent loads (12-13 us at 2^14 vertices; here 4.5, and 4.0 at
 // 2^10).  Of the 4 us the barrier is 1.6, the gather 0.6 and the epilogue 0.3
 // when measured alone; the rest is the flush of a block's writes and the first
 // misses after the L1 is invalidated.  Here every block owns a run of whole in-CSR rows, cut at equal
@@ -255,6 +255,7 @@ __global__ void __launch_bounds__(LT, 1) k_loop(const __grid_constant__ LoopPara
       int own[U];
       long long s[U];
       unsigned wb[U], x[U];
+      unsigned xv[REGS ? U : 1][4] = {};
 #pragma unroll
       for (int j = 0; j < U; j++) {
         const int w = wi + j * LW;
@@ -272,30 +273,41 @@ __global__ void __launch_bounds__(LT, 1) k_loop(const __grid_constant__ LoopPara
 #pragma unroll
         for (int e = 0; e < 4; e++) s[j] += a[e] == p.n ? 0ll : ld_weak_contrib(C + a[e], hub_end, pol_keep);
         x[j] = 0u;
-        if (FRONTIER && own[j] >= 0 && !(flag[own[j]] & 1))
+        // (REGS: the bytes are kept apart until every load of the step is under
+        // way; combined inside the branch they would be waited for there)
+        if (FRONTIER && own[j] >= 0 && !(flag[own[j]] & 1)) {
+          if (REGS) {
 #pragma unroll
-          for (int e = 0; e < 4; e++) x[j] |= a[e] == p.n ? 0u : ld_byte(X + a[e]);
+            for (int e = 0; e < 4; e++) xv[j][e] = a[e] == p.n ? 0u : ld_byte(X + a[e]);
+          } else {
+#pragma unroll
+            for (int e = 0; e < 4; e++) x[j] |= a[e] == p.n ? 0u : ld_byte(X + a[e]);
+          }
+        }
       }
+      if (REGS && FRONTIER)
+#pragma unroll
+        for (int j = 0; j < U; j++) x[j] = xv[j][0] | xv[j][1] | xv[j][2] | xv[j][3];
 #pragma unroll
       for (int j = 0; j < U; j++) {
         const int w = wi + j * LW;
         if (w >= nw) break;   // the same in every lane
         long long sum = s[j];
         const unsigned vm = __ballot_sync(0xffffffffu, own[j] >= 0);
-        const unsigned long long seg0 = (unsigned long long)(wb[j] | 1u | (vm ^ (vm << 1)));
+        const unsigned starts = wb[j] | 1u | (vm ^ (vm << 1));   // segment starts
+        const unsigned later = starts & ~upto;
+        const int end = later ? __ffs(later) - 1 : 32;       // this lane's row piece ends before it
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
           const long long os = __shfl_down_sync(0xffffffffu, sum, o);
-          if (lane + o < 32 && ((seg0 >> (lane + 1)) & ((1ull << o) - 1ull)) == 0) sum += os;
+          if (lane + o < end) sum += os;
         }
         unsigned any = 0u;
         if (FRONTIER) {
           const unsigned xm = __ballot_sync(0xffffffffu, x[j] != 0u);
-          const unsigned long long later = (seg0 >> (lane + 1)) << (lane + 1);
-          const int end = later ? __ffsll((long long)later) - 1 : 32;
-          any = (xm & (unsigned)(((1ull << end) - 1ull) & ~((1ull << lane) - 1ull))) != 0u;
+          any = (xm & (unsigned)((1ull << end) - (1ull << lane))) != 0u;
         }
-        if (own[j] >= 0 && ((seg0 >> lane) & 1ull)) {
+        if (own[j] >= 0 && ((starts >> lane) & 1u)) {
           if ((wb[j] >> lane) & 1u) {
             acc[own[j]] = sum;
             if (FRONTIER) accx[own[j]] = (uint8_t)any;
@@ -473,9 +485,9 @@ __global__ void k_loop_shares(const int64_t* __restrict__ off, int32_t n, int64_
 
 // default for a graph of fewer in-CSR slots (larger ones run the CUDA graph,
 // one launch pair and a control kernel per iteration).  Time per iteration here
-// and there, DF / ND from the previous ranks: 245K edges (2^14 vertices) 4.8
-// against 17.7 us, 1.0M 8.2 against 19, 2.0M 13.7 against 24, 4.1M 22 against
-// 32, 8.2M 41 against 49; with pruning at 8.2M edges 61 against 58 (the
+// and there, DF / ND from the previous ranks: 245K edges (2^14 vertices) 4.5
+// against 16.6 us, 1.0M 7.6 against 17.5, 2.0M 12 against 23, 4.1M 19 against
+// 30, 8.2M 40 against 45; with pruning at 8.2M edges 61 against 58 (the
 // expanded flags are bytes here, bits there)
 constexpr int64_t LOOP_SLOTS = 3ll << 20;
 
