@@ -550,16 +550,19 @@ struct pr_group {
   GState* h_state = nullptr;
   int64_t* h_pre = nullptr;
   // unit sizes (indices into GR_QPT and GR_STEPS / GR_FU), set by pr_group_set_tuning or
-  // pr_group_autotune
-  int qi = 1, fi = 2;
+  // pr_group_autotune (qi -1: not set, chosen for each update by gather_units)
+  int qi = -1, fi = 2;
   float tune_ms = 0.f;
   int32_t tune_trials = 0;
-  // one CUDA graph per epilogue form (index 1: DF-P), built on first use with
-  // the unit sizes of exec_q / exec_f
-  cudaGraph_t graph[2] = {nullptr, nullptr};
-  cudaGraphExec_t exec[2] = {nullptr, nullptr};
-  int exec_q[2] = {-1, -1}, exec_f[2] = {-1, -1}, exec_rel[2] = {-1, -1};
-  cudaGraphConditionalHandle cond[2] = {0, 0};
+  // one CUDA graph per epilogue form (odd index: DF-P), built on first use with
+  // the unit sizes of exec_q / exec_f.  Slots 2 and 3 are for updates of 32M
+  // slots or more whose gather unit was not set, so that updates of few and of
+  // many members in turn rebuild nothing
+  static constexpr int NEXEC = 4;
+  cudaGraph_t graph[NEXEC] = {};
+  cudaGraphExec_t exec[NEXEC] = {};
+  int exec_q[NEXEC] = {-1, -1, -1, -1}, exec_f[NEXEC] = {-1, -1, -1, -1}, exec_rel[NEXEC] = {-1, -1, -1, -1};
+  cudaGraphConditionalHandle cond[NEXEC] = {};
   cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
   // resident blocks per SM of the one-kernel loop [form][relative measure], 0 until asked
   int loop_bps[2][2] = {{0, 0}, {0, 0}};
@@ -575,12 +578,22 @@ struct pr_group {
   pr_method cur_method = PR_DFP;
 };
 
-static void drop_exec(pr_group* q, int k);
+static void drop_exec(pr_group* q, int x);
+
+// The gather unit of an update over `slots` in-CSR slots: four warp steps of
+// two quads per lane from 32M slots on, else one of four.  A DF-P update took
+// 26.8 against 27.5 ms at 480M edges, 11.36 against 11.78 at 189M, 3.90 against
+// 4.05 at 52M; 2.40 against 2.41 at 36M, 0.985 against 0.935 at 6M, where the
+// larger units leave warps without one.
+static int gather_units(const pr_group* q, int64_t slots) {
+  if (q->qi >= 0) return q->qi;
+  return slots >= (32ll << 20) ? 3 : 1;
+}
 
 static void group_free(pr_group* q) {
   if (!q) return;
   if (q->stream) cudaStreamSynchronize(q->stream);
-  for (int k = 0; k < 2; k++) drop_exec(q, k);
+  for (int x = 0; x < pr_group::NEXEC; x++) drop_exec(q, x);
   for (void* p : {(void*)q->d_run, (void*)q->d_desc, (void*)q->d_state, (void*)q->d_pre, (void*)q->tab_sc,
                   (void*)q->d_loop})
     if (p) cudaFree(p);
@@ -645,41 +658,41 @@ static const void* finish_fn(int k, int fi, bool rel) {
   }
 }
 
-static void drop_exec(pr_group* q, int k) {
-  if (q->exec[k]) cudaGraphExecDestroy(q->exec[k]);
-  if (q->graph[k]) cudaGraphDestroy(q->graph[k]);
-  q->exec[k] = nullptr;
-  q->graph[k] = nullptr;
-  q->exec_q[k] = q->exec_f[k] = q->exec_rel[k] = -1;
+static void drop_exec(pr_group* q, int x) {
+  if (q->exec[x]) cudaGraphExecDestroy(q->exec[x]);
+  if (q->graph[x]) cudaGraphDestroy(q->graph[x]);
+  q->exec[x] = nullptr;
+  q->graph[x] = nullptr;
+  q->exec_q[x] = q->exec_f[x] = q->exec_rel[x] = -1;
 }
 
-// init -> mark -> WHILE (gather -> finish -> control); k = 1 for the DF-P epilogue
-static cudaError_t build_exec(pr_group* q, int k, bool rel) {
+// init -> mark -> WHILE (gather -> finish -> control) into slot x; odd: the DF-P epilogue
+static cudaError_t build_exec(pr_group* q, int x, int qi, bool rel) {
   cudaError_t e;
-  cudaGraph_t& graph = q->graph[k];
+  cudaGraph_t& graph = q->graph[x];
   if ((e = cudaGraphCreate(&graph, 0)) != cudaSuccess) return e;
-  if ((e = cudaGraphConditionalHandleCreate(&q->cond[k], graph, 0, 0)) != cudaSuccess) return e;
-  const void* fin = finish_fn(k, q->fi, rel);
-  const void* gat = gather_fn(q->qi);
-  q->exec_q[k] = q->qi;
-  q->exec_f[k] = q->fi;
-  q->exec_rel[k] = rel ? 1 : 0;
+  if ((e = cudaGraphConditionalHandleCreate(&q->cond[x], graph, 0, 0)) != cudaSuccess) return e;
+  const void* fin = finish_fn(x & 1, q->fi, rel);
+  const void* gat = gather_fn(qi);
+  q->exec_q[x] = qi;
+  q->exec_f[x] = q->fi;
+  q->exec_rel[x] = rel ? 1 : 0;
   const int sms = num_sms();
   const size_t sm = prefix_bytes(q);
   const int g_init = sms * blocks_per_sm((const void*)k_g_init, GR_THREADS, sm);
   const int g_gather = sms * blocks_per_sm(gat, GR_THREADS, sm);
   const int g_finish = sms * blocks_per_sm(fin, GR_THREADS, sm);
   cudaGraphNode_t n_init, n_mark, n_loop, n_gather, n_finish, n_ctl;
-  void* a_init[] = {&q->d_run, &q->d_desc, &q->d_state, &q->cond[k]};
+  void* a_init[] = {&q->d_run, &q->d_desc, &q->d_state, &q->cond[x]};
   void* a_mark[] = {&q->d_run, &q->d_desc};
   void* a_gather[] = {&q->d_run, &q->d_desc, &q->d_state};
   void* a_finish[] = {&q->d_run, &q->d_desc, &q->d_state};
-  void* a_ctl[] = {&q->d_run, &q->d_state, &q->cond[k]};
+  void* a_ctl[] = {&q->d_run, &q->d_state, &q->cond[x]};
   if ((e = add_kernel(graph, &n_init, nullptr, 0, (const void*)k_g_init, g_init, a_init, sm)) != cudaSuccess) return e;
   if ((e = add_kernel(graph, &n_mark, &n_init, 1, (const void*)k_g_mark, g_init, a_mark, sm)) != cudaSuccess) return e;
   cudaGraphNodeParams cp = {};
   cp.type = cudaGraphNodeTypeConditional;
-  cp.conditional.handle = q->cond[k];
+  cp.conditional.handle = q->cond[x];
   cp.conditional.type = cudaGraphCondTypeWhile;
   cp.conditional.size = 1;
   if ((e = cudaGraphAddNode(&n_loop, graph, &n_mark, nullptr, 1, &cp)) != cudaSuccess) return e;
@@ -693,7 +706,7 @@ static cudaError_t build_exec(pr_group* q, int k, bool rel) {
   kp.blockDim = dim3(GR_THREADS);
   kp.kernelParams = a_ctl;
   if ((e = cudaGraphAddKernelNode(&n_ctl, body, &n_finish, 1, &kp)) != cudaSuccess) return e;
-  return cudaGraphInstantiate(&q->exec[k], graph, 0);
+  return cudaGraphInstantiate(&q->exec[x], graph, 0);
 }
 
 extern "C" {
@@ -835,11 +848,11 @@ static cudaError_t launch_one_barrier(pr_group* q, Graph* g, pr_method method, d
 // the same kernels launched one by one, the loop condition read back after
 // every iteration (PR_OPT_HOST_LOOP): for profilers that cannot see into a
 // CUDA graph with conditional nodes, and for drivers without them
-static cudaError_t host_loop(pr_group* q, int k, int32_t max_iter, bool rel) {
+static cudaError_t host_loop(pr_group* q, int k, int qi, int32_t max_iter, bool rel) {
   cudaStream_t s = q->stream;
   const int sms = num_sms();
   const void* fin = finish_fn(k, q->fi, rel);
-  const void* gat = gather_fn(q->qi);
+  const void* gat = gather_fn(qi);
   const size_t sm = prefix_bytes(q);
   const int g_init = sms * blocks_per_sm((const void*)k_g_init, GR_THREADS, sm);
   const int g_gather = sms * blocks_per_sm(gat, GR_THREADS, sm);
@@ -910,7 +923,8 @@ pr_status group_launch(pr_group* q, pr_method method, double alpha, double tau, 
                    ((o.flags & PR_OPT_ONE_KERNEL) || (loops_asked == 0 && loop_default(&q->graphs[mem[0]]->g)));
   const bool one =
       !q->one_barrier && ((o.flags & PR_OPT_ONE_KERNEL) || (loops_asked == 0 && slots < PR_ONE_KERNEL_SLOTS));
-  const int64_t gq = one ? 32 * LOOP_QPT : 32 * GR_QPT[q->qi] * GR_STEPS[q->qi];   // quads per gather unit
+  const int qi = gather_units(q, slots);
+  const int64_t gq = one ? 32 * LOOP_QPT : 32 * GR_QPT[qi] * GR_STEPS[qi];   // quads per gather unit
   const int64_t fu = one ? LOOP_FU : GR_FU[q->fi];                                 // chunks per epilogue unit
   int64_t* wpre = q->h_pre;
   int64_t* fpre = wpre + (G + 1);
@@ -1014,13 +1028,14 @@ pr_status group_launch(pr_group* q, pr_method method, double alpha, double tau, 
     }
   } else if (r.use_graph) {
     const int rel = r.metric == METRIC_RELATIVE ? 1 : 0;
-    if (q->exec[k] && (q->exec_q[k] != q->qi || q->exec_f[k] != q->fi || q->exec_rel[k] != rel)) drop_exec(q, k);
-    if (!q->exec[k] && build_exec(q, k, rel != 0) != cudaSuccess) {
+    const int x = k + (q->qi < 0 && qi == 3 ? 2 : 0);
+    if (q->exec[x] && (q->exec_q[x] != qi || q->exec_f[x] != q->fi || q->exec_rel[x] != rel)) drop_exec(q, x);
+    if (!q->exec[x] && build_exec(q, x, qi, rel != 0) != cudaSuccess) {
       cudaGetLastError();
       return PR_ECUDA;
     }
-    if (cudaGraphLaunch(q->exec[k], s) != cudaSuccess) return PR_ECUDA;
-  } else if (host_loop(q, k, o.max_iter, r.metric == METRIC_RELATIVE) != cudaSuccess) {
+    if (cudaGraphLaunch(q->exec[x], s) != cudaSuccess) return PR_ECUDA;
+  } else if (host_loop(q, k, qi, o.max_iter, r.metric == METRIC_RELATIVE) != cudaSuccess) {
     return PR_ECUDA;
   }
   if (cudaMemcpyAsync(q->h_state, q->d_state, sizeof(GState) * G, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
@@ -1122,8 +1137,11 @@ extern "C" {
 
 pr_status pr_group_get_tuning(const pr_group* q, pr_group_tuning* out) {
   if (!q || !out) return PR_EINVAL;
-  out->quads_per_lane = GR_QPT[q->qi];
-  out->steps_per_unit = GR_STEPS[q->qi];
+  int64_t slots = 0;   // an update of every graph
+  for (const pr_graph* h : q->graphs) slots += h->g.in.cap;
+  const int qi = gather_units(q, slots);
+  out->quads_per_lane = GR_QPT[qi];
+  out->steps_per_unit = GR_STEPS[qi];
   out->chunks_per_unit = GR_FU[q->fi];
   out->ms_update = q->tune_ms;
   out->candidates = q->tune_trials;
