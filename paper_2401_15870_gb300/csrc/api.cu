@@ -647,6 +647,8 @@ pr_status dfpr::run_update(pr_graph* h, int method, double alpha, double tau, do
     p.cnt_x = &g->ctl->nexp;
     p.close.tau = tau;
     p.close.dbar = dbar;
+    p.close.m = g->m;
+    p.close.n = n;
     p.close.push_below = (flags & PR_OPT_FORCE_PULL) ? -1.0 : PUSH_VERTEX_FRACTION * (double)n;
     for (int32_t it = 0; it < max_iter;) {
       if ((flags & PR_OPT_FORCE_PULL) ||

@@ -33,7 +33,8 @@ struct alignas(8) Ctl {
   int32_t nexp_last;            // expander count of the last finished iteration
   int32_t stop;                 // every-vertex sweeps: 1 the iteration converged, 2 it left a small frontier; sweeps
                                 // queued behind it return at once
-  int32_t pad;
+  int32_t decide;               // the next pull sweep looks the undecided rows' membership up first (k_decide)
+  int64_t stay_edges;           // in-edges of the vertices that stayed in this pull sweep
 };
 
 struct Scratch {

@@ -271,6 +271,7 @@ constexpr int FIN_U = 4;   // chunks per warp step of the epilogue: their loads 
 struct PullTotals {
   unsigned long long dmax = 0ull;   // max |r - R[v]| as the bits of a non-negative double
   long long edges = 0, verts = 0;
+  long long stay_edges = 0;         // in-edges of the members that stay
   long long ever_new = 0;           // vertices processed for the first time in this update
   int stays = 0, exps = 0;
 };
@@ -352,6 +353,7 @@ __device__ __forceinline__ void finish_pull_step(const P& p, long long* __restri
       const unsigned long long tp = SAME || same_tau ? tf : dbits(p.tau_p * mr);
       stay = !CLOSED || drb > tp;
       expand = drb > tf;
+      if (stay) t.stay_edges += din[u];
     } else if (valid[u] && !inplace) {
       p.Cnext[v] = cself[u];
     }

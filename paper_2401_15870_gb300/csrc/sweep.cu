@@ -56,9 +56,12 @@ __device__ __forceinline__ T block_incl_scan256(T x, T* total, T* wsum /* >= 8 *
   return x + add;
 }
 
-__device__ __forceinline__ void block_flush_stats(double dmax, long long edges, long long verts, Ctl* ctl) {
+__device__ __forceinline__ void block_flush_stats(double dmax, long long edges, long long verts, Ctl* ctl,
+                                                  long long stay_edges = 0) {
   __shared__ double s_d[SW_THREADS / WARP];
   __shared__ long long s_e[SW_THREADS / WARP], s_v[SW_THREADS / WARP];
+  stay_edges = warp_sum_ll(stay_edges);
+  if (stay_edges && (threadIdx.x & 31) == 0) atomicAdd((unsigned long long*)&ctl->stay_edges, (unsigned long long)stay_edges);
   dmax = warp_max(dmax);
   edges = warp_sum_ll(edges);
   verts = warp_sum_ll(verts);
@@ -89,6 +92,23 @@ __device__ __forceinline__ void block_flush_stats(double dmax, long long edges, 
 // reading one address past L1 would queue at its L2 slice)
 __device__ __forceinline__ bool stopped(const SweepParams& p) { return p.close.mode && p.ctl->stop; }
 
+// When a pull sweep runs k_decide first.  It pays where many rows must be looked
+// up (DECIDE_OUT: the in-edges outside the stay set, as a share) and most of them
+// soon meet an expanded source.  The latter is judged by the stay set's mean
+// in-degree against the graph's (DECIDE_DEG), which the epilogue has at hand: with
+// the default tolerances the stay and the expanded sets are the same, and
+// vertices of high in-degree mostly have many out-edges.  DF-P sweeps without and
+// with it, (share outside, degree ratio): R-MAT 25 (0.95, 5.5) 5.24 / 4.07 ms,
+// (0.07, 2.6) 3.77 / 3.80, DF there (0.22, 14) 3.94 / 4.04; R-MAT 23 (0.84, 2.4)
+// 1.20 / 1.00, (0.98, 1.1) 1.16 / 1.16; a stream graph of 2^23 vertices (0.94,
+// 1.3) 0.97 / 0.88, (0.96, 1.0) 0.97 / 0.98, (0.99, 0.8) 0.90 / 1.06.  Below
+// DECIDE_N vertices the expanded set's bits mostly hit L1 anyway: R-MAT 22 0.395 /
+// 0.334, 21 0.197 / 0.186, 20 0.096 / 0.099.
+constexpr double DECIDE_OUT = 0.3;
+constexpr double DECIDE_DEG = 1.25;
+constexpr int32_t DECIDE_N = 1 << 22;
+constexpr int DECIDE_STEPS = 4;   // (one or two: the same within 2%, slower where hits are few)
+
 // One warp: the control block is read whole, a word per lane, changed and
 // written back to the device and to the host's pinned copy (a copy engine
 // between two sweeps costs the stream about 10 us, this kernel 2).  In the
@@ -118,6 +138,9 @@ __global__ void __launch_bounds__(32, 1) k_close(Ctl* ctl, SweepClose c) {
       v.nexp = 0;
       if (!v.stop && c.push_below >= 0.0 && (double)v.count[1 - cur] + c.dbar * (double)v.nexp_last < c.push_below)
         v.stop = 2;
+      v.decide = (double)(c.m - v.stay_edges) > DECIDE_OUT * (double)c.m &&
+                 (double)v.stay_edges * (double)c.n > DECIDE_DEG * (double)c.m * (double)v.count[1 - cur];
+      v.stay_edges = 0;
     }
   }
   __syncwarp();
@@ -409,9 +432,11 @@ __global__ void __launch_bounds__(1024, QPT == 2 ? 2 : 1) k_gather_rows(const in
                                                       const int32_t* __restrict__ rowbase, int64_t nquads, int32_t sent,
                                                       long long* __restrict__ acc, uint32_t* __restrict__ anyb,
                                                       int32_t hub_k, int32_t hub_kx, const int64_t* __restrict__ ioff,
-                                                      int32_t v_lo, int32_t v_hi, const int32_t* stop) {
+                                                      int32_t v_lo, int32_t v_hi, const Ctl* ctl,
+                                                      const uint32_t* __restrict__ decided) {
   extern __shared__ __align__(16) unsigned char hub_smem[];
-  if (stop && *stop) return;
+  if (ctl && ctl->stop) return;
+  if (PULL && !NOX && decided && ctl->decide) S = decided;   // (decided only with ctl)
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const uint64_t pol_stream = policy_evict_first();
@@ -439,6 +464,62 @@ __global__ void __launch_bounds__(1024, QPT == 2 ? 2 : 1) k_gather_rows(const in
                                                    pol_keep, hub, qlo);
 }
 
+// Membership of the rows outside the stay set, ahead of a pull sweep.  A row
+// outside S is in the frontier if any of its sources expanded, and the gather
+// looks every one of them up: a second random access per in-edge, which evicts the
+// hub contributions from L1 (5.24 ms a sweep at R-MAT 25 where few rows stay,
+// against 3.4 without look-ups).  Here a row's sources are looked up only until
+// the first hit: the first four quads by one lane per row, then up to DECIDE_STEPS
+// x 32 quads by the warp; `anyb` takes the hits and `decided` the rows whose
+// membership is known (in S, hit, or walked to the end), for which the gather
+// looks nothing up.  Rows still open stay with the gather.  Bound by the latency of
+// the scattered row starts: about 0.2 ms for 16M open rows, 0.6 for 33M; with it
+// those sweeps take 4.07 ms.
+__global__ void __launch_bounds__(256) k_decide(SweepParams p, uint32_t* __restrict__ anyb,
+                                                uint32_t* __restrict__ decided) {
+  if (stopped(p) || !p.ctl->decide) return;
+  const int lane = threadIdx.x & 31;
+  const int64_t nchunks = ((int64_t)p.n + 31) / 32, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  const uint64_t pol = policy_evict_first();
+  const auto bit = [&](int32_t c) { return c == p.n ? 0u : (__ldg(p.X_cur + (c >> 5)) >> (c & 31)) & 1u; };
+  const auto any = [&](int4 c) { return bit(c.x) | bit(c.y) | bit(c.z) | bit(c.w); };
+  for (int64_t ch = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; ch < nchunks; ch += nw) {
+    const int64_t v = ch * 32 + lane;
+    const bool open = v < p.n && !((__ldg(p.S_cur + ch) >> lane) & 1u);
+    const int64_t q0 = open ? __ldg(p.ioff + v) >> 2 : 0;
+    const int nq = open ? (__ldg(p.ideg + v) + 3) >> 2 : 0;
+    unsigned hit = 0u;
+#pragma unroll
+    for (int k = 0; k < 4; k += 2) {   // (two quads: one 32-byte sector when aligned)
+      if (hit || k >= nq) continue;
+      const int4 a = ld_stream4(p.icol + 4 * (q0 + k), pol);
+      const int4 b = k + 1 < nq ? ld_stream4(p.icol + 4 * (q0 + k + 1), pol) : make_int4(p.n, p.n, p.n, p.n);
+      hit = any(a) | any(b);
+    }
+    bool known = hit || nq <= 4;
+    unsigned todo = __ballot_sync(0xffffffffu, !known);
+    while (todo) {
+      const int l = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const int64_t q = __shfl_sync(0xffffffffu, q0, l) + lane;
+      const int m = __shfl_sync(0xffffffffu, nq, l);
+      unsigned found = 0u;
+      int k = 4;
+      for (int st = 0; st < DECIDE_STEPS && k < m && !found; st++, k += 32)
+        found = __ballot_sync(0xffffffffu, k + lane < m && any(ld_stream4(p.icol + 4 * (q + k), pol)));
+      if (lane == l) {
+        hit = found;
+        known = found || k >= m;
+      }
+    }
+    const unsigned hits = __ballot_sync(0xffffffffu, hit != 0u), done = __ballot_sync(0xffffffffu, known);
+    if (lane == 0) {
+      if (hits) anyb[ch] = hits;   // (zero before every sweep)
+      decided[ch] = done;
+    }
+  }
+}
+
 // (the 32-vertex chunks [ch_lo, ch_hi); ch_lo a multiple of FIN_U)
 template <bool CLOSED, bool REL, bool SAME = false>
 __global__ void __launch_bounds__(256, 3) k_finish_pull(SweepParams p, long long* __restrict__ acc,
@@ -454,7 +535,7 @@ __global__ void __launch_bounds__(256, 3) k_finish_pull(SweepParams p, long long
     if (t.stays) atomicAdd(p.cnt_next, t.stays);
     if (t.exps) atomicAdd(p.cnt_x, t.exps);
   }
-  block_flush_stats(__longlong_as_double((long long)t.dmax), t.edges, t.verts, p.ctl);
+  block_flush_stats(__longlong_as_double((long long)t.dmax), t.edges, t.verts, p.ctl, t.stay_edges);
 }
 
 // Epilogue of a sweep over every vertex with Eq. 1 (Static, ND): all vertices
@@ -701,7 +782,7 @@ static cudaError_t sweep_rows_dispatch(const SweepParams& p, const GatherCfg& cf
 template <bool PULL, int QPT, bool HUB>
 static cudaError_t gather_launch(const SweepParams& p, const uint32_t* rowbits, const int32_t* rowbase, uint32_t* anyb,
                                  int64_t nquads, int threads, int32_t hub_k, int32_t hub_kx, int32_t v_lo, int32_t v_hi,
-                                 bool one_wave, cudaStream_t s) {
+                                 bool one_wave, const uint32_t* decided, cudaStream_t s) {
   const auto kernel = PULL && !p.X_cur ? k_gather_rows<PULL, QPT, HUB, PULL> : k_gather_rows<PULL, QPT, HUB, false>;
   const void* fn = (const void*)kernel;
   const size_t smem = HUB ? gather_hub_bytes(hub_k, hub_kx) : 0;
@@ -721,26 +802,26 @@ static cudaError_t gather_launch(const SweepParams& p, const uint32_t* rowbits, 
   note_launch();
   kernel<<<grid, threads, smem, s>>>(p.icol, p.Ccur, PULL ? p.X_cur : nullptr, PULL ? p.S_cur : nullptr, rowbits,
                                      rowbase, nquads, p.n, p.gacc, anyb, hub_k, hub_kx, p.ioff, v_lo, v_hi,
-                                     p.close.mode ? &p.ctl->stop : nullptr);
+                                     p.close.mode ? p.ctl : nullptr, decided);
   return cudaGetLastError();
 }
 
 template <bool PULL>
 static cudaError_t gather_dispatch(const SweepParams& p, const GatherCfg& cfg, const uint32_t* rowbits,
                                    const int32_t* rowbase, uint32_t* anyb, int64_t nquads, int32_t v_lo, int32_t v_hi,
-                                   cudaStream_t s) {
+                                   cudaStream_t s, const uint32_t* decided = nullptr) {
   const bool ow = cfg.parts > 1;
   const int32_t hub_k = std::min<int32_t>(cfg.hub, p.n + 1);
   const int32_t hub_kx = PULL && p.X_cur ? (int32_t)cdiv(std::min<int32_t>(hub_k, p.n), 32) : 0;
   const bool hub = hub_k > 0;
   const int t = cfg.threads;
   switch (cfg.qpt * 2 + (hub ? 1 : 0)) {
-    case 4: return gather_launch<PULL, 2, false>(p, rowbits, rowbase, anyb, nquads, t, 0, 0, v_lo, v_hi, ow, s);
-    case 5: return gather_launch<PULL, 2, true>(p, rowbits, rowbase, anyb, nquads, t, hub_k, hub_kx, v_lo, v_hi, ow, s);
-    case 8: return gather_launch<PULL, 4, false>(p, rowbits, rowbase, anyb, nquads, t, 0, 0, v_lo, v_hi, ow, s);
-    case 9: return gather_launch<PULL, 4, true>(p, rowbits, rowbase, anyb, nquads, t, hub_k, hub_kx, v_lo, v_hi, ow, s);
-    case 16: return gather_launch<PULL, 8, false>(p, rowbits, rowbase, anyb, nquads, t, 0, 0, v_lo, v_hi, ow, s);
-    case 17: return gather_launch<PULL, 8, true>(p, rowbits, rowbase, anyb, nquads, t, hub_k, hub_kx, v_lo, v_hi, ow, s);
+    case 4: return gather_launch<PULL, 2, false>(p, rowbits, rowbase, anyb, nquads, t, 0, 0, v_lo, v_hi, ow, decided, s);
+    case 5: return gather_launch<PULL, 2, true>(p, rowbits, rowbase, anyb, nquads, t, hub_k, hub_kx, v_lo, v_hi, ow, decided, s);
+    case 8: return gather_launch<PULL, 4, false>(p, rowbits, rowbase, anyb, nquads, t, 0, 0, v_lo, v_hi, ow, decided, s);
+    case 9: return gather_launch<PULL, 4, true>(p, rowbits, rowbase, anyb, nquads, t, hub_k, hub_kx, v_lo, v_hi, ow, decided, s);
+    case 16: return gather_launch<PULL, 8, false>(p, rowbits, rowbase, anyb, nquads, t, 0, 0, v_lo, v_hi, ow, decided, s);
+    case 17: return gather_launch<PULL, 8, true>(p, rowbits, rowbase, anyb, nquads, t, hub_k, hub_kx, v_lo, v_hi, ow, decided, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -873,6 +954,15 @@ cudaError_t launch_full_sweep(int mode, const SweepParams& p, const GatherCfg& c
                         : ((aux && cfg.parts > 1 && p.n >= 128 * cfg.parts) ? cfg.parts : 1);
   if (ordered) aux = nullptr;
   cudaStream_t fs = P > 1 && !ordered ? aux->stream : s;
+  const uint32_t* decided = nullptr;
+  if (pull && !ordered && P == 1 && p.X_cur && p.close.mode == 2 && p.n >= DECIDE_N) {
+    int bps = 1;
+    const cudaError_t e = gather_occupancy((const void*)k_decide, 256, 0, &bps);
+    if (e != cudaSuccess) return e;
+    note_launch();
+    k_decide<<<(int)std::min<int64_t>(grid_for(p.n, 256), (int64_t)num_sms() * bps), 256, 0, s>>>(p, anyb, p.S_next);
+    decided = p.S_next;   // free until the epilogue writes it
+  }
   for (int k = 0; k < P; k++) {
     // the asynchronous order's ranges hold equal shares of the in-edges;
     // ranges overlapping gather and epilogue are cut by vertex count
@@ -880,7 +970,7 @@ cudaError_t launch_full_sweep(int mode, const SweepParams& p, const GatherCfg& c
     const int32_t v_hi = ordered && bounds ? bounds[k + 1]
                                            : (k + 1 == P ? p.n : (int32_t)((int64_t)p.n * (k + 1) / P / 128 * 128));
     if (ordered && v_hi <= v_lo) continue;   // an empty range (a hub range holding several shares)
-    cudaError_t e = pull ? gather_dispatch<true>(p, cfg, rowbits, rowbase, anyb, nquads, v_lo, v_hi, s)
+    cudaError_t e = pull ? gather_dispatch<true>(p, cfg, rowbits, rowbase, anyb, nquads, v_lo, v_hi, s, decided)
                          : gather_dispatch<false>(p, cfg, rowbits, rowbase, anyb, nquads, v_lo, v_hi, s);
     if (e != cudaSuccess) return e;
     if (P > 1 && !ordered) {

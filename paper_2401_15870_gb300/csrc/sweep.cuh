@@ -55,6 +55,8 @@ struct SweepClose {
   double tau;          // stop = 1 when the change is at most tau
   double dbar;         // mean degree, and the frontier size below which a pull
   double push_below;   // sweep hands over to lists (stop = 2; negative: never)
+  int64_t m;           // edges and vertices of the graph
+  int32_t n;
   Ctl* snap;           // pinned host copy of the control block, written by the device
 };
 
