@@ -143,7 +143,7 @@ struct GatherSpan {
 // bits are loaded.  The loads then wait for the S word, which costs sweeps whose
 // frontier holds nearly every edge about as much as it saves them (0.161 against
 // 0.163 ms at 97% of 34M edges) and halves one that holds 46% of 1.08e9 (4.36 ->
-// 2.37 ms).
+// 2.16 ms).
 template <bool PULL, int QPT = SW_QPT, bool HUB = false, bool SPAN = false, bool COH = false, bool NOX = false>
 __device__ __forceinline__ GatherSpan gather_step(const int32_t* __restrict__ icol, const long long* __restrict__ C,
                                                   const uint32_t* __restrict__ X, const uint32_t* __restrict__ S,
