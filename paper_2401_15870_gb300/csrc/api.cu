@@ -1,8 +1,10 @@
 // api.cu -- the C ABI of include/dfpr.h and the method drivers.
 //
 // pr_update drives the iterations of Alg. 1 (and of the comparators) from the
-// host: every iteration enqueues its kernels on the graph's stream and reads
-// back the 100-byte control block, which holds the iteration's L-inf change.
+// host (or hands a small graph to a device loop): every iteration enqueues its
+// kernels on the graph's stream and reads back the control block, which holds
+// the iteration's L-inf change; every-vertex sweeps are queued one ahead of it
+// (run_sweeps).
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
