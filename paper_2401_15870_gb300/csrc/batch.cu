@@ -18,6 +18,7 @@
 #include <cstring>
 #include <new>
 #include "batch.cuh"
+#include "edit_marks.cuh"
 #include "frontier.cuh"
 #include "prim.cuh"
 #include "sweep.cuh"
@@ -579,14 +580,15 @@ constexpr int EDIT_WARPS = 4;   // warps of a k_edit_long block
 __global__ void __launch_bounds__(EDIT_WARPS * 32) k_edit_long(const __grid_constant__ EditBufs B,
                                                                const __grid_constant__ EditArgs p, int bits) {
   __shared__ __align__(16) int32_t stage[EDIT_WARPS][RW_CH];
-  __shared__ int32_t delta[EDIT_WARPS][RW_CH + 1];   // change of the shift at an element, + DEAD where it is deleted
-  constexpr int32_t DEAD = 1 << 30;                  // (a row gets fewer than 2^29 insertions)
+  __shared__ int32_t delta[EDIT_WARPS][RW_CH + 1];     // edit_marks.cuh: change of the shift at an element
+  __shared__ uint32_t gone[EDIT_WARPS][RW_CH / 32];    // and whether it is deleted
   const EditStatus& st = *B.st;
   const int lane = threadIdx.x & 31;
   const int nw = gridDim.x * EDIT_WARPS;
   const uint64_t mask = (1ull << bits) - 1;
   int32_t* const T = stage[threadIdx.x >> 5];
   int32_t* const D = delta[threadIdx.x >> 5];
+  uint32_t* const dead = gone[threadIdx.x >> 5];
   const int e0 = (p.dirs & 1) && !st.skip[0] ? st.chunks[0] : 0;
   const int e1 = e0 + ((p.dirs & 2) && !st.skip[1] ? st.chunks[1] : 0);
   for (int w = blockIdx.x * EDIT_WARPS + (threadIdx.x >> 5); w < e1; w += nw) {
@@ -670,16 +672,16 @@ __global__ void __launch_bounds__(EDIT_WARPS * 32) k_edit_long(const __grid_cons
       }
     } else {
       for (int32_t i = lane; i <= no; i += 32) D[i] = 0;
+      if (lane < RW_CH / 32) dead[lane] = 0u;
       __syncwarp();
       for (int k = da + lane; k < db; k += 32) {
         const int32_t i = lower_i32(T, 0, no, (int32_t)(dl[k] & mask));   // its element (present)
-        atomicAdd(&D[i], DEAD);
-        atomicAdd(&D[i + 1], -1);
+        editmarks::mark_deleted(D, dead, i);
       }
       for (int k = ia + lane; k < ib; k += 32) {
         const int32_t y = (int32_t)(il[k] & mask);
         const int32_t i = lower_i32(T, 0, no, y);
-        atomicAdd(&D[i], 1);
+        editmarks::mark_inserted(D, i, 1);
         const int below = (int)(lower_key(dl, da, db, ((uint64_t)r << bits) | (uint64_t)y) - pl.x);
         const int32_t at = (k - pl.z) + x0 + i - below;
         if (at >= 0 && at < cap) row[at] = y;
@@ -687,9 +689,8 @@ __global__ void __launch_bounds__(EDIT_WARPS * 32) k_edit_long(const __grid_cons
       __syncwarp();
       int run = shift;
       for (int32_t b = 0; b < no; b += 32) {
-        const int32_t i = b + lane, m = i < no ? D[i] : 0;
-        const bool dead = m > DEAD / 2;
-        int sh = dead ? m - DEAD : m;
+        const int32_t i = b + lane;
+        int sh = i < no ? D[i] : 0;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
           const int y = __shfl_up_sync(0xffffffffu, sh, o);
@@ -699,7 +700,7 @@ __global__ void __launch_bounds__(EDIT_WARPS * 32) k_edit_long(const __grid_cons
         sh += run;
         run += all;
         const int32_t at = x0 + i + sh;
-        if (i < no && !dead && sh != 0 && at >= 0 && at < cap) row[at] = T[i];
+        if (i < no && !editmarks::is_deleted(dead, i) && sh != 0 && at >= 0 && at < cap) row[at] = T[i];
       }
     }
     for (int32_t x = x0 + lane; x < min(x0 + RW_CH, len); x += 32)
