@@ -275,9 +275,8 @@ __global__ void k_gather_f64(const double* __restrict__ in, const int32_t* __res
 // Ranks given in the caller's order: rank and contribution of every vertex in
 // one pass, read through iperm (the random side is an 8-byte load; R and C are
 // written in order).  Bound by the sectors of those loads: 28 us at 2.6M
-// vertices, 90 at 8.4M.  Once the vectors are larger than L2 a loaded sector is
-// gone before its other ranks are wanted, and scattering R through perm first
-// is the faster way: 374 against 413 us at 33.5M.
+// vertices.  For larger vectors R is scattered through perm first
+// (launch_import_ranks).
 __global__ void k_import_ranks(const double* __restrict__ in, const int32_t* __restrict__ iperm, double* __restrict__ R,
                                long long* __restrict__ C, const int32_t* __restrict__ odeg,
                                const double* __restrict__ tab_sc, int32_t n) {
@@ -312,7 +311,13 @@ cudaError_t launch_gather_f64(const double* in, const int32_t* idx, double* out,
   note_launch(); k_gather_f64<<<grid_for(n, 256), 256, 0, s>>>(in, idx, out, n);
   return cudaGetLastError();
 }
-constexpr int32_t IMPORT_SCATTER_N = 1 << 24;   // 134 MB per vector, against an L2 of 126 MB
+// From here on ranks are scattered through perm and the contributions made in a
+// second pass: a store does not wait for its sector, while the one-pass form's
+// loads do, and the more of them miss L2.  Below it the second launch costs more.
+// pr_set_ranks_device whole, one pass / two (us, R-MAT order): 2^16 vertices 33 /
+// 36, 2^20 50 / 53, 2^21 59 / 61, 2^22 95 / 90, 2^23 141 / 129, 2^24 246 / 230,
+// 33.5M 476 / 434; after a flush of L2 the same order at every size.
+constexpr int32_t IMPORT_SCATTER_N = 3 << 20;
 
 cudaError_t launch_import_ranks(const double* in, const int32_t* perm, const int32_t* iperm, double* R, long long* C,
                                 const int32_t* odeg, const double* tab_sc, int32_t n, cudaStream_t s) {
