@@ -1212,7 +1212,7 @@ static cudaError_t grow_delta(Graph* g, uint64_t** list, int64_t* cap, int64_t u
 template <int E>
 static cudaError_t launch_ingest(Graph* g, int N, const SmallCsr& out, const SmallCsr& in, const EditBufs& B) {
   int bps;   // (raises the kernel's shared memory limit once)
-  cudaError_t e = gather_occupancy((const void*)k_small_ingest<E>, SMALL_THREADS, small_smem<E>(), &bps);
+  cudaError_t e = kernel_occupancy((const void*)k_small_ingest<E>, SMALL_THREADS, small_smem<E>(), &bps);
   if (e != cudaSuccess) return e;
   note_launch();
   k_small_ingest<E><<<2, SMALL_THREADS, small_smem<E>(), g->stream>>>(N, g->id_bits, out, in, B);

@@ -555,7 +555,7 @@ cudaError_t launch_loop(const Graph* g, LoopParams p, cudaStream_t s) {
     default: fn = loop_kernel<false, false, true>(regs); break;                                               // Static, ND
   }
   int bps = 0;
-  cudaError_t e = gather_occupancy(fn, LT, l.bytes, &bps);   // also raises the kernel's shared memory limit
+  cudaError_t e = kernel_occupancy(fn, LT, l.bytes, &bps);   // also raises the kernel's shared memory limit
   if (e != cudaSuccess) return e;
   void* args[] = {&p};
   note_launch();

@@ -1,6 +1,6 @@
 // prim.cu -- scan, radix sort, compaction and fills (see prim.cuh).
 #include <atomic>
-#include <mutex>
+#include "kernel_limits.cuh"
 #include "prim.cuh"
 
 namespace dfpr {
@@ -38,6 +38,25 @@ int grid_for(int64_t n, int block) {
   int64_t want = cdiv(n > 0 ? n : 1, block);
   int64_t cap = (int64_t)num_sms() * 16;
   return (int)(want < cap ? want : cap);
+}
+
+namespace {
+struct CudaLimits {
+  using Error = cudaError_t;
+  static constexpr Error ok = cudaSuccess, does_not_fit = cudaErrorInvalidConfiguration;
+  static Error device(int* d) { return cudaGetDevice(d); }
+  static Error raise(const void* fn, size_t bytes) {
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  }
+  static Error blocks(int* b, const void* fn, int threads, size_t smem) {
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(b, fn, threads, smem);
+  }
+};
+}  // namespace
+
+cudaError_t kernel_occupancy(const void* fn, int threads, size_t smem, int* bps) {
+  static KernelLimits<CudaLimits> limits;
+  return limits.get(fn, threads, smem, bps);
 }
 
 // ================================================================== scan
@@ -310,12 +329,9 @@ cudaError_t radix_sort_u64(uint64_t* keys, uint64_t* alt, int64_t n, int lo_bit,
                            cudaStream_t s) {
   if (n <= 1 || hi_bit <= lo_bit) return cudaSuccess;
   if (n >= (int64_t(1) << 31)) return cudaErrorInvalidValue;
-  static std::once_flag smem_set;
-  static cudaError_t smem_err = cudaSuccess;
-  std::call_once(smem_set, [] {
-    smem_err = cudaFuncSetAttribute(k_rs_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RS_STAGE_BYTES);
-  });
-  if (smem_err != cudaSuccess) return smem_err;
+  int bps;   // (raises the kernel's shared memory limit)
+  const cudaError_t limit = kernel_occupancy((const void*)k_rs_scatter, RS_THREADS, RS_STAGE_BYTES, &bps);
+  if (limit != cudaSuccess) return limit;
   int64_t ntiles = rs_tiles(n);
   const int passes = (hi_bit - lo_bit + RS_BITS - 1) / RS_BITS;
   const int bits = (hi_bit - lo_bit + passes - 1) / passes;

@@ -41,4 +41,9 @@ cudaError_t iota_i32(int32_t* p, int64_t n, cudaStream_t s);
 int grid_for(int64_t n, int block);
 int num_sms();
 
+// resident blocks per SM of a kernel with `smem` bytes of dynamic shared memory
+// on the current device (an error when not even one fits); raises the kernel's
+// limit on that memory first where it is lower
+cudaError_t kernel_occupancy(const void* fn, int threads, size_t smem, int* bps);
+
 }  // namespace dfpr

@@ -18,9 +18,6 @@
 #include <algorithm>
 #include <vector>
 #include <climits>
-#include <map>
-#include <mutex>
-#include <tuple>
 #include "sweep.cuh"
 #include "pull_step.cuh"
 #include "fixconv.cuh"
@@ -751,7 +748,7 @@ static cudaError_t sweep_rows_launch(const SweepParams& p, const uint32_t* rowbi
   const void* fn = (const void*)k_sweep_rows<MODE, QPT, HUB>;
   const size_t smem = HUB ? gather_hub_bytes(hub_k, hub_kx) : 0;
   int bps = 1;
-  cudaError_t e = gather_occupancy(fn, threads, smem, &bps);
+  cudaError_t e = kernel_occupancy(fn, threads, smem, &bps);
   if (e != cudaSuccess) return e;
   const int64_t tasks = cdiv(p.ntiles_host, TASK_Q);
   const int64_t cap = (int64_t)num_sms() * bps;
@@ -787,7 +784,7 @@ static cudaError_t gather_launch(const SweepParams& p, const uint32_t* rowbits, 
   const void* fn = (const void*)kernel;
   const size_t smem = HUB ? gather_hub_bytes(hub_k, hub_kx) : 0;
   int bps = 1;
-  cudaError_t e = gather_occupancy(fn, threads, smem, &bps);
+  cudaError_t e = kernel_occupancy(fn, threads, smem, &bps);
   if (e != cudaSuccess) return e;
   // one wave of resident blocks when each block stages a hub cache, else up
   // to 64 blocks of 256 threads per SM (eight waves of 1024-thread blocks at
@@ -828,34 +825,6 @@ static cudaError_t gather_dispatch(const SweepParams& p, const GatherCfg& cfg, c
 
 size_t gather_hub_bytes(int32_t hub_k, int32_t hub_kx) {
   return sizeof(long long) * (size_t)hub_k + sizeof(uint32_t) * (size_t)hub_kx;
-}
-
-// resident blocks per SM of a gather kernel with `smem` bytes of dynamic
-// shared memory (raising the kernel's dynamic shared memory limit once)
-cudaError_t gather_occupancy(const void* fn, int threads, size_t smem, int* bps) {
-  static std::mutex mu;
-  static std::map<const void*, size_t> limit;
-  static std::map<std::tuple<const void*, int, size_t>, int> cache;
-  std::lock_guard<std::mutex> lock(mu);
-  auto key = std::make_tuple(fn, threads, smem);
-  auto it = cache.find(key);
-  if (it != cache.end()) {
-    *bps = it->second;
-    return cudaSuccess;
-  }
-  size_t& lim = limit[fn];
-  if (smem > lim) {
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    lim = smem;
-  }
-  int b = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, threads, smem);
-  if (e != cudaSuccess) return e;
-  if (b < 1) return cudaErrorInvalidConfiguration;
-  cache[key] = b;
-  *bps = b;
-  return cudaSuccess;
 }
 
 bool gather_cfg_valid(const GatherCfg& c) {
@@ -957,7 +926,7 @@ cudaError_t launch_full_sweep(int mode, const SweepParams& p, const GatherCfg& c
   const uint32_t* decided = nullptr;
   if (pull && !ordered && P == 1 && p.X_cur && p.close.mode == 2 && p.n >= DECIDE_N) {
     int bps = 1;
-    const cudaError_t e = gather_occupancy((const void*)k_decide, 256, 0, &bps);
+    const cudaError_t e = kernel_occupancy((const void*)k_decide, 256, 0, &bps);
     if (e != cudaSuccess) return e;
     note_launch();
     k_decide<<<(int)std::min<int64_t>(grid_for(p.n, 256), (int64_t)num_sms() * bps), 256, 0, s>>>(p, anyb, p.S_next);
@@ -988,7 +957,7 @@ cudaError_t launch_full_sweep(int mode, const SweepParams& p, const GatherCfg& c
                       : rel && p.tau_f == p.tau_p ? (const void*)k_finish_pull<true, true, true>
                       : rel                        ? (const void*)k_finish_pull<true, true>
                                                    : (const void*)k_finish_pull<true, false>;
-    if ((e = gather_occupancy(fin, 256, 0, &bps)) != cudaSuccess) return e;
+    if ((e = kernel_occupancy(fin, 256, 0, &bps)) != cudaSuccess) return e;
     const int rgrid = (int)std::min<int64_t>(grid_for(v_hi - v_lo, 256), (int64_t)num_sms() * bps);
     switch (mode) {
       case SWEEP_FULL: note_launch(); k_finish_full<<<rgrid, 256, 0, fs>>>(p, p.gacc, v_lo, v_hi); break;

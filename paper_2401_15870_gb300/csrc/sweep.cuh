@@ -134,7 +134,6 @@ struct SweepAux {
 constexpr int GATHER_SMEM_MAX = 227 * 1024;   // dynamic shared memory of one block on sm_103
 size_t gather_hub_bytes(int32_t hub_k, int32_t hub_kx);
 bool gather_cfg_valid(const GatherCfg& c);
-cudaError_t gather_occupancy(const void* fn, int threads, size_t smem, int* bps);
 // the gather alone: adds every row's sum to p.gacc (and, if pull, sets anyb)
 cudaError_t launch_gather(bool pull, const SweepParams& p, const GatherCfg& cfg, const uint32_t* rowbits,
                           const int32_t* rowbase, uint32_t* anyb, int64_t nquads, cudaStream_t s);
