@@ -128,6 +128,8 @@ typedef struct {
  * slots in all (one graph alone: fewer than three times as many, unless one
  * in-row holds most of them); PR_OPT_DEVICE_LOOP alone asks for the CUDA graph.  At most one
  * of PR_OPT_HOST_LOOP, PR_OPT_DEVICE_LOOP and PR_OPT_ONE_KERNEL may be set.
+ * Where the one-kernel loop of a single graph is refused (the process may not
+ * use every SM), the update runs as it would for more graphs of the same size.
  * The result is the same bit for bit.  A barrier wait gives up after about a
  * second (a block that never arrives); the update then returns PR_ETIMEOUT
  * and its graphs are left without ranks. */
@@ -565,6 +567,15 @@ pr_status pr_set_tuning(pr_graph* g, const pr_tuning* in);
  * the device.
  */
 void pr_debug_fail_alloc(int64_t k);
+
+/*
+ * Testing aid as above, for the one-kernel loop of a single graph
+ * (PR_OPT_ONE_KERNEL): its next launch in the process fails.  how = 1: it is
+ * refused, as a cooperative launch is when the process may not use every SM;
+ * the update then runs in the loop that it would take without it.  how = 0
+ * disarms.  Nothing is faulted on the device.
+ */
+void pr_debug_fail_loop(int32_t how);
 
 /* Number of CUDA kernels this library has launched in this process so far
  * (all graphs); the difference across a region counts its launches. */

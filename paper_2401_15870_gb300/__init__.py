@@ -139,6 +139,7 @@ def load():
         "pr_server_destroy": ([_P], None),
         "pr_autotune": ([_P, ctypes.c_int, f64, f64, i32, _P], ctypes.c_int),
         "pr_debug_fail_alloc": ([i64], None),
+        "pr_debug_fail_loop": ([i32], None),
         "pr_apply_batches_device": ([i32, _P, _P, _P, _P, _P, _P, _P], ctypes.c_int),
         "pr_apply_batches": ([i32, _P, _P, _P, _P, _P, _P, _P], ctypes.c_int),
         "pr_get_tuning": ([_P, _P], ctypes.c_int),
@@ -551,6 +552,11 @@ def pr_group_set_tuning(q, quads_per_lane=4, chunks_per_unit=4, steps_per_unit=1
 def pr_debug_fail_alloc(k):
     """Make the k-th device allocation of the library from now fail (0: disarm)."""
     load().pr_debug_fail_alloc(int(k))
+
+
+def pr_debug_fail_loop(how):
+    """Make the next launch of a single graph's one-kernel loop fail: 1, it is refused (0: disarm)."""
+    load().pr_debug_fail_loop(int(how))
 
 
 def pr_kernel_launches() -> int:

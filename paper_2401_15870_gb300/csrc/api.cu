@@ -18,6 +18,7 @@
 #include "frontier.cuh"
 #include "graph.cuh"
 #include "handle.cuh"
+#include "loop.cuh"
 #include "prim.cuh"
 #include "sweep.cuh"
 
@@ -1498,6 +1499,8 @@ unsigned long long pr_kernel_launches(void) { return launches_so_far(); }
 const char* pr_last_error(const pr_graph* h) { return h ? h->g.err.c_str() : ""; }
 
 void pr_debug_fail_alloc(int64_t k) { arm_alloc_failure(k); }
+
+void pr_debug_fail_loop(int32_t how) { arm_loop_failure(how); }
 
 const char* pr_status_string(pr_status s) {
   switch (s) {

@@ -880,10 +880,9 @@ static cudaError_t host_loop(pr_group* q, int k, int qi, int32_t max_iter, bool 
   return cudaGetLastError();
 }
 
-// launch an update of the members (indices into the group; NULL: every graph)
-// on the group's stream without waiting for it
-pr_status group_launch(pr_group* q, pr_method method, double alpha, double tau, const pr_options* opts,
-                       const int32_t* members, int32_t nm) {
+// group_launch; barrier_loop: the one-barrier loop may be taken
+static pr_status launch_update(pr_group* q, pr_method method, double alpha, double tau, const pr_options* opts,
+                               const int32_t* members, int32_t nm, bool barrier_loop) {
   if (!q || q->in_flight) return PR_EINVAL;
   if (method != PR_STATIC && method != PR_NAIVE_DYNAMIC && method != PR_DF && method != PR_DFP) return PR_EINVAL;
   if (!(alpha >= 0.0 && alpha < 1.0) || !(tau >= 0.0)) return PR_EINVAL;
@@ -919,7 +918,7 @@ pr_status group_launch(pr_group* q, pr_method method, double alpha, double tau, 
   for (int i = 0; i < G; i++) slots += q->graphs[mem[i]]->g.in.cap;
   // (one graph whose rows can be shared out to the blocks: the loop with one
   // barrier per iteration, whatever its size)
-  q->one_barrier = G == 1 && loop_fits(&q->graphs[mem[0]]->g) &&
+  q->one_barrier = barrier_loop && G == 1 && loop_fits(&q->graphs[mem[0]]->g) &&
                    ((o.flags & PR_OPT_ONE_KERNEL) || (loops_asked == 0 && loop_default(&q->graphs[mem[0]]->g)));
   const bool one =
       !q->one_barrier && ((o.flags & PR_OPT_ONE_KERNEL) || (loops_asked == 0 && slots < PR_ONE_KERNEL_SLOTS));
@@ -1007,8 +1006,10 @@ pr_status group_launch(pr_group* q, pr_method method, double alpha, double tau, 
   }
   if (q->one_barrier) {
     if (launch_one_barrier(q, &q->graphs[mem[0]]->g, method, alpha, tau, o, r.metric) != cudaSuccess) {
+      // a grid that needs every SM at once is refused where the process may not
+      // use them all: the loop that sizes below and above it take
       cudaGetLastError();
-      return PR_ECUDA;
+      return launch_update(q, method, alpha, tau, opts, members, nm, false);
     }
     if (cudaEventRecord(q->ev[1], s) != cudaSuccess) return PR_ECUDA;
     q->in_flight = true;
@@ -1045,6 +1046,13 @@ pr_status group_launch(pr_group* q, pr_method method, double alpha, double tau, 
   q->in_flight = true;
   q->cur_method = method;
   return PR_OK;
+}
+
+// launch an update of the members (indices into the group; NULL: every graph)
+// on the group's stream without waiting for it
+pr_status group_launch(pr_group* q, pr_method method, double alpha, double tau, const pr_options* opts,
+                       const int32_t* members, int32_t nm) {
+  return launch_update(q, method, alpha, tau, opts, members, nm, true);
 }
 
 // true when the launched update has finished (does not block)

@@ -24,6 +24,7 @@
 // the epilogue adds a row's start and its words.  Integer sums, so the order
 // does not change a bit: the ranks and statistics are those of the other loops.
 #include <algorithm>
+#include <atomic>
 #include "loop.cuh"
 #include "prim.cuh"
 #include "pull_step.cuh"
@@ -512,6 +513,9 @@ Layout layout(const Graph* g) {
 int loop_blocks() { return std::min(num_sms(), LOOP_MAX_BLOCKS); }
 size_t loop_state_bytes() { return sizeof(LoopState); }
 
+static std::atomic<int> g_loop_failure{0};   // of the next launch
+void arm_loop_failure(int how) { g_loop_failure.store(how == LOOP_REFUSED ? how : 0); }
+
 cudaError_t loop_reset(LoopState* st, cudaStream_t s) {
   return cudaMemsetAsync(st, 0, sizeof(*st), s);
 }
@@ -541,6 +545,8 @@ static const void* loop_kernel(bool regs) {
 }
 
 cudaError_t launch_loop(const Graph* g, LoopParams p, cudaStream_t s) {
+  const int fail = g_loop_failure.exchange(0);
+  if (fail == LOOP_REFUSED) return cudaErrorCooperativeLaunchTooLarge;
   const Layout l = layout(g);
   p.rows_cap = l.rows_cap;
   p.words_cap = l.words_cap;

@@ -59,6 +59,10 @@ cudaError_t loop_reset(LoopState* st, cudaStream_t s);
 // queue the update; p.rows_cap, words_cap and staged are filled in here
 cudaError_t launch_loop(const Graph* g, LoopParams p, cudaStream_t s);
 int loop_blocks();
+// the next launch fails (pr_debug_fail_loop): LOOP_REFUSED, the launch returns
+// cudaErrorCooperativeLaunchTooLarge and nothing is launched; 0 disarms
+enum LoopFailure : int { LOOP_REFUSED = 1 };
+void arm_loop_failure(int how);
 
 // the shares of the in-CSR's rows that loop_blocks() blocks get: writes
 // {largest rows, largest quads} of a block to out[0..1]
