@@ -572,8 +572,10 @@ void pr_debug_fail_alloc(int64_t k);
  * Testing aid as above, for the one-kernel loop of a single graph
  * (PR_OPT_ONE_KERNEL): its next launch in the process fails.  how = 1: it is
  * refused, as a cooperative launch is when the process may not use every SM;
- * the update then runs in the loop that it would take without it.  how = 0
- * disarms.  Nothing is faulted on the device.
+ * the update then runs in the loop that it would take without it.  how = 2: its
+ * first barrier waits for arrivals that never come, and gives up after some
+ * milliseconds; the update returns PR_ETIMEOUT.  how = 0 disarms.  Nothing is
+ * faulted on the device.
  */
 void pr_debug_fail_loop(int32_t how);
 

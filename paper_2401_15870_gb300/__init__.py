@@ -555,7 +555,8 @@ def pr_debug_fail_alloc(k):
 
 
 def pr_debug_fail_loop(how):
-    """Make the next launch of a single graph's one-kernel loop fail: 1, it is refused (0: disarm)."""
+    """Make the next launch of a single graph's one-kernel loop fail: 1, it is refused; 2, its
+    first barrier never completes and gives up (0: disarm)."""
     load().pr_debug_fail_loop(int(how))
 
 

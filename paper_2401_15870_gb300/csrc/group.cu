@@ -395,9 +395,9 @@ __global__ void k_g_control(GRun* run, GState* st, cudaGraphConditionalHandle co
 // from L2 (COH), never through the read-only path.
 
 // iterations of a barrier wait before it gives up (after the first 4096 each
-// with a short sleep: about a second in all, against microseconds when every
-// block runs)
-constexpr long long BAR_SPINS = 1ll << 24;
+// with a short sleep: about a second in all -- 2^20 took 0.40 s -- against
+// microseconds when every block runs)
+constexpr long long BAR_SPINS = 3ll << 20;
 // resident blocks per SM of the one-kernel loop, at most: fewer blocks make
 // the barriers cheaper (one arrival each), more make the phases of larger
 // graphs faster.  One per SM: R-MAT graphs of 2^8 to 2^14 vertices update

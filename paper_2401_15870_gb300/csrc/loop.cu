@@ -35,9 +35,11 @@ namespace {
 
 constexpr int LT = 1024;                        // threads per block
 constexpr int LW = LT / 32;
-// polls of a barrier wait before it gives up (after the first 4096 with a
-// short sleep each: about a second, against microseconds when every block runs)
-constexpr long long LOOP_SPINS = 1ll << 24;
+// polls of a barrier wait before it gives up, after the first 4096 with a short
+// sleep each: about a second (2^20 polls took 0.33 s), against microseconds when
+// every block runs
+constexpr long long LOOP_SPINS = 3ll << 20;
+constexpr long long LOOP_SPINS_STUCK = 1ll << 13;   // where a wait is made to run out (LOOP_STUCK)
 // shared memory of a block: above STAGE_MAX the columns stay in L2.  The rest
 // of the 256 KB is the L1 that the gathers land in: random 8-byte gathers of a
 // 64 MB table ran at 236 G/s with 64 KB in shared memory, 217 with 128 KB and
@@ -76,7 +78,7 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long x)
 // an arrival counter plus a release word 2.1; a slot per block polled by 152
 // threads of every block (no atomics) 3.9 to 5.2, the polls contending for a
 // few L2 lines.
-__device__ __forceinline__ bool grid_wait(LoopState* st, LoopOut* out, unsigned long long target) {
+__device__ __forceinline__ bool grid_wait(LoopState* st, LoopOut* out, unsigned long long target, long long polls) {
   fence_acq_rel();   // this block's writes before its arrival
   atomicAdd(&st->count, 1ull);
   long long spins = 0;
@@ -87,7 +89,7 @@ __device__ __forceinline__ bool grid_wait(LoopState* st, LoopOut* out, unsigned 
       good = false;
       break;
     }
-    if (spins > LOOP_SPINS) {
+    if (spins > polls) {
       atomicExch(&st->err, 1);
       *(volatile int32_t*)&out->err = 1;
       good = false;
@@ -152,7 +154,7 @@ __global__ void __launch_bounds__(LT, 1) k_loop(const __grid_constant__ LoopPara
   auto barrier = [&]() -> bool {
     __syncthreads();
     bool good = true;
-    if (tid == 0) good = grid_wait(st, p.out, (k + 1) * NB);
+    if (tid == 0) good = grid_wait(st, p.out, (k + 1) * NB, p.polls);
     k++;
     return __syncthreads_and(good) != 0;
   };
@@ -430,7 +432,7 @@ __global__ void __launch_bounds__(LT, 1) k_loop(const __grid_constant__ LoopPara
       if (lane == 0) {
         if (blockIdx.x == 0) st_relaxed_u64(&st->dR[(it + 1) % 3], 0ull);
         if (m) atomicMax(&st->dR[it % 3], m);
-        good = grid_wait(st, p.out, (k + 1) * NB);
+        good = grid_wait(st, p.out, (k + 1) * NB, p.polls);
         next_dR = ld_relaxed_u64(&st->dR[it % 3]);
         if (!REGS) red[LW] = next_dR;
       }
@@ -514,7 +516,7 @@ int loop_blocks() { return std::min(num_sms(), LOOP_MAX_BLOCKS); }
 size_t loop_state_bytes() { return sizeof(LoopState); }
 
 static std::atomic<int> g_loop_failure{0};   // of the next launch
-void arm_loop_failure(int how) { g_loop_failure.store(how == LOOP_REFUSED ? how : 0); }
+void arm_loop_failure(int how) { g_loop_failure.store(how == LOOP_REFUSED || how == LOOP_STUCK ? how : 0); }
 
 cudaError_t loop_reset(LoopState* st, cudaStream_t s) {
   return cudaMemsetAsync(st, 0, sizeof(*st), s);
@@ -547,6 +549,14 @@ static const void* loop_kernel(bool regs) {
 cudaError_t launch_loop(const Graph* g, LoopParams p, cudaStream_t s) {
   const int fail = g_loop_failure.exchange(0);
   if (fail == LOOP_REFUSED) return cudaErrorCooperativeLaunchTooLarge;
+  p.polls = LOOP_SPINS;
+  if (fail == LOOP_STUCK) {
+    // barriers counted whose arrivals never come: every block's first wait runs out
+    p.polls = LOOP_SPINS_STUCK;
+    const unsigned long long far = 1ull << 40;
+    const cudaError_t e = cudaMemcpyAsync(&p.st->barriers, &far, sizeof(far), cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) return e;
+  }
   const Layout l = layout(g);
   p.rows_cap = l.rows_cap;
   p.words_cap = l.words_cap;

@@ -47,6 +47,7 @@ struct LoopParams {
   LoopOut* out;             // pinned host memory; err must be 0 on entry
   int32_t rows_cap, words_cap, staged;
   int32_t l1_hub;           // contributions of internal ids below it are kept in L1
+  long long polls;          // of a barrier wait before it gives up
 };
 
 // Whether a graph's rows can be shared out to the blocks as the loop wants it.
@@ -56,12 +57,14 @@ bool loop_default(const Graph* g);
 size_t loop_state_bytes();
 // first use of a state, or after a launch that gave up
 cudaError_t loop_reset(LoopState* st, cudaStream_t s);
-// queue the update; p.rows_cap, words_cap and staged are filled in here
+// queue the update; p.rows_cap, words_cap, staged, l1_hub and polls are filled in here
 cudaError_t launch_loop(const Graph* g, LoopParams p, cudaStream_t s);
 int loop_blocks();
 // the next launch fails (pr_debug_fail_loop): LOOP_REFUSED, the launch returns
-// cudaErrorCooperativeLaunchTooLarge and nothing is launched; 0 disarms
-enum LoopFailure : int { LOOP_REFUSED = 1 };
+// cudaErrorCooperativeLaunchTooLarge and nothing is launched; LOOP_STUCK, its
+// first barrier waits for arrivals that never come and gives up after a short
+// wait; 0 disarms
+enum LoopFailure : int { LOOP_REFUSED = 1, LOOP_STUCK = 2 };
 void arm_loop_failure(int how);
 
 // the shares of the in-CSR's rows that loop_blocks() blocks get: writes
