@@ -518,11 +518,8 @@ pr_status dfpr::run_update(pr_graph* h, int method, double alpha, double tau, do
   int32_t iters = 0;
   double dR = 0.0;
   bool conv = false;
-  // with the gather and the epilogue in separate launches over one range, the
-  // epilogue updates the contributions in place (the gather that reads them has
-  // finished; one buffer instead of two in L2); otherwise into the other
-  // buffer.  Asynchronous order: in place after every range, on purpose
-  const bool inplace = async || (!h->gcfg.fused && h->gcfg.parts == 1);
+  // (asynchronous order: in place after every range, on purpose)
+  const bool inplace = async || sweep_in_place(h->gcfg);
   // the one-launch form has no variant without X: it gets an empty one
   const bool with_x = h->gcfg.fused && !async;
   memset(g->ctl_h, 0, sizeof(Ctl));

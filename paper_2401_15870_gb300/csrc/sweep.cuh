@@ -126,6 +126,12 @@ struct GatherCfg {
   int32_t parts = 1;   // vertex ranges whose epilogue overlaps the next range's gather (1, 2, 4, 8)
 };
 
+// Whether an every-vertex sweep of this setting writes the new contributions over
+// the ones it gathered (synchronous order): with the gather and the epilogue in
+// separate launches over one range the gather has finished by then, and one buffer
+// instead of two passes through L2
+inline bool sweep_in_place(const GatherCfg& c) { return !c.fused && c.parts == 1; }
+
 // the second stream and the events of a sweep cut into vertex ranges
 struct SweepAux {
   cudaStream_t stream = nullptr;

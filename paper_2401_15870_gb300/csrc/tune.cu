@@ -83,9 +83,11 @@ std::vector<GatherCfg> candidates(int32_t n) {
 }
 
 // Static / ND: one Eq. 1 sweep over every vertex per trial, from the current
-// contributions.  A trial writes the next contribution buffer (scratch between
-// updates) and R in place, so R is saved first and restored at the end; every
-// update resets the control block the sweeps add their totals to.
+// contributions, written where an update of that setting writes them
+// (sweep_in_place): over the current ones or into the other buffer (scratch
+// between updates).  R is written in place too, so it is saved first, and at the
+// end restored with the contributions made from it; every update resets the
+// control block the sweeps add their totals to.
 pr_status tune_sweeps(pr_graph* h, double alpha, int32_t reps, GatherCfg* best, float* best_ms, int32_t* trials) {
   Graph* g = &h->g;
   cudaStream_t s = g->stream;
@@ -96,16 +98,20 @@ pr_status tune_sweeps(pr_graph* h, double alpha, int32_t reps, GatherCfg* best, 
   }
   SweepParams p = base_params(g, alpha, 1e-6, 1e-6);
   p.Ccur = g->C[g->ccur];
-  p.Cnext = g->C[1 - g->ccur];
   p.ntiles_host = g->in.cap >> 2;
   cudaError_t e = cudaMemcpyAsync(h->vec_tmp, g->R, sizeof(double) * (size_t)g->n, cudaMemcpyDeviceToDevice, s);
   if (e != cudaSuccess) return (pr_status)cuda_fail(g, e, "pr_autotune");
   cudaEvent_t e0 = h->ev[4], e1 = h->ev[5];
   auto sweep = [&](const GatherCfg& c) {
+    p.Cnext = g->C[sweep_in_place(c) ? g->ccur : 1 - g->ccur];
     const SweepAux* aux = nullptr;
     cudaError_t ae = sweep_aux(h, c, &aux);
     return ae == cudaSuccess ? launch_full_sweep(SWEEP_FULL, p, c, g->rowbits, g->rowbase, g->anyb, g->done, aux, s)
                              : ae;
+  };
+  auto restore = [&] {
+    cudaError_t re = cudaMemcpyAsync(g->R, h->vec_tmp, sizeof(double) * (size_t)g->n, cudaMemcpyDeviceToDevice, s);
+    return re == cudaSuccess && g->has_ranks ? launch_contrib_all(g->R, g->C[g->ccur], g->out.deg, g->tab_sc, g->n, s) : re;
   };
   for (const GatherCfg& c : candidates(g->n)) {
     // one untimed sweep (also raises the kernel's shared memory limit), then
@@ -120,7 +126,7 @@ pr_status tune_sweeps(pr_graph* h, double alpha, int32_t reps, GatherCfg* best, 
     float ms = 0.f;
     if (!ok || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
       cudaError_t err = cudaGetLastError();
-      cudaMemcpyAsync(g->R, h->vec_tmp, sizeof(double) * (size_t)g->n, cudaMemcpyDeviceToDevice, s);
+      restore();
       return (pr_status)cuda_fail(g, err != cudaSuccess ? err : cudaErrorUnknown, "pr_autotune");
     }
     ms /= (float)reps;
@@ -130,7 +136,7 @@ pr_status tune_sweeps(pr_graph* h, double alpha, int32_t reps, GatherCfg* best, 
       *best = c;
     }
   }
-  e = cudaMemcpyAsync(g->R, h->vec_tmp, sizeof(double) * (size_t)g->n, cudaMemcpyDeviceToDevice, s);
+  e = restore();
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   return e == cudaSuccess ? PR_OK : (pr_status)cuda_fail(g, e, "pr_autotune");
 }
