@@ -125,9 +125,14 @@ typedef struct {
  * microseconds the launches cost more than the work.  Without this flag,
  * PR_OPT_DEVICE_LOOP or a host-loop flag, the device loop runs in one kernel
  * when the graphs of the update hold fewer than PR_ONE_KERNEL_SLOTS in-CSR
- * slots in all (one graph alone: fewer than three times as many, unless one
- * in-row holds most of them); PR_OPT_DEVICE_LOOP alone asks for the CUDA graph.  At most one
- * of PR_OPT_HOST_LOOP, PR_OPT_DEVICE_LOOP and PR_OPT_ONE_KERNEL may be set.
+ * slots in all (one graph alone, also as the only member of a group's update:
+ * fewer than three times as many, unless its longest in-rows make some block's
+ * share of the slots both half as large again as an equal one and 16384 slots
+ * larger, or a block's rows do not fit its shared memory); PR_OPT_DEVICE_LOOP
+ * alone asks for the CUDA graph.  At most one of PR_OPT_HOST_LOOP,
+ * PR_OPT_DEVICE_LOOP and PR_OPT_ONE_KERNEL may be set.
+ * The kernel needs every SM at once: it starts when the kernels of other
+ * streams have left them, and after every other such launch of the process.
  * Where the one-kernel loop of a single graph is refused (the process may not
  * use every SM), the update runs as it would for more graphs of the same size.
  * The result is the same bit for bit.  A barrier wait gives up after about a
@@ -218,7 +223,10 @@ pr_status pr_graph_resize(pr_graph* g, int32_t n_new);
  * every batch, Sec. 5.2.2).  The CSR and its transpose are edited in place on
  * the device, and the effective change Delta- = E_{t-1} \ E_t, Delta+ =
  * E_t \ E_{t-1} is kept for the next pr_update.  Contributions of sources
- * whose out-degree changed are refreshed.  Errors: PR_EINVAL (null pointer
+ * whose out-degree changed are refreshed.  The first host batch of at most
+ * 16384 edges allocates 128 KB of pinned host memory, kept with the graph, and
+ * the first batch a status block of some 100 bytes; later ones only what grows.
+ * Errors: PR_EINVAL (null pointer
  * with a positive count, negative count), PR_ERANGE (an id outside [0, n);
  * nothing is changed), PR_ENOMEM, PR_ECUDA.
  */
@@ -250,8 +258,9 @@ pr_status pr_apply_batches_device(int32_t count, pr_graph* const* graphs, const 
                                   const int32_t* const* ins_dst, const int64_t* n_ins);
 
 /* As pr_apply_batches_device with every endpoint array in host memory (ids
- * are checked on the host before anything of that graph is queued; each
- * batch is staged into its graph's device scratch on the pool's stream). */
+ * are checked on the host before anything of that graph is queued; a batch of
+ * at most 16384 edges is staged in its graph's pinned host memory and read from
+ * there, a larger one copied to the graph's device scratch on the pool's stream). */
 pr_status pr_apply_batches(int32_t count, pr_graph* const* graphs, const int32_t* const* del_src,
                            const int32_t* const* del_dst, const int64_t* n_del, const int32_t* const* ins_src,
                            const int32_t* const* ins_dst, const int64_t* n_ins);
@@ -374,7 +383,8 @@ pr_status pr_sweep_noalloc(int32_t n, const int64_t* in_off, const int32_t* in_s
  *   conditional nodes and for drivers without them), PR_OPT_DEVICE_LOOP (the
  *   CUDA graph) and PR_OPT_ONE_KERNEL (one cooperative kernel); with none of
  *   the three the group runs in one kernel below PR_ONE_KERNEL_SLOTS in-CSR
- *   slots over its graphs and as the CUDA graph above.  The update runs after
+ *   slots over its graphs (one graph alone: below the size given at
+ *   PR_OPT_ONE_KERNEL) and as the CUDA graph above.  The update runs after
  *   the work already queued on every graph's stream and is complete on
  *   return.  stats: NULL or count entries, one per graph in creation order;
  *   ms_update is the time of the whole group, ms_sweep is 0.  Errors:
@@ -401,7 +411,8 @@ void pr_group_destroy(pr_group* grp);
  * (4, 1), (8, 1), (2, 4)), an epilogue unit is chunks_per_unit 32-vertex chunks
  * (1, 2 or 4) whose loads a warp issues together.  Smaller units spread small
  * graphs over more warps; larger ones keep more loads in flight per warp or
- * look the graph up less often.  Defaults 4 / 1 / 4.  The setting changes no
+ * look the graph up less often.  Defaults 4 / 1 / 4, and 2 / 4 / 4 for updates
+ * of 2^25 in-CSR slots or more until a setting is made.  The setting changes no
  * result (the sums are exact).  It applies to the CUDA-graph and host loops;
  * the one-kernel loop (PR_OPT_ONE_KERNEL) uses units of one warp step of
  * 32 x 2 quads and one chunk.

@@ -471,7 +471,8 @@ def pr_group_update(q, method, alpha=0.85, tau=1e-10, tau_f=1e-6, tau_p=1e-6, ma
                     measure=None):
     """One update of every graph of the group; returns one Stats per graph.
     loop: None (by size: one kernel below PR_ONE_KERNEL_SLOTS in-CSR slots in
-    all, else the CUDA graph), "device" (CUDA graph), "one" (one cooperative
+    all -- one graph alone: below three times as many, see dfpr.h -- else the
+    CUDA graph), "device" (CUDA graph), "one" (one cooperative
     kernel) or "host" (kernels launched one by one).  measure: as in pr_update."""
     m = METHODS[method] if isinstance(method, str) else int(method)
     opts = pr_options(tau_f, tau_p, int(max_iter), LOOPS[loop] | MEASURES[measure])

@@ -636,7 +636,6 @@ pr_status dfpr::run_update(pr_graph* h, int method, double alpha, double tau, do
     const size_t wbytes = sizeof(uint32_t) * (size_t)(cdiv(n, 32) + 1);
     const double dbar = (double)g->m / (double)n;
     int cur = 0;
-    bool pull = false;
     // quad prefix of F_0: its edge volume picks push or pull for the first sweep
     TRY(launch_list_scan(g->wl[0], &g->ctl->count[0], g->in.deg, n, g->qs, g->tfirst, &g->ctl->qtot,
                          &g->ctl->ntiles, h->ls_tmp, s));

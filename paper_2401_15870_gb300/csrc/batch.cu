@@ -1219,8 +1219,8 @@ static cudaError_t launch_ingest(Graph* g, int N, const SmallCsr& out, const Sma
   return cudaGetLastError();
 }
 
-// phase 1 of a small batch: everything up to the status copy to the host,
-// queued on the graph's stream without waiting
+// phase 1 of a small batch: keys, ingest (which writes the status to the host's
+// pinned copy) and row edit, queued on the graph's stream without waiting
 static int small_launch(Graph* g, const int32_t* ds, const int32_t* dd, int64_t nd, const int32_t* is,
                         const int32_t* id, int64_t ni, SmallApply* A) {
   cudaStream_t s = g->stream;

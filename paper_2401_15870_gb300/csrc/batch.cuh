@@ -18,9 +18,10 @@ struct SmallApply {
   EditBufs* B = nullptr;   // set while a small batch is pending
   int32_t* S[2] = {nullptr, nullptr};
 };
-// a host batch's endpoint arrays where the device can read them (a copy is
-// queued on the graph's stream): *out holds nd deletion sources, nd targets, ni
-// insertion sources, ni targets
+// a host batch's endpoint arrays where the device can read them (up to 16384
+// edges the graph's pinned host memory, else device scratch, the copy queued on
+// the graph's stream): *out holds nd deletion sources, nd targets, ni insertion
+// sources, ni targets
 int stage_host_batch(Graph* g, const int32_t* ds, const int32_t* dd, int64_t nd, const int32_t* is, const int32_t* id,
                      int64_t ni, int32_t** out);
 int apply_batch_launch(Graph* g, const int32_t* ds, const int32_t* dd, int64_t nd, const int32_t* is,

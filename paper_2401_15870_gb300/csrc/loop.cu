@@ -486,12 +486,21 @@ __global__ void k_loop_shares(const int64_t* __restrict__ off, int32_t n, int64_
   }
 }
 
-// default for a graph of fewer in-CSR slots (larger ones run the CUDA graph,
-// one launch pair and a control kernel per iteration).  Time per iteration here
-// and there, DF / ND from the previous ranks: 245K edges (2^14 vertices) 4.5
-// against 16.6 us, 1.0M 7.6 against 17.5, 2.0M 12 against 23, 4.1M 19 against
-// 30, 8.2M 40 against 45; with pruning at 8.2M edges 61 against 58 (the
-// expanded flags are bytes here, bits there)
+// default for a graph of fewer in-CSR slots, about 2.2M edges (larger ones run
+// the CUDA graph, one launch pair and a control kernel per iteration).  Time per
+// iteration here and there (us), ND, DF and DF-P from the previous ranks:
+//   245K edges  4.5 / 16.6 (ND)
+//   1.0M        7.5 / 18.7    9.9 / 19.1   13.9 / 23.5
+//   2.1M       11.6 / 24.0   15.5 / 24.6   19.6 / 29.8
+//   4.2M       19.5 / 32.5   26.4 / 33.1   31.2 / 37.2
+//   6.6M       31.8 / 42.3   39.8 / 44.1   47.6 / 50.6
+//   8.5M       41.8 / 46.8   47.6 / 48.0   55.8 / 54.0
+// (above 10M a block's rows do not fit, loop_fits).  So the two cross near 8M
+// edges for a graph that has the chip to itself.  The line is below that, at three
+// times PR_ONE_KERNEL_SLOTS as dfpr.h says, because the loop holds every SM for
+// the whole update and waits for every other such launch of the process, while
+// the CUDA graph shares the chip with other streams' work: between 2.2M and 8M
+// edges PR_OPT_ONE_KERNEL asks for it.
 constexpr int64_t LOOP_SLOTS = 3ll << 20;
 
 struct Layout {

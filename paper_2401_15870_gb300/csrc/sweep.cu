@@ -98,9 +98,10 @@ __device__ __forceinline__ bool stopped(const SweepParams& p) { return p.close.m
 // with it, (share outside, degree ratio): R-MAT 25 (0.95, 5.5) 5.24 / 4.07 ms,
 // (0.07, 2.6) 3.77 / 3.80, DF there (0.22, 14) 3.94 / 4.04; R-MAT 23 (0.84, 2.4)
 // 1.20 / 1.00, (0.98, 1.1) 1.16 / 1.16; a stream graph of 2^23 vertices (0.94,
-// 1.3) 0.97 / 0.88, (0.96, 1.0) 0.97 / 0.98, (0.99, 0.8) 0.90 / 1.06.  Below
-// DECIDE_N vertices the expanded set's bits mostly hit L1 anyway: R-MAT 22 0.395 /
-// 0.334, 21 0.197 / 0.186, 20 0.096 / 0.099.
+// 1.3) 0.97 / 0.88, (0.96, 1.0) 0.97 / 0.98, (0.99, 0.8) 0.90 / 1.06.  The smaller
+// the graph, the more of the expanded set's bits hit L1 anyway: R-MAT 22 0.395 /
+// 0.334, 21 0.197 / 0.186, 20 0.096 / 0.099.  The line DECIDE_N lies at the last
+// size with a clear gain; the 6% at 2^21 are 0.01 ms a sweep.
 constexpr double DECIDE_OUT = 0.3;
 constexpr double DECIDE_DEG = 1.25;
 constexpr int32_t DECIDE_N = 1 << 22;
