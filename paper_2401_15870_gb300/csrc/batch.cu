@@ -385,9 +385,8 @@ static int repack_direction(Graph* g, Csr* c, const uint64_t* dl, int64_t nd, co
 //   k_edit_long   the others in chunks of RW_CH slots, one warp per chunk
 //                 staged in shared memory; a row of several chunks is copied to
 //                 scratch first (k_edit_copy), because its chunks move into one
-//                 another's places;
-//   k_edit_crowd  the chunks of those that take more insertions than they have
-//                 slots.
+//                 another's places; chunks that take more insertions than they
+//                 have slots go to its first blocks (edit_crowd).
 // A survivor x goes to x - (deletions below it) + (insertions below it), an
 // insertion to its rank among the insertions + old elements below it -
 // deletions below it.  A chunk looks only at the changes that fall into it:
@@ -579,21 +578,134 @@ __global__ void __launch_bounds__(256) k_edit_short(const __grid_constant__ Edit
 
 constexpr int EDIT_WARPS = 4;   // warps of a k_edit_long block
 
+// Crowded chunks: those with more insertions than slots, because the batch
+// refills a row that was emptied, or puts new ids behind a row's last one.  Work
+// is shared out by insertions, 1024 of the whole sorted list to a warp, not by
+// chunks of the old rows: with one warp per gap 10^6 insertions behind a hub's
+// last element took 17.7 ms per batch (now 1.42), 10^5 1.53 (0.61).  A crowded chunk holds
+// more insertions than a share, so the ones in a share are those of the chunk of
+// its first and of the chunk of its last insertion.  The warp
+//   - places them, each by searches between the places of the share's ends;
+//   - moves the survivors of the chunk whose insertions begin in its share: an
+//     element finds the changes below it by searches, the first of each 32 among
+//     all of the chunk's, the others between two of those.
+// The first blocks of k_edit_long, only for batches of more than 1024 insertions:
+// nothing here reads what the others write, and a launch of its own cost a batch
+// without crowded chunks 5 to 9 us.  Bound by the latency of the searches.
+
+// the insertions [ia, ib) that fall into one chunk of a row, and what the row is
+struct CrowdChunk {
+  int32_t ch = 0, ia = 0, ib = 0;   // ia == ib: not crowded
+  int32_t r = 0, d_old = 0, cap = 0;
+  int4 pl = make_int4(0, 0, 0, 0);
+  const int32_t* old = nullptr;
+  int32_t* row = nullptr;
+};
+
+// the crowded chunk that insertion k of direction d belongs to, if it does
+__device__ __forceinline__ CrowdChunk crowd_chunk(const EditBufs& B, const EditArgs& p, const EditStatus& st, int d,
+                                                  int bits, int64_t k) {
+  const uint64_t* il = B.il[d];
+  const uint64_t key = il[k];
+  CrowdChunk q;
+  q.r = (int32_t)(key >> bits);
+  const int j = lower_i32(B.rows[d], 0, st.nr[d], q.r);
+  q.pl = B.plan[d][j];
+  if (q.pl.w - q.pl.z <= RW_CH) return q;   // (more: a row of several chunks, so in the scratch)
+  q.d_old = B.od[d][j];
+  q.old = p.S[d] + (int64_t)B.lsc[d][lower_i32(B.lrow[d], 0, st.nlong[d], j)] * RW_CH;
+  const int64_t base = p.off[d][q.r];
+  q.cap = (int32_t)min(p.off[d][q.r + 1] - base, (int64_t)INT32_MAX);
+  q.row = p.col[d] + base;
+  // a chunk's insertions: those above the element before it and below its last
+  // one (the last chunk: all that are left)
+  const uint64_t rk = (uint64_t)q.r << bits, mask = (1ull << bits) - 1;
+  q.ch = min(lower_i32(q.old, 0, q.d_old, (int32_t)(key & mask)), q.d_old - 1) / RW_CH;
+  const int32_t x0 = q.ch * RW_CH;
+  const int ia = x0 > 0 ? (int)lower_key(il, q.pl.z, q.pl.w, rk | (uint64_t)q.old[x0 - 1]) : q.pl.z;
+  const int ib = x0 + (int64_t)RW_CH < q.d_old ? (int)lower_key(il, ia, q.pl.w, rk | (uint64_t)q.old[x0 + RW_CH - 1])
+                                               : q.pl.w;
+  if (ib - ia > RW_CH) {
+    q.ia = ia;
+    q.ib = ib;
+  }
+  return q;
+}
+
+// warps w0, w0 + nw, ... of the shares of both directions
+__device__ __forceinline__ void edit_crowd(const EditBufs& B, const EditArgs& p, int bits, int w0, int nw) {
+  const EditStatus& st = *B.st;
+  const int lane = threadIdx.x & 31;
+  const uint64_t mask = (1ull << bits) - 1;
+  const int shares = (int)cdiv(st.n_ins, RW_CH);
+  const int e0 = (p.dirs & 1) && !st.skip[0] ? shares : 0, e1 = e0 + ((p.dirs & 2) && !st.skip[1] ? shares : 0);
+  for (int w = w0; w < e1; w += nw) {
+    const int d = w >= e0 ? 1 : 0;
+    const int64_t ka = (int64_t)(w - (d ? e0 : 0)) * RW_CH, kb = min((int64_t)st.n_ins, ka + RW_CH);
+    const uint64_t *dl = B.dl[d], *il = B.il[d];
+    for (int end = 0; end < 2; end++) {
+      const CrowdChunk q = crowd_chunk(B, p, st, d, bits, end ? kb - 1 : ka);
+      if (q.ia == q.ib || (end && q.ia <= ka)) continue;   // (the second time: the chunk seen first)
+      const uint64_t rk = (uint64_t)q.r << bits;
+      const int64_t k0 = max(ka, (int64_t)q.ia), k1 = min(kb, (int64_t)q.ib);
+      {
+        const uint64_t at_end = il[(lane & 1) ? k1 - 1 : k0];
+        const int32_t pa = lower_i32(q.old, 0, q.d_old, (int32_t)(at_end & mask));
+        const int32_t pd = (int32_t)lower_key(dl, q.pl.x, q.pl.y, at_end);
+        const int32_t a0 = __shfl_sync(0xffffffffu, pa, 0), a1 = __shfl_sync(0xffffffffu, pa, 1);
+        const int32_t b0 = __shfl_sync(0xffffffffu, pd, 0), b1 = __shfl_sync(0xffffffffu, pd, 1);
+        for (int64_t k = k0 + lane; k < k1; k += 32) {
+          const uint64_t key = il[k];
+          const int32_t at = (int32_t)(k - q.pl.z) + lower_i32(q.old, a0, a1, (int32_t)(key & mask)) -
+                             ((int32_t)lower_key(dl, b0, b1, key) - q.pl.x);
+          if (at >= 0 && at < q.cap) q.row[at] = (int32_t)(key & mask);
+        }
+      }
+      __syncwarp();
+      if (q.ia < ka) continue;   // its survivors: the warp of the share before
+      const int32_t x0 = q.ch * RW_CH, no = min(q.d_old - x0, RW_CH);
+      const int da = (int)lower_key(dl, q.pl.x, q.pl.y, rk | (uint64_t)q.old[x0]);
+      const int db = (int)lower_key(dl, da, q.pl.y, (rk | (uint64_t)q.old[x0 + no - 1]) + 1);
+      const bool any = lane * 32 < no;
+      const uint64_t head = any ? rk | (uint64_t)q.old[x0 + lane * 32] : 0;
+      const int fi = any ? (int)lower_key(il, q.ia, q.ib, head) : q.ib, fd = any ? (int)lower_key(dl, da, db, head) : db;
+      for (int32_t b = 0; b < no; b += 32) {
+        const int g = b >> 5, h = g < 31 ? g + 1 : 31;
+        const int i0 = __shfl_sync(0xffffffffu, fi, g), d0 = __shfl_sync(0xffffffffu, fd, g);
+        const int ni = __shfl_sync(0xffffffffu, fi, h), nd = __shfl_sync(0xffffffffu, fd, h);
+        const int i1 = g < 31 ? ni : q.ib, d1 = g < 31 ? nd : db;
+        if (b + lane < no) {
+          const int32_t x = x0 + b + lane, v = q.old[x];
+          const uint64_t key = rk | (uint64_t)v;
+          const int ki = (int)lower_key(il, i0, i1, key), kd = (int)lower_key(dl, d0, d1, key);
+          const int32_t at = x - (kd - q.pl.x) + (ki - q.pl.z);
+          if (!(kd < d1 && dl[kd] == key) && at != x && at >= 0 && at < q.cap) q.row[at] = v;
+        }
+      }
+    }
+  }
+}
+
 __global__ void __launch_bounds__(EDIT_WARPS * 32) k_edit_long(const __grid_constant__ EditBufs B,
-                                                               const __grid_constant__ EditArgs p, int bits) {
+                                                               const __grid_constant__ EditArgs p, int bits,
+                                                               int crowd_blocks) {
+  if ((int)blockIdx.x < crowd_blocks) {
+    edit_crowd(B, p, bits, blockIdx.x * EDIT_WARPS + (threadIdx.x >> 5), crowd_blocks * EDIT_WARPS);
+    return;
+  }
   __shared__ __align__(16) int32_t stage[EDIT_WARPS][RW_CH];
   __shared__ int32_t delta[EDIT_WARPS][RW_CH + 1];     // edit_marks.cuh: change of the shift at an element
   __shared__ uint32_t gone[EDIT_WARPS][RW_CH / 32];    // and whether it is deleted
   const EditStatus& st = *B.st;
   const int lane = threadIdx.x & 31;
-  const int nw = gridDim.x * EDIT_WARPS;
+  const int nw = (gridDim.x - crowd_blocks) * EDIT_WARPS;
   const uint64_t mask = (1ull << bits) - 1;
   int32_t* const T = stage[threadIdx.x >> 5];
   int32_t* const D = delta[threadIdx.x >> 5];
   uint32_t* const dead = gone[threadIdx.x >> 5];
   const int e0 = (p.dirs & 1) && !st.skip[0] ? st.chunks[0] : 0;
   const int e1 = e0 + ((p.dirs & 2) && !st.skip[1] ? st.chunks[1] : 0);
-  for (int w = blockIdx.x * EDIT_WARPS + (threadIdx.x >> 5); w < e1; w += nw) {
+  for (int w = (blockIdx.x - crowd_blocks) * EDIT_WARPS + (threadIdx.x >> 5); w < e1; w += nw) {
     const int d = w >= e0 ? 1 : 0, c = w - (d ? e0 : 0);
     const int li = long_row(B.lpre[d], st.nlong[d], c);
     const int j = B.lrow[d][li], part = c - B.lpre[d][li];
@@ -650,7 +762,7 @@ __global__ void __launch_bounds__(EDIT_WARPS * 32) k_edit_long(const __grid_cons
     const int shift = (ia - pl.z) - (da - pl.x);   // of the chunk's first element
     const int cd = db - da, ci = ib - ia;
     if (ci > RW_CH) {
-      // k_edit_crowd
+      // edit_crowd
     } else if (cd + ci <= EDIT_FEW) {
       // one change per lane, compared with every element
       int32_t y = 0;
@@ -713,115 +825,6 @@ __global__ void __launch_bounds__(EDIT_WARPS * 32) k_edit_long(const __grid_cons
   }
 }
 
-// Crowded chunks: those with more insertions than slots, because the batch
-// refills a row that was emptied, or puts new ids behind a row's last one.  Work
-// is shared out by insertions, 1024 of the whole sorted list to a warp, not by
-// chunks of the old rows: with one warp per gap 10^6 insertions behind a hub's
-// last element took 17.7 ms per batch (now 1.45), 10^5 1.53 (0.63).  A crowded chunk holds
-// more insertions than a share, so the ones in a share are those of the chunk of
-// its first and of the chunk of its last insertion.  The warp
-//   - places them, each by searches between the places of the share's ends;
-//   - moves the survivors of the chunk whose insertions begin in its share: an
-//     element finds the changes below it by searches, the first of each 32 among
-//     all of the chunk's, the others between two of those.
-// Launched only for batches of more than 1024 insertions; reads nothing that
-// k_edit_long writes.  Bound by the latency of the searches; a batch without
-// crowded chunks pays the launch and one search per share.
-
-// the insertions [ia, ib) that fall into one chunk of a row, and what the row is
-struct CrowdChunk {
-  int32_t ch = 0, ia = 0, ib = 0;   // ia == ib: not crowded
-  int32_t r = 0, d_old = 0, cap = 0;
-  int4 pl = make_int4(0, 0, 0, 0);
-  const int32_t* old = nullptr;
-  int32_t* row = nullptr;
-};
-
-// the crowded chunk that insertion k of direction d belongs to, if it does
-__device__ __forceinline__ CrowdChunk crowd_chunk(const EditBufs& B, const EditArgs& p, const EditStatus& st, int d,
-                                                  int bits, int64_t k) {
-  const uint64_t* il = B.il[d];
-  const uint64_t key = il[k];
-  CrowdChunk q;
-  q.r = (int32_t)(key >> bits);
-  const int j = lower_i32(B.rows[d], 0, st.nr[d], q.r);
-  q.pl = B.plan[d][j];
-  if (q.pl.w - q.pl.z <= RW_CH) return q;   // (more: a row of several chunks, so in the scratch)
-  q.d_old = B.od[d][j];
-  q.old = p.S[d] + (int64_t)B.lsc[d][lower_i32(B.lrow[d], 0, st.nlong[d], j)] * RW_CH;
-  const int64_t base = p.off[d][q.r];
-  q.cap = (int32_t)min(p.off[d][q.r + 1] - base, (int64_t)INT32_MAX);
-  q.row = p.col[d] + base;
-  // a chunk's insertions: those above the element before it and below its last
-  // one (the last chunk: all that are left)
-  const uint64_t rk = (uint64_t)q.r << bits, mask = (1ull << bits) - 1;
-  q.ch = min(lower_i32(q.old, 0, q.d_old, (int32_t)(key & mask)), q.d_old - 1) / RW_CH;
-  const int32_t x0 = q.ch * RW_CH;
-  const int ia = x0 > 0 ? (int)lower_key(il, q.pl.z, q.pl.w, rk | (uint64_t)q.old[x0 - 1]) : q.pl.z;
-  const int ib = x0 + (int64_t)RW_CH < q.d_old ? (int)lower_key(il, ia, q.pl.w, rk | (uint64_t)q.old[x0 + RW_CH - 1])
-                                               : q.pl.w;
-  if (ib - ia > RW_CH) {
-    q.ia = ia;
-    q.ib = ib;
-  }
-  return q;
-}
-
-__global__ void __launch_bounds__(256) k_edit_crowd(const __grid_constant__ EditBufs B, const __grid_constant__ EditArgs p,
-                                                    int bits) {
-  const EditStatus& st = *B.st;
-  const int lane = threadIdx.x & 31;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  const uint64_t mask = (1ull << bits) - 1;
-  const int shares = (int)cdiv(st.n_ins, RW_CH);
-  const int e0 = (p.dirs & 1) && !st.skip[0] ? shares : 0, e1 = e0 + ((p.dirs & 2) && !st.skip[1] ? shares : 0);
-  for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < e1; w += nw) {
-    const int d = w >= e0 ? 1 : 0;
-    const int64_t ka = (int64_t)(w - (d ? e0 : 0)) * RW_CH, kb = min((int64_t)st.n_ins, ka + RW_CH);
-    const uint64_t *dl = B.dl[d], *il = B.il[d];
-    for (int end = 0; end < 2; end++) {
-      const CrowdChunk q = crowd_chunk(B, p, st, d, bits, end ? kb - 1 : ka);
-      if (q.ia == q.ib || (end && q.ia <= ka)) continue;   // (the second time: the chunk seen first)
-      const uint64_t rk = (uint64_t)q.r << bits;
-      const int64_t k0 = max(ka, (int64_t)q.ia), k1 = min(kb, (int64_t)q.ib);
-      {
-        const uint64_t at_end = il[(lane & 1) ? k1 - 1 : k0];
-        const int32_t pa = lower_i32(q.old, 0, q.d_old, (int32_t)(at_end & mask));
-        const int32_t pd = (int32_t)lower_key(dl, q.pl.x, q.pl.y, at_end);
-        const int32_t a0 = __shfl_sync(0xffffffffu, pa, 0), a1 = __shfl_sync(0xffffffffu, pa, 1);
-        const int32_t b0 = __shfl_sync(0xffffffffu, pd, 0), b1 = __shfl_sync(0xffffffffu, pd, 1);
-        for (int64_t k = k0 + lane; k < k1; k += 32) {
-          const uint64_t key = il[k];
-          const int32_t at = (int32_t)(k - q.pl.z) + lower_i32(q.old, a0, a1, (int32_t)(key & mask)) -
-                             ((int32_t)lower_key(dl, b0, b1, key) - q.pl.x);
-          if (at >= 0 && at < q.cap) q.row[at] = (int32_t)(key & mask);
-        }
-      }
-      __syncwarp();
-      if (q.ia < ka) continue;   // its survivors: the warp of the share before
-      const int32_t x0 = q.ch * RW_CH, no = min(q.d_old - x0, RW_CH);
-      const int da = (int)lower_key(dl, q.pl.x, q.pl.y, rk | (uint64_t)q.old[x0]);
-      const int db = (int)lower_key(dl, da, q.pl.y, (rk | (uint64_t)q.old[x0 + no - 1]) + 1);
-      const bool any = lane * 32 < no;
-      const uint64_t head = any ? rk | (uint64_t)q.old[x0 + lane * 32] : 0;
-      const int fi = any ? (int)lower_key(il, q.ia, q.ib, head) : q.ib, fd = any ? (int)lower_key(dl, da, db, head) : db;
-      for (int32_t b = 0; b < no; b += 32) {
-        const int g = b >> 5, h = g < 31 ? g + 1 : 31;
-        const int i0 = __shfl_sync(0xffffffffu, fi, g), d0 = __shfl_sync(0xffffffffu, fd, g);
-        const int ni = __shfl_sync(0xffffffffu, fi, h), nd = __shfl_sync(0xffffffffu, fd, h);
-        const int i1 = g < 31 ? ni : q.ib, d1 = g < 31 ? nd : db;
-        if (b + lane < no) {
-          const int32_t x = x0 + b + lane, v = q.old[x];
-          const uint64_t key = rk | (uint64_t)v;
-          const int ki = (int)lower_key(il, i0, i1, key), kd = (int)lower_key(dl, d0, d1, key);
-          const int32_t at = x - (kd - q.pl.x) + (ki - q.pl.z);
-          if (!(kd < d1 && dl[kd] == key) && at != x && at >= 0 && at < q.cap) q.row[at] = v;
-        }
-      }
-    }
-  }
-}
-
 // queue the edit of the directions in `dirs`; rows: touched rows of both, at
 // most; ins: insertions, at most
 static void launch_edit(Graph* g, const EditBufs& B, int32_t* const* S, int dirs, int64_t rows, int64_t ins) {
@@ -841,10 +844,8 @@ static void launch_edit(Graph* g, const EditBufs& B, int32_t* const* S, int dirs
   p.dirs = dirs;
   note_launch(); k_edit_copy<<<num_sms() * 4, 256, 0, s>>>(B, p);
   note_launch(); k_edit_short<<<grid_for(8 * rows, 256), 256, 0, s>>>(B, p, g->id_bits);
-  note_launch(); k_edit_long<<<num_sms() * 6, EDIT_WARPS * 32, 0, s>>>(B, p, g->id_bits);
-  if (ins > RW_CH) {
-    note_launch(); k_edit_crowd<<<grid_for(2 * 32 * cdiv(ins, RW_CH), 256), 256, 0, s>>>(B, p, g->id_bits);
-  }
+  const int crowd = ins > RW_CH ? grid_for(2 * cdiv(ins, RW_CH), EDIT_WARPS) : 0;
+  note_launch(); k_edit_long<<<crowd + num_sms() * 6, EDIT_WARPS * 32, 0, s>>>(B, p, g->id_bits, crowd);
 }
 
 // what a row of `len` slots adds to the lists of long rows: one entry, its

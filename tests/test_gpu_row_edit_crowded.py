@@ -1,4 +1,4 @@
-"""Rows that take more insertions than a chunk has slots (k_edit_crowd): all in
+"""Rows that take more insertions than a chunk has slots (edit_crowd): all in
 one gap of a row that was emptied, in front of the first or behind the last
 element, in a few gaps of many chunks, with deletions beside them; by batches of
 the small and the large path, against the edge sets exactly.  And that such
